@@ -55,7 +55,9 @@ def listed():
         # BCs, Algorithm 3, four levels, FP64
         _restore("zero256_f64_l4", 256, "disk", 17, 7.0, "zero", "sym", 4, 6, dtype="f64", alpha=0.3),
         # a megapixel image, motion blur, Algorithm 1, Bregman variable in BF16
-        _restore("rect1024_bf16", 1024, "motion", 21, 21.0, "rect", "bccb", 2, 10, z_store="bf16",
+        # (the first two iterations: rounding z to 8 bits makes later iterates
+        # depend on the last bit of every sum before it)
+        _restore("rect1024_bf16", 1024, "motion", 21, 21.0, "rect", "bccb", 2, 2, z_store="bf16",
                  alpha=0.5, angle=0.9),
         # the same image with the Krylov preconditioner (Algorithm 2)
         _restore("rect1024_krylov", 1024, "motion", 21, 21.0, "rect", "krylov", 2, 3, angle=0.9),
@@ -119,9 +121,10 @@ def draw(rng):
     dtype = rng.choice(("f32", "f32", "f32", "f64"))
     hi = 300 if dtype == "f64" else 1600
     if kind == "batch":
+        zs = rng.choice(("f32", "f32", "bf16"))
         return dict(kind="batch", count=rng.randint(2, 48), spec=rng.randrange(1 << 20),
-                    lo=rng.choice((64, 100, 128)), hi=_log_int(rng, 160, 800), iters=rng.randint(3, 6),
-                    levels=rng.choice((1, 2, 2, 3)), z_store=rng.choice(("f32", "f32", "bf16")))
+                    lo=rng.choice((64, 100, 128)), hi=_log_int(rng, 160, 800),
+                    iters=2 if zs == "bf16" else rng.randint(3, 6), levels=rng.choice((1, 2, 2, 3)), z_store=zs)
     if kind == "blur":
         return dict(kind="blur", n=_draw_n(rng, 64, hi, dtype), psf=psf, p=p, size=size, angle=angle,
                     bc=rng.choice(("zero", "periodic", "reflective", "rect", "antireflective")),
@@ -151,9 +154,10 @@ def draw(rng):
     if precond != "krylov":
         form = rng.choice(("synthesis",) * 7 + ("balanced",))
         path = rng.choice(("direct",) * 7 + ("fft",))
+    zs = rng.choice(("f32", "f32", "bf16"))
     return _restore(None, n, psf, p, size, bc, precond, rng.choice((1, 2, 2, 4)),
-                    rng.randint(2, most), dtype=dtype,
-                    z_store=rng.choice(("f32", "f32", "bf16")), alpha=alpha, angle=angle,
+                    2 if zs == "bf16" and dtype == "f32" else rng.randint(2, most), dtype=dtype,
+                    z_store=zs, alpha=alpha, angle=angle,
                     nu=round(rng.uniform(0.005, 0.03), 4), formulation=form, blur_path=path)
 
 
