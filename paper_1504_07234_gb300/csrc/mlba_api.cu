@@ -611,11 +611,31 @@ void destroy_batch(mlba_batch* B) {
   delete B;
 }
 
+// Complex values per transform CTA for a set of problems whose passes run as
+// `launches` launches each.
+// A CTA is a chain of barrier-separated phases, so a launch with fewer CTAs
+// than the chip has SMs takes as long as its fullest CTA: below TR_FILL_CTAS
+// full CTAs the transforms spread over more of them instead.  Both sides of the line
+// (one CTA holding up to TR_CAP values against 2 per SM; a pass measured alone):
+// 256^2 DCT rows 10.5 -> 6.7 us, forward columns with the candidate sums 29.5
+// -> 18 us; 256^2 FP64 columns 111 -> 36 us; 1000^2 DFT, all three passes
+// 48 -> 40 us.  The 64-problem batch has 2400 full CTAs and keeps them (the
+// split measured no gain there).
+constexpr int TR_FILL_CTAS = 304;
+int transform_fill(const std::vector<HostProb>& v, int launches) {
+  double elems = 0.0;
+  for (const HostProb& h : v)
+    if (h.pd.transform != TR_NONE) elems += (double)((h.pd.n + 1) / 2) * h.pd.nfft;
+  return (int)std::min<double>(TR_CAP, elems / launches / TR_FILL_CTAS);
+}
+
 // Launch geometry of the transform passes of a length-n problem (FFT length
 // pd.nfft): transforms per CTA and the column blocking of the spectrum.
-void transform_geometry(Prob& pd) {
+// fill: complex values a CTA should hold (at least one transform, at most
+// TR_CAP).
+void transform_geometry(Prob& pd, int fill) {
   const int n = pd.n;
-  const int cap = TR_CAP / std::max(pd.nfft, n);      // transforms per CTA
+  const int cap = std::max(1, std::min(fill, TR_CAP) / std::max(pd.nfft, n));      // transforms per CTA
   const int pairs = (n + 1) / 2;
   {
     const int nb = (pairs + cap - 1) / cap;            // row CTAs, then pairs spread evenly
@@ -661,7 +681,6 @@ bool setup_conv_entry(const HostProb& own, int owner, int adj, HostProb& h) {
   pd.alpha = 1.0; pd.max_iter = -1; pd.sidx = owner;
   pd.nfft = M;
   if (!fft_plan(pd)) return false;
-  transform_geometry(pd);
   pd.nblk_vec = vec_blocks((size_t)M * M);
   const int p = op.p;
   h.psf_pre.resize((size_t)p * p);
@@ -773,7 +792,6 @@ int setup_problem(const mlba_problem& in, const mlba_opts& o, HostProb& h) {
   pd.nblk_corr = stencil_tiles(pd.ne);
   // the frame kernel indexes a z array (all bands) with 32-bit offsets
   if ((double)pd.nbands * pd.nf * pd.nf >= 2147483647.0) return MLBA_E_UNSUPPORTED;
-  transform_geometry(pd);
   pd.nblk_vec = vec_blocks((size_t)n * n);
   return MLBA_OK;
 }
@@ -1187,6 +1205,13 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
       B->fc.push_back(sa);
       h.pd.fc = (o.blur_path == 1) ? 1 : 0;       // 2: measured below
     }
+  }
+  // transforms per CTA: as many as fit, or fewer so that the batch's row and
+  // column passes have about two CTAs per SM
+  {
+    const int fill = transform_fill(B->hp, 1), ffill = transform_fill(B->fc, 2);   // (forward, adjoint entries)
+    for (HostProb& h : B->hp) transform_geometry(h.pd, fill);
+    for (HostProb& h : B->fc) transform_geometry(h.pd, ffill);
   }
   if (o.stream) { B->stream = (cudaStream_t)o.stream; }
   else {

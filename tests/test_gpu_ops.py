@@ -212,3 +212,25 @@ def test_antireflective_transform_precond(M, dtype, n, psf):
             got = ctx.precond(r, alpha, which)
             assert rel_err(got, ref) <= (1e-11 if dtype == "f64" else 2e-5), (which, alpha)
     ctx.close()
+
+
+@pytest.mark.parametrize("n,transform,psf", [(64, "dct", "disk2"), (48, "dft", "motion7"), (45, "dft", "motion7"),
+                                             (50, "dct", "gauss9")])
+def test_transform_ctas_full_and_split(M, n, transform, psf):
+    """The transforms of one small problem are spread over more CTAs than the
+    same problem's in a batch that fills the chip (there a CTA holds as many
+    transforms as fit): the iterates agree to FP32 rounding (the column blocks,
+    and so the order of the alpha_n sums, differ).  A relative bound of 1e-5 is
+    the per-operator bar."""
+    bc = "reflective" if transform == "dct" else "periodic"
+    h = PSFS[psf]
+    f = I.true_image(n, n)
+    g, delta = I.observe_periodic(f, h, 0.02, n)
+    desc = dict(psf=h, g=g.astype(np.float32), delta=delta, bc=bc, precond="tikh_ns", transform=transform)
+    out = []
+    for count in (1, 1400):
+        b = M.Batch([desc] * count, dtype="f32", levels=1, stop=False, max_iter=3)
+        b.iterate(2)
+        out.append(b.result(count - 1))
+        b.close()
+    assert rel_err(out[1], out[0]) <= 1e-5
