@@ -20,6 +20,7 @@
 // u comes from (per problem): the full correlation V folded by the BC
 // transpose (A^T t for imposed boundary conditions), V itself (rectangular
 // A), or t (Algorithm 4 forms, where C^T is already applied).
+#include <type_traits>
 #include "mlba_internal.cuh"
 #include "mlba_launch.h"
 
@@ -103,8 +104,10 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* b, unsigned parity
 // ---------------------------------------------------------------------------
 // Warp row-sweep variant for L <= 2 (the measured workloads).
 //
-// A CTA owns an F3_TX x (32 F3_NWR) tile of f and of every z band; warp w
-// owns the 32-row segment w of it.  In each level a lane owns one column of
+// A CTA owns an F3_TX x (SEG F3_NWR) tile of f and of every z band; warp w
+// owns the SEG-row segment w of it (32 rows; fewer in launches with few warps,
+// whose time is one warp's chain of rows: the host's frame_segment has the
+// rule and its measurements).  In each level a lane owns one column of
 // the band region (coefficients at columns tx0 - X .. tx0 - X + 31) and the
 // warp sweeps down the rows:
 //   analysis   h_j(y, x) = sum_t b_j[t] c(y, x + (t-1)D)     (shared memory)
@@ -128,7 +131,8 @@ constexpr int F3_TX = 26;      // tile columns: level-2 output lanes 3..28 after
 // per framelet launch; distances 1..10 tried)
 constexpr int Z_L2_AHEAD = 2;   // k_frame3
 constexpr int LV_L2_AHEAD = 1;  // k_frame_lev
-constexpr int F3_SEG = 32;     // rows per warp
+constexpr int F3_SEG = 32;     // rows per warp of the tile shapes below
+constexpr int F3_SEG_NWR = 2;   // warps per CTA of the sweeps with shorter segments (16, 8, 4 rows)
 // Tile shapes the autotuner chooses from: warps (32-row segments) per CTA and
 // the z prefetch distance in rows.  Every shape computes the same values in
 // the same order (a warp's sweep does not depend on its CTA), so the choice
@@ -143,9 +147,9 @@ struct F3Shape { int nwr, pf, ring; };
 constexpr F3Shape F3_SHAPES[FRAME_SHAPES] = {{2, 2, 0}, {1, 2, 0}, {4, 2, 0}, {2, 3, 0}, {1, 3, 0},
                                              {2, 2, 6}, {2, 2, 10}, {1, 2, 12}};
 
-template <int L, int NWR>
+template <int L, int NWR, int SEG = F3_SEG>
 struct F3 {
-  static constexpr int TY = F3_SEG * NWR;
+  static constexpr int TY = SEG * NWR;
   static constexpr int C0 = (L == 2) ? 6 : 2;         // radius of the u tile
   static constexpr int UW = F3_TX + 2 * C0, UH = TY + 2 * C0;
   static constexpr size_t elems = (size_t)UW * UH + (L == 2 ? (size_t)F3_TX * TY : 0);
@@ -155,13 +159,13 @@ template <typename TZ>
 __host__ __device__ constexpr size_t f3_slot_bytes() { return 32 * 8 * sizeof(TZ); }
 // shared memory: u tile and level-2 part of f (T), then per warp `ring` slots
 // and `ring` mbarriers
-template <typename T, typename TZ, int L, int NWR, int RING>
+template <typename T, typename TZ, int L, int NWR, int RING, int SEG = F3_SEG>
 __host__ __device__ constexpr size_t frame3_ring_offset() {
-  return (F3<L, NWR>::elems * sizeof(T) + 15) / 16 * 16;
+  return (F3<L, NWR, SEG>::elems * sizeof(T) + 15) / 16 * 16;
 }
-template <typename T, typename TZ, int L, int NWR, int RING>
+template <typename T, typename TZ, int L, int NWR, int RING, int SEG = F3_SEG>
 __host__ __device__ constexpr size_t frame3_smem_bytes() {
-  return frame3_ring_offset<T, TZ, L, NWR, RING>() + (size_t)NWR * RING * (f3_slot_bytes<TZ>() + 8);
+  return frame3_ring_offset<T, TZ, L, NWR, RING, SEG>() + (size_t)NWR * RING * (f3_slot_bytes<TZ>() + 8);
 }
 
 // half-sample reflection of an index with the parity of the mirroring; the
@@ -473,13 +477,13 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
 
 // One framelet tile on the thread group `blk` of 32 F3_NWR threads with its
 // shared memory at smraw.
-template <typename T, typename TZ, int L, int F3_NWR, int F3_PF, int RING, typename BLK>
+template <typename T, typename TZ, int L, int F3_NWR, int F3_PF, int RING, int SEG, typename BLK>
 __device__ __forceinline__ void frame3_body(const int2 item, const Prob* __restrict__ probs,
                                             State* __restrict__ states, int u_slot, int f_slot,
                                             const void* zin_op, void* zout_op, double op_mu,
                                             unsigned char* smraw, BLK blk) {
   const int tid = blk.tid();
-  using Gm = F3<L, F3_NWR>;
+  using Gm = F3<L, F3_NWR, SEG>;
   constexpr int F3_TY = Gm::TY;
   const Prob& pd = probs[item.x];
   const State& st = states[item.x];
@@ -546,7 +550,7 @@ __device__ __forceinline__ void frame3_body(const int2 item, const Prob* __restr
   }
   blk.sync();
   const int w = tid >> 5;
-  const int seg_lo = ty0 + w * F3_SEG, seg_hi = seg_lo + F3_SEG;
+  const int seg_lo = ty0 + w * SEG, seg_hi = seg_lo + SEG;
   if (seg_lo >= nf) return;        // no barrier follows
   T* f = static_cast<T*>(pd.buf[f_slot]);
   // this warp's ring of z rows and its mbarriers (RING > 0)
@@ -556,7 +560,7 @@ __device__ __forceinline__ void frame3_body(const int2 item, const Prob* __restr
   rg.buf = nullptr;
   rg.bar = nullptr;
   if constexpr (RING > 0) {
-    unsigned char* rb = smraw + frame3_ring_offset<T, TZ, L, F3_NWR, RING>();
+    unsigned char* rb = smraw + frame3_ring_offset<T, TZ, L, F3_NWR, RING, SEG>();
     rg.buf = reinterpret_cast<TZ*>(rb + (size_t)w * RING * f3_slot_bytes<TZ>());
     rg.bar = reinterpret_cast<unsigned long long*>(rb + (size_t)F3_NWR * RING * f3_slot_bytes<TZ>()) +
              w * RING;
@@ -581,12 +585,12 @@ __device__ __forceinline__ void frame3_body(const int2 item, const Prob* __restr
     vs->stopped = 1;
   }
 }
-template <typename T, typename TZ, int L, int F3_NWR, int F3_PF, int RING>
+template <typename T, typename TZ, int L, int F3_NWR, int F3_PF, int RING, int SEG = F3_SEG>
 __global__ void __launch_bounds__(32 * F3_NWR)
 k_frame3(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __restrict__ items,
          int u_slot, int f_slot, const void* zin_op, void* zout_op, double op_mu) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  frame3_body<T, TZ, L, F3_NWR, F3_PF, RING>(items[blockIdx.x], probs, states, u_slot, f_slot, zin_op,
+  frame3_body<T, TZ, L, F3_NWR, F3_PF, RING, SEG>(items[blockIdx.x], probs, states, u_slot, f_slot, zin_op,
                                              zout_op, op_mu, smraw, BlkFull{});
 }
 
@@ -939,15 +943,15 @@ void launch_frame_levels(const Prob* probs, State* states, const int2* items, co
   }
 }
 
-int frame_tiles(int nf, int levels, int shape) {
-  const int ty = F3_SEG * F3_SHAPES[shape].nwr;
+int frame_tiles(int nf, int levels, int shape, int seg) {
+  const int ty = seg < F3_SEG ? seg * F3_SEG_NWR : F3_SEG * F3_SHAPES[shape].nwr;
   (void)levels;
   return ((nf + F3_TX - 1) / F3_TX) * ((nf + ty - 1) / ty);
 }
 
-void frame_shape(int shape, int* tile_x, int* tile_y, int* prefetch) {
+void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch) {
   *tile_x = F3_TX;
-  *tile_y = F3_SEG * F3_SHAPES[shape].nwr;
+  *tile_y = seg < F3_SEG ? seg * F3_SEG_NWR : F3_SEG * F3_SHAPES[shape].nwr;
   *prefetch = F3_SHAPES[shape].ring > 0 ? F3_SHAPES[shape].ring : F3_SHAPES[shape].pf;
 }
 
@@ -1018,9 +1022,21 @@ size_t frame3_smem(int shape) {
   }
 }
 template <typename T, typename TZ, int L>
-void launch_frame3_shape(int shape, const Prob* probs, State* states, const int2* items, int nitems,
+void launch_frame3_shape(int shape, int seg, const Prob* probs, State* states, const int2* items, int nitems,
                          int u_slot, int f_slot, const void* zin, void* zout, double op_mu,
                          cudaStream_t s) {
+  if (seg < F3_SEG) {
+    auto go = [&](auto sg) {
+      constexpr int SG = decltype(sg)::value;
+      k_frame3<T, TZ, L, F3_SEG_NWR, 2, 0, SG>
+          <<<nitems, 32 * F3_SEG_NWR, frame3_smem_bytes<T, TZ, L, F3_SEG_NWR, 0, SG>(), s>>>(
+              probs, states, items, u_slot, f_slot, zin, zout, op_mu);
+    };
+    if (seg == 16) go(std::integral_constant<int, 16>{});
+    else if (seg == 8) go(std::integral_constant<int, 8>{});
+    else go(std::integral_constant<int, 4>{});
+    return;
+  }
   if constexpr (sizeof(T) == 8) {
     k_frame3<T, TZ, L, 2, 2, 0><<<nitems, 64, frame3_smem_bytes<T, TZ, L, 2, 0>(), s>>>(
         probs, states, items, u_slot, f_slot, zin, zout, op_mu);
@@ -1043,12 +1059,12 @@ void launch_frame3_shape(int shape, const Prob* probs, State* states, const int2
 template <typename T, typename TZ>
 void launch_frame(const Prob* probs, State* states, const int2* items, int nitems, const int* sec,
                   int u_slot, int f_slot, const void* zin, void* zout, double op_mu, int levels,
-                  int shape, cudaStream_t s) {
+                  int shape, int seg, cudaStream_t s) {
   if (nitems <= 0) return;
   if (levels == 1)
-    launch_frame3_shape<T, TZ, 1>(shape, probs, states, items, nitems, u_slot, f_slot, zin, zout, op_mu, s);
+    launch_frame3_shape<T, TZ, 1>(shape, seg, probs, states, items, nitems, u_slot, f_slot, zin, zout, op_mu, s);
   else if (levels == 2)
-    launch_frame3_shape<T, TZ, 2>(shape, probs, states, items, nitems, u_slot, f_slot, zin, zout, op_mu, s);
+    launch_frame3_shape<T, TZ, 2>(shape, seg, probs, states, items, nitems, u_slot, f_slot, zin, zout, op_mu, s);
   else
     launch_frame_levels<T, TZ>(probs, states, items, sec, levels, u_slot, f_slot, zin, zout, op_mu, s);
 }
@@ -1082,6 +1098,9 @@ cudaError_t frame_set_smem() {
   return cudaSuccess;
 }
 
+template <typename T, typename TZ, int L, int SG>
+const void* frame3_seg_kernel() { return (const void*)k_frame3<T, TZ, L, F3_SEG_NWR, 2, 0, SG>; }
+
 bool is_frame_kernel(const void* func) {
   for (int sh = 0; sh < FRAME_SHAPES; ++sh) {
     const void* k[] = {frame3_kernel<float, float, 1>(sh), frame3_kernel<float, float, 2>(sh),
@@ -1090,6 +1109,14 @@ bool is_frame_kernel(const void* func) {
     for (const void* f : k)
       if (f == func) return true;
   }
+#define X(SG)                                                                                     \
+  for (const void* f : {frame3_seg_kernel<float, float, 1, SG>(), frame3_seg_kernel<float, float, 2, SG>(), \
+                        frame3_seg_kernel<float, __nv_bfloat16, 1, SG>(),                         \
+                        frame3_seg_kernel<float, __nv_bfloat16, 2, SG>(),                         \
+                        frame3_seg_kernel<double, double, 1, SG>(), frame3_seg_kernel<double, double, 2, SG>()}) \
+    if (f == func) return true;
+  X(16) X(8) X(4)
+#undef X
   for (int k = 0; k < 3; ++k)
     if (func == lev_kernels<float, float>()[k] || func == lev_kernels<float, __nv_bfloat16>()[k] ||
         func == lev_kernels<double, double>()[k])
@@ -1099,7 +1126,7 @@ bool is_frame_kernel(const void* func) {
 
 #define INST(T, TZ)                                                                          \
   template void launch_frame<T, TZ>(const Prob*, State*, const int2*, int, const int*, int,   \
-                                    int, const void*, void*, double, int, int, cudaStream_t); \
+                                    int, const void*, void*, double, int, int, int, cudaStream_t); \
   template cudaError_t frame_set_smem<T, TZ>();
 INST(float, float)
 INST(float, __nv_bfloat16)

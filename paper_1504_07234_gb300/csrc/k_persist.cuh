@@ -123,7 +123,7 @@ k_persist(const Prob* __restrict__ probs, State* __restrict__ states, int nprob,
             const int i = 4 * u + sub4;
             if (i >= cnt) continue;
             const BlkSub<64> b{1 + sub4};
-            frame3_body<T, TZ, L, 2, 2, 0>(it[i], probs, states, -1, SL_F, nullptr, nullptr, 0.0,
+            frame3_body<T, TZ, L, 2, 2, 0, F3_SEG>(it[i], probs, states, -1, SL_F, nullptr, nullptr, 0.0,
                                            smraw + (size_t)sub4 * frame_slot, b);
             b.sync();
           }

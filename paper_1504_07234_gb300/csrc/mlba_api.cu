@@ -77,10 +77,10 @@ struct StepItems {
 // (section 0); levels >= 3, the BC fold of the correlation (section 0, BC
 // problems that apply A^T), the low-pass chain (section 1) and the level
 // kernels of level L .. 1 (sections 2 ..).
-void add_frame_items(const Prob& pd, int i, int levels, int shape,
+void add_frame_items(const Prob& pd, int i, int levels, int shape, int seg,
                      std::vector<int2> (&fs)[FRAME_SECTIONS]) {
   auto add = [&](std::vector<int2>& L, int nblk) { for (int k = 0; k < nblk; ++k) L.push_back(make_int2(i, k)); };
-  if (levels <= 2) { add(fs[0], frame_tiles(pd.nf, levels, shape)); return; }
+  if (levels <= 2) { add(fs[0], frame_tiles(pd.nf, levels, shape, seg)); return; }
   if (pd.use_adj && pd.bc != BC_RECT && pd.bc != BC_AR && !pd.balanced) add(fs[0], pd.nblk_vec);
   add(fs[1], lowpass_blocks(pd.nf));
   for (int k = 0; k < levels; ++k) add(fs[2 + k], lev_tiles(pd.nf, levels - k));
@@ -138,6 +138,7 @@ struct mlba_batch {
   cudaGraphExec_t x_head = nullptr, x_body = nullptr, x_tail = nullptr;
   // framelet tile shape (k_frame.cu) and how it was chosen
   int frame_shape = 0;
+  int frame_seg = 32;           // rows a warp sweeps (frame_segment)
   int frame_tuned = 0;          // 0 default, 1 measured here, 2 from the cache, 3 forced
   float frame_us = 0.f;         // measured time of one launch of the chosen shape
   // Persistent schedule (opts.persistent): the stage program of one step, the
@@ -391,7 +392,7 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
     launch_balance<T>(P, S, L.balance.dev, L.balance.count, s);
     // a1: z += W u, x = S_mu(z), f = W^T x
     launch_frame<T, TZ>(P, S, L.frame.dev, L.frame.count, L.frame.sec, -1, SL_F, nullptr, nullptr,
-                        0.0, B->levels, B->frame_shape, s);
+                        0.0, B->levels, B->frame_shape, B->frame_seg, s);
   }
 }
 
@@ -432,10 +433,10 @@ void collect_fc(const Prob& pd, int i, const Prob& sf, const Prob& sa, StepItems
   }
 }
 
-void collect_step(const Prob& pd, int i, int levels, int shape, StepItems& V) {
+void collect_step(const Prob& pd, int i, int levels, int shape, int seg, StepItems& V) {
   auto add = [&](std::vector<int2>& L, int nblk) { for (int k = 0; k < nblk; ++k) L.push_back(make_int2(i, k)); };
   if (!pd.fc) add(V.blur, pd.nblk_blur);
-  add_frame_items(pd, i, levels, shape, V.frame);
+  add_frame_items(pd, i, levels, shape, seg, V.frame);
   if (pd.use_adj && !pd.fc) {
     if (pd.bc == BC_AR) add(V.reblur, pd.nblk_blur);
     else add(V.corr, pd.nblk_corr);
@@ -531,7 +532,7 @@ int build_split(mlba_batch* B) {
   StepItems V[2];
   for (int i = 0; i < count; ++i) {
     const Prob& pd = B->hp[i].pd;
-    collect_step(pd, i, B->levels, B->frame_shape, V[grp[i]]);
+    collect_step(pd, i, B->levels, B->frame_shape, B->frame_seg, V[grp[i]]);
     if (pd.fc)
       collect_fc(pd, i, B->fc[pd.fc_sh[0] - count].pd, B->fc[pd.fc_sh[1] - count].pd, V[grp[i]]);
   }
@@ -581,7 +582,7 @@ int set_smem_attrs(mlba_batch* B) {
 }
 
 void frame_shape_of(const mlba_batch* B, int* tx, int* ty, int* pf) {
-  frame_shape(B->frame_shape, tx, ty, pf);
+  frame_shape(B->frame_shape, B->frame_seg, tx, ty, pf);
 }
 
 void destroy_batch(mlba_batch* B) {
@@ -939,19 +940,19 @@ void tune_store(const std::string& key, int shape, float us) {
 void launch_frame_any(mlba_batch* B, const int2* items, int count, int shape, cudaStream_t s) {
   if (B->dtype == MLBA_F64)
     launch_frame<double, double>(B->d_probs, B->d_states, items, count, nullptr, -1, SL_F, nullptr,
-                                 nullptr, 0.0, B->levels, shape, s);
+                                 nullptr, 0.0, B->levels, shape, 32, s);
   else if (B->z_store == MLBA_BF16)
     launch_frame<float, __nv_bfloat16>(B->d_probs, B->d_states, items, count, nullptr, -1, SL_F,
-                                       nullptr, nullptr, 0.0, B->levels, shape, s);
+                                       nullptr, nullptr, 0.0, B->levels, shape, 32, s);
   else
     launch_frame<float, float>(B->d_probs, B->d_states, items, count, nullptr, -1, SL_F, nullptr,
-                               nullptr, 0.0, B->levels, shape, s);
+                               nullptr, 0.0, B->levels, shape, 32, s);
 }
 
 std::vector<int2> frame_items(const mlba_batch* B, int shape) {
   std::vector<int2> v;
   for (size_t i = 0; i < B->hp.size(); ++i) {
-    const int nb = frame_tiles(B->hp[i].pd.nf, B->levels, shape);
+    const int nb = frame_tiles(B->hp[i].pd.nf, B->levels, shape, 32);
     for (int k = 0; k < nb; ++k) v.push_back(make_int2((int)i, k));
   }
   return v;
@@ -985,9 +986,32 @@ int time_frame_shape(mlba_batch* B, int shape, float* us) {
   return MLBA_OK;
 }
 
+// Rows a warp of the fused framelet sweep owns (L <= 2, built-in shape).  A
+// warp's sweep is one chain of rows (72 of them for 32 owned rows at L = 2),
+// so a launch with few warps lasts as long as that chain while most of the
+// chip idles; shorter segments give more and shorter chains at the price of
+// recomputed halo rows (2.25 swept rows per owned row at 32, 2.5 at 16, 3 at
+// 8, 4 at 4).  Halve while the doubled number of warps is resident at once:
+// about 20 FP32 warps per SM; in FP64 one warp per scheduler, because the
+// FP64 pipe is already full with one.  Measured per launch, 32 rows against
+// the choice: 256^2 FP32 32 -> 10 us (4 rows), 72^2 FP64 L = 1 150 -> 27 us (4);
+// 1044^2 BF16 z 45 -> 39 us (16; 8: 44, 4: 54); the 64-problem batch stays at
+// 32 (16: +0.5 %, 8: +10 %).
+int frame_segment(const mlba_batch* B) {
+  const double resident = B->dtype == MLBA_F64 ? 608.0 : 3040.0;
+  for (int seg = 32;; seg /= 2) {
+    double warps = 0.0;      // at half the segment
+    for (const HostProb& h : B->hp) warps += 2.0 * frame_tiles(h.pd.nf, B->levels, 0, seg / 2);
+    if (seg == 4 || warps > resident) return seg;
+  }
+}
+
 int choose_frame_shape(mlba_batch* B, const mlba_opts& o) {
   B->frame_shape = 0;
   B->frame_tuned = 0;
+  // (a forced or measured shape, and the persistent schedule, keep 32 rows)
+  B->frame_seg = 32;
+  if (B->levels <= 2 && o.frame_shape < 0 && !o.autotune && !o.persistent) B->frame_seg = frame_segment(B);
   const bool shaped = B->levels <= 2 && B->dtype != MLBA_F64;   // FP64: one shape
   if (!shaped) return MLBA_OK;
   if (o.frame_shape >= 0) {
@@ -1490,7 +1514,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
     const int trc = choose_frame_shape(B, o);
     if (trc != MLBA_OK) { destroy_batch(B); return trc; }
     std::vector<int2> fs[FRAME_SECTIONS];
-    for (int i = 0; i < count; ++i) add_frame_items(B->hp[i].pd, i, B->levels, B->frame_shape, fs);
+    for (int i = 0; i < count; ++i) add_frame_items(B->hp[i].pd, i, B->levels, B->frame_shape, B->frame_seg, fs);
     if (build_frame_list(B, B->frame, fs, B->levels) != MLBA_OK) { destroy_batch(B); return MLBA_E_CUDA; }
   }
   // ---- capture one step (branch streams first: a capture forks into them)
@@ -1771,7 +1795,7 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
         launch_stencil<double>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->smem_stencil, s);
         launch_stencil<double>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->smem_stencil, s);
       }
-      if (stage == 4) launch_frame<double, double>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, s);
+      if (stage == 4) launch_frame<double, double>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, B->frame_seg, s);
     } else {
       if (stage == 1) launch_stencil<float>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->smem_stencil, s);
       if (stage == 2) {
@@ -1790,9 +1814,9 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
       }
       if (stage == 4) {
         if (B->z_store == MLBA_BF16)
-          launch_frame<float, __nv_bfloat16>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, s);
+          launch_frame<float, __nv_bfloat16>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, B->frame_seg, s);
         else
-          launch_frame<float, float>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, s);
+          launch_frame<float, float>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, B->frame_seg, s);
       }
     }
   }
@@ -2248,11 +2272,11 @@ int mlba_op_frame(mlba_ctx* c, const void* z_in, const void* u, void* z_out, voi
   if (rc != MLBA_OK) return rc;
   if (reset_opstates(B) != MLBA_OK) return MLBA_E_CUDA;
   if (B->dtype == MLBA_F64)
-    launch_frame<double, double>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->stream);
+    launch_frame<double, double>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->frame_seg, B->stream);
   else if (B->z_store == MLBA_BF16)
-    launch_frame<float, __nv_bfloat16>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->stream);
+    launch_frame<float, __nv_bfloat16>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->frame_seg, B->stream);
   else
-    launch_frame<float, float>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->stream);
+    launch_frame<float, float>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->frame_seg, B->stream);
   CK(cudaGetLastError());
   if (grouped) {
     launch_z_layout(dzo, gzo, pd.levels, pd.nf, es, 0, B->stream);

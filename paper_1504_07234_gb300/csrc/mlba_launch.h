@@ -96,11 +96,11 @@ void launch_spectrum_setup(int transform, int n, int p, int half, int cb, const 
 template <typename T, typename TZ>
 void launch_frame(const Prob* probs, State* states, const int2* items, int nitems, const int* sec,
                   int u_slot, int f_slot, const void* zin, void* zout, double op_mu, int levels,
-                  int shape, cudaStream_t s);
-int frame_tiles(int nf, int levels, int shape);   // CTAs of the fused sweep for one problem (L <= 2)
+                  int shape, int seg, cudaStream_t s);
+int frame_tiles(int nf, int levels, int shape, int seg);   // CTAs of the fused sweep for one problem (L <= 2)
 int lev_tiles(int nf, int lev);                   // CTAs of one level kernel (L >= 3)
 int lowpass_blocks(int nf);                       // CTAs of one low-pass launch (L >= 3)
-void frame_shape(int shape, int* tile_x, int* tile_y, int* prefetch);
+void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch);
 bool is_frame_kernel(const void* func);  // func is one of the framelet-update kernels
 int stencil_tiles(int outN);             // CTAs of the stencil for an outN x outN output
 // z layout: the 8 high-pass bands of a level contiguous per position, in

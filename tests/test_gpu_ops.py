@@ -234,3 +234,31 @@ def test_transform_ctas_full_and_split(M, n, transform, psf):
         out.append(b.result(count - 1))
         b.close()
     assert rel_err(out[1], out[0]) <= 1e-5
+
+
+@pytest.mark.parametrize("dtype,zs", [("f32", "f32"), ("f32", "bf16"), ("f64", "f64")])
+@pytest.mark.parametrize("levels", [1, 2])
+def test_frame_segments_give_the_same_iterates(M, dtype, zs, levels):
+    """The rows a warp of the framelet sweep owns follow from the number of
+    warps of the batch (4, 8, 16 or 32 rows; the reported tile has two
+    segments).  Every segment height computes the same values: batches of 1 to
+    600 copies of two problems (50 x 50 reflective, 33 + 4 squared rectangular)
+    end with the bits of the batch of one."""
+    ra = I.psf_gaussian(0.8, 5)
+    descs = []
+    for bc, n in (("reflective", 50), ("rect", 33)):
+        f = I.true_image(n + 4, n)
+        g, delta = I.observe(f, ra, 0.02, n)
+        descs.append(dict(psf=ra, g=g.astype(np.float64 if dtype == "f64" else np.float32), delta=delta,
+                          bc=bc, precond="none"))
+    ref, seen = None, set()
+    for count in (1, 8, 16, 30, 75, 150, 600):
+        b = M.Batch(descs * count, dtype=dtype, z_store=zs, levels=levels, stop=False, max_iter=4)
+        seen.add(b.tiles()["tile_y"])
+        b.iterate(3)
+        out = [b.result(2 * count - 2), b.result(2 * count - 1)]
+        b.close()
+        ref = ref or out
+        for a, c in zip(ref, out):
+            np.testing.assert_array_equal(a, c)
+    assert seen == {8, 16, 32, 64}, seen
