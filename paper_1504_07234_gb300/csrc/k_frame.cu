@@ -131,12 +131,23 @@ constexpr int F3_TX = 26;      // tile columns: level-2 output lanes 3..28 after
 // per framelet launch; distances 1..10 tried)
 constexpr int Z_L2_AHEAD = 2;   // k_frame3
 constexpr int LV_L2_AHEAD = 1;  // k_frame_lev
+// k_frame_lev: rows of the register queue and resident CTAs per SM (FP32) by
+// segment height.  Long segments run with the SM full of warps, where a row
+// takes longer than an L2 access: one queued row and 64 registers (4096^2,
+// L = 4, a step: 2.04 ms with 3 rows at 96 registers, 1.98 with 3 rows in 80,
+// 1.97 with 1 row in 64).  Short ones run in idle SMs: 3 rows (226^2: 2 %
+// faster per step than 1).
+__host__ __device__ constexpr int lv_pf(int seg) { return seg >= 16 ? 1 : 3; }
+__host__ __device__ constexpr int lv_minb(int seg, int elem_bytes) { return seg >= 16 && elem_bytes == 4 ? 32 : 1; }
 constexpr int F3_SEG = 32;     // rows per warp of the tile shapes below
 constexpr int F3_SEG_NWR = 2;   // warps per CTA of the sweeps with shorter segments (16, 8, 4 rows)
 // Tile shapes the autotuner chooses from: warps (32-row segments) per CTA and
 // the z prefetch distance in rows.  Every shape computes the same values in
 // the same order (a warp's sweep does not depend on its CTA), so the choice
-// changes the time only.  Shape 0 is the default; FP64 always uses it.
+// changes the time only.  Shape 0 is the default; FP64 always uses it.  Its
+// queue of one row (the L2 prefetch hides the rest) lets the sweep keep its
+// rings in place (f3_level): a launch of 4096^2, L = 2 went from 419 to 406 us
+// together with the sum / difference form of the masks (f3_row).
 // Shapes with ring > 0 stream each warp's z rows through a ring of `ring`
 // row slots in shared memory, filled by bulk asynchronous copies (one 1 KB
 // copy per row for FP32 z, 512 B for BF16) so that many rows are in flight
@@ -144,7 +155,7 @@ constexpr int F3_SEG_NWR = 2;   // warps per CTA of the sweeps with shorter segm
 // image edge (mirrored columns) fill the same ring with per-lane 16-byte
 // asynchronous copies.
 struct F3Shape { int nwr, pf, ring; };
-constexpr F3Shape F3_SHAPES[FRAME_SHAPES] = {{2, 2, 0}, {1, 2, 0}, {4, 2, 0}, {2, 3, 0}, {1, 3, 0},
+constexpr F3Shape F3_SHAPES[FRAME_SHAPES] = {{2, 1, 0}, {1, 2, 0}, {4, 2, 0}, {2, 3, 0}, {1, 3, 0},
                                              {2, 2, 6}, {2, 2, 10}, {1, 2, 12}};
 
 template <int L, int NWR, int SEG = F3_SEG>
@@ -193,6 +204,85 @@ __device__ __forceinline__ float to_z(float v, float*) { return v; }
 __device__ __forceinline__ double to_z(double v, double*) { return v; }
 __device__ __forceinline__ __nv_bfloat16 to_z(float v, __nv_bfloat16*) { return __float2bfloat16_rn(v); }
 
+// S_mu(v) = v - clamp(v, -mu, mu).  FP64: the comparison on the bits of |v|
+// (for mu >= 0 the same values, NaN and infinities included), because a
+// comparison in FP64 costs as much as an addition there and the FP64 pipe is
+// what bounds the sweep.
+__device__ __forceinline__ float f3_soft(float v, float mu) { return v - fminf(fmaxf(v, -mu), mu); }
+__device__ __forceinline__ double f3_soft(double v, double mu) {
+  const long long m = __double_as_longlong(v) & 0x7fffffffffffffffll;
+  const double c = m > __double_as_longlong(mu) ? copysign(mu, v) : v;
+  return v - c;
+}
+// v with its sign flipped when the (sign-bit) mask is set
+__device__ __forceinline__ float f3_flip(float v, int m) { return __int_as_float(__float_as_int(v) ^ m); }
+__device__ __forceinline__ double f3_flip(double v, int m) {
+  return __hiloint2double(__double2hiint(v) ^ m, __double2loint(v));
+}
+
+// One row of coefficients of a level: rows ha, hb, hc of the horizontal
+// analysis at y - D, y, y + D (h[j], mask j), the row's z (group and, with
+// LOW, the low-pass value zl), the threshold, and the vertical synthesis
+// into pa += (row y - D), pb += (row y), pc = (row y + D, its first
+// contribution).  mrow, mcol, m11: sign masks of mirrored rows / columns for
+// the antisymmetric bands.  The masks are applied through their sums and
+// differences: with s = h_a + h_c, d = h_a - h_c,
+//   z0 += s / 4 + h_b / 2,  z1 += (sqrt 2 / 4) d,  z2 += h_b / 2 - s / 4,
+// and the transpose the same way: 14 operations per horizontal mask instead
+// of 19 (FP32: an issue-bound sweep; FP64: the pipe is full).
+template <bool LOW, typename T, typename TZ>
+__device__ __forceinline__ void f3_row(const T (&ha)[3], const T (&hb)[3], const T (&hc)[3],
+                                       const ZGroup<TZ>& zi, TZ zl, int mrow, int mcol, T mu,
+                                       ZGroup<TZ>& zo, TZ& zlo, T (&pa)[3], T (&pb)[3], T (&pc)[3]) {
+  const T s2q = T(0.35355339059327376220);               // sqrt(2) / 4
+  const int m11 = mrow ^ mcol;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const T s = ha[j] + hc[j], d = ha[j] - hc[j];
+    auto in = [&](int i) {                               // z of band (i, j), mirrored sign applied
+      T v = T(ld_z(&zi.e[3 * i + j - 1]));
+      if (i == 1 && j == 1) v = f3_flip(v, m11);
+      else if (i == 1) v = f3_flip(v, mrow);
+      else if (j == 1) v = f3_flip(v, mcol);
+      return v;
+    };
+    T x0 = T(0);
+    if (j > 0 || LOW) {
+      const T v = j == 0 ? T(ld_z(&zl)) : in(0);
+      const T zn = fma(T(0.5), hb[j], fma(T(0.25), s, v));
+      if (j == 0) zlo = to_z(zn, (TZ*)nullptr);
+      else zo.e[j - 1] = to_z(zn, (TZ*)nullptr);
+      x0 = f3_soft(zn, mu);
+    }
+    const T z1 = fma(s2q, d, in(1));
+    const T z2 = fma(T(0.5), hb[j], fma(T(-0.25), s, in(2)));
+    zo.e[3 + j - 1] = to_z(z1, (TZ*)nullptr);
+    zo.e[6 + j - 1] = to_z(z2, (TZ*)nullptr);
+    const T x1 = f3_soft(z1, mu), x2 = f3_soft(z2, mu);
+    const T D = (j > 0 || LOW) ? x0 - x2 : -x2;
+    const T S = (j > 0 || LOW) ? x0 + x2 : x2;
+    pa[j] = fma(s2q, x1, fma(T(0.25), D, pa[j]));
+    pb[j] = fma(T(0.5), S, pb[j]);
+    pc[j] = fma(-s2q, x1, T(0.25) * D);
+  }
+}
+// horizontal analysis of one position (values at x - D, x, x + D)
+template <typename T>
+__device__ __forceinline__ void f3_hrow(T cm, T c0, T cp, T (&h)[3]) {
+  const T t = T(0.25) * (cm + cp);
+  h[0] = fma(T(0.5), c0, t);
+  h[1] = T(0.35355339059327376220) * (cm - cp);
+  h[2] = fma(T(0.5), c0, -t);
+}
+// horizontal synthesis parts of a completed row: A(x + D) + B(x) + C(x - D)
+template <typename T>
+__device__ __forceinline__ void f3_abc(const T (&P)[3], T& A, T& B, T& C) {
+  const T e = T(0.25) * (P[0] - P[2]), s2q = T(0.35355339059327376220);
+  A = fma(s2q, P[1], e);
+  B = T(0.5) * (P[0] + P[2]);
+  C = fma(-s2q, P[1], e);
+}
+
 // A warp's ring of z rows (RING > 0): slot k holds one row's 32 groups at
 // buf + k * 256 values and completes on bar[k]; seq counts the rows that went
 // through the bulk path (every bulk row advances one slot and, every RING rows,
@@ -216,9 +306,6 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
   constexpr bool TOP = (LEV == L);
   constexpr int XO = (LEV == 2) ? 3 : 1;                 // first coefficient column tx0 - XO
   constexpr int NL = (LEV == 2) ? 32 : F3_TX + 2;        // lanes with a coefficient column
-  constexpr int K0 = TOP ? 0 : 1;                        // band k = 3 j + i; (0,0) only at level L
-  constexpr int NB = 9 - K0;
-  const T s2q = T(0.35355339059327376220);               // sqrt(2) / 4
   const int lane = threadIdx.x & 31;
   const int x = tx0 - XO + lane;
   const bool act = lane < NL;
@@ -231,7 +318,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
   // column part of the z offsets and its mirroring parity
   bool pcx;
   const int zc = f3_refl(x, nf, &pcx);
-  const T scol = pcx ? T(-1) : T(1);
+  const int mcol = pcx ? (int)0x80000000 : 0;
   const bool own_c = act && x >= tx0 && x < tx0 + F3_TX && x < nf;
   // owned rows [seg_lo, own_hi): one unsigned compare per row
   const unsigned own_rows = (unsigned)max(min(seg_hi, nf) - seg_lo, 0);
@@ -266,15 +353,19 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
       const T* r = ccol + (y - cy0) * cpitch;
       cm = r[-D]; c0 = r[0]; cp = r[D];
     }
-    const T sp = cm + cp;
-    h[0] = T(0.25) * sp + T(0.5) * c0;
-    h[1] = s2q * (cm - cp);
-    h[2] = T(0.5) * c0 - T(0.25) * sp;
+    f3_hrow(cm, c0, cp, h);
   };
   if constexpr (LEV == 2) {
     grow(yc0 - D - 1, gr[0]);
     grow(yc0 - D, gr[1]);
   }
+  // Ring slots.  A queue of one row: the sweep is unrolled by the ring length
+  // and the rows keep their slots (row y of phase ph has slot ph + D, modulo
+  // the length): nothing moves.  Deeper queues are unrolled by the queue's
+  // length and shift the rings by one row per step (phase 0 always).
+  constexpr int RL = 2 * D + 1;
+  constexpr bool STATIC_RING = F3_PF == 1 && RING == 0;
+  constexpr int UNR = STATIC_RING ? RL : F3_PF;
 #pragma unroll
   for (int k = 0; k < 2 * D; ++k) hrow(yc0 - D + k, hr[k]);
   // z queue: rows y .. y + PF - 1 (group and low-pass value per row; with a
@@ -284,14 +375,14 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
   // each queued row's mirrored offset and mirroring parity, mapped once when
   // the row is queued and used again when it is swept
   int zqo[F3_PF];
-  bool zqp[F3_PF];
+  int zqm[F3_PF];              // (the parity as a sign mask)
   // (idle lanes load a valid mirrored column too; their values are unused.
   // Offsets stay in 32 bits: nbands nf^2 < 2^31.)
   auto zload = [&](int y, int k) {
     bool par;
     const int q = f3_refl(y, nf, &par) * nf + zc;
     zqo[k] = q;
-    zqp[k] = par;
+    zqm[k] = par ? (int)0x80000000 : 0;
     if constexpr (RING == 0) {
       const uint4* src = reinterpret_cast<const uint4*>(zin + (gbase + 8 * q));
 #pragma unroll
@@ -351,7 +442,9 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
   // one coefficient row; queue slot kq holds its z and is refilled with row
   // y + PF.  The queue is indexed statically (the sweep is unrolled by PF) so
   // that no register receiving an outstanding load is copied before it is used.
-  auto step = [&](int y, int kq) {
+  auto step = [&](int y, int k) {
+    const int kq = STATIC_RING ? 0 : k, ph = STATIC_RING ? k : 0;
+    const int ia = ph, ib = (ph + D) % RL, ic = (ph + 2 * D) % RL;   // rows y - D, y, y + D
     if constexpr (RING > 0) {
       // this row's groups from the ring, then the slot is refilled with row y + RING
       const int i = y - yc0;
@@ -374,34 +467,15 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
       if (i + RING < nrows && !rg.bad) issue(i + RING);
       else if (!bulk) cp_commit();
     }
-    hrow(y + D, hr[2 * D]);
+    hrow(y + D, hr[ic]);
     // z outside the image is its mirror image; antisymmetric (b1) bands
     // change sign under an odd number of mirrorings
-    const T srow = zqp[kq] ? T(-1) : T(1);
-    const T s11 = srow * scol;
     const bool own = own_c && (unsigned)(y - seg_lo) < own_rows;
     const int zwo = zqo[kq];
     ZGroup<TZ> zo;
     TZ zlo = TZ(0.0f);
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int k = K0 + b, i = k % 3, j = k / 3;
-      const T bi0 = (i == 0) ? T(0.25) : (i == 1 ? s2q : T(-0.25));
-      const T bi1 = (i == 1) ? T(0) : T(0.5);
-      const T bi2 = (i == 0) ? T(0.25) : (i == 1 ? -s2q : T(-0.25));
-      T a = bi0 * hr[0][j] + bi2 * hr[2 * D][j];
-      if (i != 1) a += bi1 * hr[D][j];
-      const int pos = 3 * i + j - 1;              // place in the group ((0,0): low-pass)
-      const T zv = (i == 0 && j == 0) ? T(ld_z(&zl[kq])) : T(ld_z(&zq[RING > 0 ? 0 : kq].e[pos]));
-      const T zn = (i == 1 && j == 1) ? fma(zv, s11, a)
-                 : (i == 1) ? fma(zv, srow, a) : (j == 1) ? fma(zv, scol, a) : zv + a;
-      if (i == 0 && j == 0) zlo = to_z(zn, (TZ*)nullptr);
-      else zo.e[pos] = to_z(zn, (TZ*)nullptr);
-      const T xv = zn - fmin(fmax(zn, -mu), mu);     // S_mu
-      pr[0][j] += bi0 * xv;
-      if (i != 1) pr[D][j] += bi1 * xv;
-      pr[2 * D][j] += bi2 * xv;
-    }
+    f3_row<TOP, T, TZ>(hr[ia], hr[ib], hr[ic], zq[RING > 0 ? 0 : kq], zl[kq], zqm[kq], mcol, mu, zo, zlo,
+                       pr[ia], pr[ib], pr[ic]);
     if (own) {
       uint4* dstz = reinterpret_cast<uint4*>(zout + (gbase + 8 * zwo));
 #pragma unroll
@@ -424,9 +498,8 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     // row y - D has all its contributions: horizontal synthesis
     const int r = y - D;
     if (r >= yo0) {
-      const T A = T(0.25) * pr[0][0] + s2q * pr[0][1] - T(0.25) * pr[0][2];
-      const T B = T(0.5) * (pr[0][0] + pr[0][2]);
-      const T C = T(0.25) * pr[0][0] - s2q * pr[0][1] - T(0.25) * pr[0][2];
+      T A, B, C;
+      f3_abc(pr[ia], A, B, C);
       const T out = B + __shfl_down_sync(FULL, A, D) + __shfl_up_sync(FULL, C, D);
       if (LEV == 2 && L == 2) {
         // s_1 row r (lanes 2..29) -> (b0 x b0)^T s_1 row r - 1 (lanes 3..28)
@@ -444,17 +517,17 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
         }
       }
     }
-    // shift the rings
+    if constexpr (!STATIC_RING) {
 #pragma unroll
-    for (int k = 0; k < 2 * D; ++k)
+      for (int q = 0; q < 2 * D; ++q)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) { hr[k][j] = hr[k + 1][j]; pr[k][j] = pr[k + 1][j]; }
-    pr[2 * D][0] = pr[2 * D][1] = pr[2 * D][2] = T(0);
+        for (int j = 0; j < 3; ++j) { hr[q][j] = hr[q + 1][j]; pr[q][j] = pr[q + 1][j]; }
+    }
   };
 #pragma unroll 1
-  for (int y = yc0; y < yc1; y += F3_PF) {
+  for (int y = yc0; y < yc1; y += UNR) {
 #pragma unroll
-    for (int k = 0; k < F3_PF; ++k)
+    for (int k = 0; k < UNR; ++k)
       if (y + k < yc1) step(y + k, k);
   }
   if constexpr (RING > 0) {
@@ -673,49 +746,49 @@ k_lowpass(const Prob* __restrict__ probs, const State* __restrict__ states,
 // order of dp (Poly): the taps dp apart join neighbouring positions m - 1, m,
 // m + 1 of one sub-lattice, so the kernel runs the dilation-1 sweep on each
 // of the dp^2 sub-lattices (a, b) (columns x = a + dp m, rows y = b + dp m).
-// A CTA of LV_NWR warps owns OUTW positions of a column sub-lattice x 32
-// LV_NWR positions of a row sub-lattice; lane k of a warp owns the
-// coefficient column m = tx0 - 1 + k (every lane computes coefficients, lanes
-// 1 .. 30 produce output).  The halo is one position whatever dp is.
+// A CTA (one warp) owns OUTW positions of a column sub-lattice x SEG
+// positions of a row sub-lattice; lane k owns the coefficient column
+// m = tx0 - 1 + k (every lane computes coefficients, lanes 1 .. 30 produce
+// output).  The halo is one position whatever dp is.
+template <int SEG>
 struct LV {
   static constexpr int OUTW = 30;                 // output columns of a tile
-  static constexpr int TY = 32 * LV_NWR;
+  static constexpr int TY = SEG;
   static constexpr int CW = 34, CH = TY + 4;      // c tile: positions tx0 - 2.., ty0 - 2..
-  static constexpr int PR = 3;                    // synthesis ring rows
 };
-template <typename T>
+template <typename T, int SEG>
 __host__ __device__ constexpr size_t lev_smem_bytes() {
-  return ((size_t)LV::CW * LV::CH + (size_t)LV_NWR * LV::PR * 3 * 32) * sizeof(T);
+  return (size_t)LV<SEG>::CW * LV<SEG>::CH * sizeof(T);
 }
 // tiles of one sub-lattice pair and of the whole level
-__host__ __device__ inline void lev_tile_grid(int nf, int dp, int* tx, int* ty) {
+__host__ __device__ inline void lev_tile_grid(int nf, int dp, int seg, int* tx, int* ty) {
   const int m = Poly(nf, dp).count_max();
-  *tx = (m + LV::OUTW - 1) / LV::OUTW;
-  *ty = (m + LV::TY - 1) / LV::TY;
+  *tx = (m + LV<32>::OUTW - 1) / LV<32>::OUTW;
+  *ty = (m + seg - 1) / seg;
 }
 
 // One level of the step.  The warp sweeps down its rows (one row
-// sub-lattice): the horizontal analysis of the three rows m - 1, m, m + 1 of
-// c_{l-1} (shared-memory tile, polyphase order of dp), the vertical masks,
-// the update of z (register queue, PF rows ahead; z of the level in the same
-// order), the threshold, and the vertical synthesis scattered into a ring of
-// three rows (shared memory, one column per lane); row m - 1 then has all
-// its contributions and is combined horizontally by warp shuffles at +-1 and,
-// for l < L, with (b0 x b0)^T s_l: each lane loads s_l at its own column
-// with the z rows (PF rows ahead) and keeps the horizontally filtered rows
-// m - 2 .. m in registers (shuffles at +-1).  s_{l-1} is written in the
+// sub-lattice): the horizontal analysis of row m + 1 of c_{l-1} (shared-memory
+// tile, polyphase order of dp) joins rows m - 1 and m in a register ring, then
+// the vertical masks, the update of z (register queue, PF rows ahead; z of the
+// level in the same order), the threshold, and the vertical synthesis into a
+// register ring of three rows (f3_row); row m - 1 then has all its
+// contributions and is combined horizontally by warp shuffles at +-1 and, for
+// l < L, with (b0 x b0)^T s_l: each lane loads s_l at its own column with the
+// z rows and keeps the horizontally filtered rows m - 2 .. m in registers
+// (shuffles at +-1).  The sweep is unrolled by the ring length, so every ring
+// and queue index is static and nothing moves.  s_{l-1} is written in the
 // polyphase order of dp / 2 (f, and s_1, plainly).  Coefficients outside the
 // image are mirrored with the sign of the band's symmetry, as in k_frame3.
-template <typename T, typename TZ, bool TOP>
-__global__ void __launch_bounds__(32 * LV_NWR)
+template <typename T, typename TZ, bool TOP, int SEG>
+__global__ void __launch_bounds__(32, lv_minb(SEG, sizeof(T)))
 k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
             const int2* __restrict__ items, int lev, int u_slot, int f_slot, const void* zin_op,
             void* zout_op, double op_mu) {
-  using G = LV;
-  constexpr int PF = 2;
+  using G = LV<SEG>;
+  constexpr int PF = lv_pf(SEG);
+  static_assert(PF == 1 || PF == 3, "queue index static under the unrolling by 3");
   constexpr unsigned FULL = 0xffffffffu;
-  constexpr int K0 = TOP ? 0 : 1;            // band k = 3 j + i; (0,0) only at the top level
-  constexpr int NB = 9 - K0;
   constexpr int NV = 8 * (int)sizeof(TZ) / 16;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int2 item = items[blockIdx.x];
@@ -727,7 +800,7 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
   const int dp = 1 << (lev - 1);
   const Poly P(nf, dp), PO(nf, dp > 1 ? dp / 2 : 1);
   int tX, tY;
-  lev_tile_grid(nf, dp, &tX, &tY);
+  lev_tile_grid(nf, dp, SEG, &tX, &tY);
   int t = item.y;
   const int tx = t % tX;
   t /= tX;
@@ -751,44 +824,36 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
   // (mirrored into the image first)
   auto cpos = [&](int m, int off, bool* par) { return P.pos(f3_refl(off + dp * m, nf, par)); };
   T* sc = reinterpret_cast<T*>(smraw);       // c_{l-1} on rows ty0 - 2.., cols tx0 - 2..
-  T* sring = sc + G::CW * G::CH;             // per-warp synthesis rings
+  const int lane = threadIdx.x;
   {
     const T* cin = (lev == 1) ? frame_u<T>(pd, u_slot)
                               : static_cast<const T*>(pd.lp) + (size_t)(lev - 2) * plane;
-    // one warp per tile row (the row's position mapped once), lanes along the
-    // row (columns lane and lane + 32, mapped once per lane)
+    // lanes along the row (columns lane and lane + 32, mapped once per lane),
+    // each row's position mapped once
     static_assert(G::CW <= 64, "two columns per lane");
-    const int wq = threadIdx.x >> 5, ln = threadIdx.x & 31;
     bool par;
-    const int ax0 = cpos(tx0 - 2 + ln, sa, &par);
-    const bool two = ln + 32 < G::CW;
-    const int ax1 = two ? cpos(tx0 - 2 + ln + 32, sa, &par) : 0;
-    for (int ry = wq; ry < G::CH; ry += LV_NWR) {
+    const int ax0 = cpos(tx0 - 2 + lane, sa, &par);
+    const bool two = lane + 32 < G::CW;
+    const int ax1 = two ? cpos(tx0 - 2 + lane + 32, sa, &par) : 0;
+    for (int ry = 0; ry < G::CH; ++ry) {
       const T* row = cin + (size_t)cpos(ty0 - 2 + ry, sb, &par) * nf;
-      T* d = sc + ry * G::CW + ln;
+      T* d = sc + ry * G::CW + lane;
       if (sizeof(T) == 8) cp_async_8(d, row + ax0); else cp_async_4(d, row + ax0);
       if (two) {
         if (sizeof(T) == 8) cp_async_8(d + 32, row + ax1); else cp_async_4(d + 32, row + ax1);
       }
     }
     cp_commit();
-    for (int idx = threadIdx.x; idx < LV_NWR * G::PR * 3 * 32; idx += 32 * LV_NWR) sring[idx] = T(0);
-    cp_wait<0>();
   }
-  __syncthreads();
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int seg_lo = ty0 + 32 * w, seg_hi = seg_lo + 32;
-  if (seg_lo >= Mb) return;                  // no barrier follows
-  const T s2q = T(0.35355339059327376220);   // sqrt(2) / 4
+  const int seg_lo = ty0, seg_hi = ty0 + SEG;
   const int mx = tx0 - 1 + lane;             // this lane's coefficient column (local)
   bool pcx;
   const int zc = cpos(mx, sa, &pcx);
-  const T scol = pcx ? T(-1) : T(1);
+  const int mcol = pcx ? (int)0x80000000 : 0;
   const bool own_c = lane >= 1 && lane < 31 && mx < Ma;
-  const int yc0 = seg_lo - 1, yc1 = seg_hi + 1;
-  T* ring = sring + w * (G::PR * 3 * 32) + lane;    // (row slot k, j) at ring[(3 k + j) 32]
-  const T* ccol = sc + (lane + 1);                  // c tile column of mx
-  const int crow0 = ty0 - 2;
+  const unsigned own_rows = (unsigned)(min(seg_hi, Mb) - seg_lo);   // owned rows [seg_lo, seg_lo + own_rows)
+  const int yc0 = seg_lo - 1, yc1 = seg_lo + (int)own_rows + 1;
+  const T* ccol = sc + (lane + 1);                  // c tile column of mx, row ty0 - 2
   const int gbase = (lev - 1) * 8 * plane, lbase = 8 * L * plane;
   T* dst = (lev == 1) ? static_cast<T*>(pd.buf[f_slot])
                       : static_cast<T*>(pd.sy) + (size_t)(lev - 2) * plane;
@@ -797,73 +862,53 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
   ZGroup<TZ> zq[PF];
   TZ zl[PF];
   T sq[PF];
-  int zqo[PF];                               // queued rows' offsets and parities
-  bool zqp[PF];
+  int zqo[PF];                               // queued rows' offsets and mirroring masks
+  int zqm[PF];
   auto zload = [&](int y, int k) {
     bool par;
     const int q = cpos(y, sb, &par) * nf + zc;
     zqo[k] = q;
-    zqp[k] = par;
+    zqm[k] = par ? (int)0x80000000 : 0;
     const uint4* src = reinterpret_cast<const uint4*>(zin + (gbase + 8 * q));
 #pragma unroll
     for (int v = 0; v < NV; ++v) zq[k].v[v] = src[v];
     if (TOP) zl[k] = zin[lbase + q];
     else sq[k] = sin[q];                     // s_l at (y, mx), mirrored like z
   };
-  // (b0 x b0)^T s_l: horizontally filtered s_l rows m - 2, m - 1 (registers)
-  T hs2 = T(0), hs1 = T(0);
 #pragma unroll
   for (int k = 0; k < PF; ++k) zload(yc0 + k, k);
-  // ring slots of rows m - 1, m, m + 1 (advanced by one per row)
-  int k0 = 0, k1 = 1, k2 = 2;
-  auto step = [&](int y, int kq) {
-    // horizontal analysis of rows y - 1, y, y + 1: h[s][j]
-    T h[3][3];
+  cp_wait<0>();
+  __syncwarp();
+  auto hrow = [&](int y, T (&h)[3]) {
+    const T* r = ccol + (y - (ty0 - 2)) * G::CW;
+    f3_hrow(r[-1], r[0], r[1], h);
+  };
+  // register rings: slot of row y - 1 is the step's phase, of y the next, of
+  // y + 1 the one after
+  T hr[3][3], pr[3][3];
+  T hs[3] = {T(0), T(0), T(0)};              // horizontally filtered s_l rows
+  hrow(yc0 - 1, hr[0]);
+  hrow(yc0, hr[1]);
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      const T* r = ccol + (y + (s - 1) - crow0) * G::CW;
-      const T cm = r[-1], c0 = r[0], cp = r[1];
-      const T sp = cm + cp;
-      h[s][0] = T(0.25) * sp + T(0.5) * c0;
-      h[s][1] = s2q * (cm - cp);
-      h[s][2] = T(0.5) * c0 - T(0.25) * sp;
-    }
-    const T srow = zqp[kq] ? T(-1) : T(1);
-    const T s11 = srow * scol;
-    const bool own = own_c && y >= seg_lo && y < seg_hi && y < Mb;
+  for (int j = 0; j < 3; ++j) pr[0][j] = pr[1][j] = pr[2][j] = T(0);
+  auto step = [&](int y, int ph) {
+    const int ia = ph, ib = (ph + 1) % 3, ic = (ph + 2) % 3, kq = ph % PF;
+    hrow(y + 1, hr[ic]);
+    const bool own = own_c && (unsigned)(y - seg_lo) < own_rows;
     const int zwo = zqo[kq];
     ZGroup<TZ> zo;
     TZ zlo = TZ(0.0f);
-    T p0[3] = {T(0), T(0), T(0)}, p1[3] = {T(0), T(0), T(0)}, p2[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int k = K0 + b, i = k % 3, j = k / 3;
-      const T bi0 = (i == 0) ? T(0.25) : (i == 1 ? s2q : T(-0.25));
-      const T bi1 = (i == 1) ? T(0) : T(0.5);
-      const T bi2 = (i == 0) ? T(0.25) : (i == 1 ? -s2q : T(-0.25));
-      T a = bi0 * h[0][j] + bi2 * h[2][j];
-      if (i != 1) a += bi1 * h[1][j];
-      const int pos = 3 * i + j - 1;
-      const T zv = (i == 0 && j == 0) ? T(ld_z(&zl[kq])) : T(ld_z(&zq[kq].e[pos]));
-      const T zn = (i == 1 && j == 1) ? fma(zv, s11, a)
-                 : (i == 1) ? fma(zv, srow, a) : (j == 1) ? fma(zv, scol, a) : zv + a;
-      if (i == 0 && j == 0) zlo = to_z(zn, (TZ*)nullptr);
-      else zo.e[pos] = to_z(zn, (TZ*)nullptr);
-      const T xv = zn - fmin(fmax(zn, -mu), mu);     // S_mu
-      p0[j] += bi0 * xv;
-      if (i != 1) p1[j] += bi1 * xv;
-      p2[j] += bi2 * xv;
-    }
+    f3_row<TOP, T, TZ>(hr[ia], hr[ib], hr[ic], zq[kq], zl[kq], zqm[kq], mcol, mu, zo, zlo, pr[ia],
+                       pr[ib], pr[ic]);
     if (own) {
       uint4* dz = reinterpret_cast<uint4*>(zout + (gbase + 8 * zwo));
 #pragma unroll
       for (int v = 0; v < NV; ++v) dz[v] = zo.v[v];
       if (TOP) zout[lbase + zwo] = zlo;
     }
-    T hs0 = T(0);
     if (!TOP) {
       const T sv = sq[kq];
-      hs0 = T(0.25) * (__shfl_up_sync(FULL, sv, 1) + __shfl_down_sync(FULL, sv, 1)) + T(0.5) * sv;
+      hs[ic] = T(0.25) * (__shfl_up_sync(FULL, sv, 1) + __shfl_down_sync(FULL, sv, 1)) + T(0.5) * sv;
     }
     if (y + PF < yc1) zload(y + PF, kq);
     {
@@ -876,54 +921,47 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
         else prefetch_l2(sin + qa);
       }
     }
-    // scatter into rows y - 1, y, y + 1; row y - 1 is then complete
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      ring[(3 * k1 + j) * 32] += p1[j];
-      ring[(3 * k2 + j) * 32] += p2[j];
-    }
-    T Pj[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      Pj[j] = ring[(3 * k0 + j) * 32] + p0[j];
-      ring[(3 * k0 + j) * 32] = T(0);         // the slot becomes row y + 2
-    }
+    // row y - 1 is complete
     const int r = y - 1;
-    const T A = T(0.25) * Pj[0] + s2q * Pj[1] - T(0.25) * Pj[2];
-    const T B = T(0.5) * (Pj[0] + Pj[2]);
-    const T C = T(0.25) * Pj[0] - s2q * Pj[1] - T(0.25) * Pj[2];
+    T A, B, C;
+    f3_abc(pr[ia], A, B, C);
     T out = B + __shfl_down_sync(FULL, A, 1) + __shfl_up_sync(FULL, C, 1);
-    if (r >= seg_lo && own_c && r < Mb) {
-      // (b0 x b0)^T s_l at (r, mx): rows r - 1 = y - 2, r, r + 1 = y
-      if (!TOP) out += T(0.25) * (hs2 + hs0) + T(0.5) * hs1;
+    if (r >= seg_lo && own_c) {
+      // (b0 x b0)^T s_l at (r, mx): rows r - 1, r, r + 1 = y
+      if (!TOP) out += T(0.25) * (hs[ia] + hs[ic]) + T(0.5) * hs[ib];
       dst[(size_t)PO.pos(sb + dp * r) * nf + dcol] = out;
     }
-    hs2 = hs1;
-    hs1 = hs0;
-    k0 = (k0 + 1 == G::PR) ? 0 : k0 + 1;
-    k1 = (k1 + 1 == G::PR) ? 0 : k1 + 1;
-    k2 = (k2 + 1 == G::PR) ? 0 : k2 + 1;
   };
 #pragma unroll 1
-  for (int y = yc0; y < yc1; y += PF) {
+  for (int y = yc0; y < yc1; y += 3) {
 #pragma unroll
-    for (int k = 0; k < PF; ++k)
+    for (int k = 0; k < 3; ++k)
       if (y + k < yc1) step(y + k, k);
   }
 }
 
 #ifndef MLBA_BODIES_ONLY  // launchers: not in the persistent kernel's unit
-int lev_tiles(int nf, int lev) {
+int lev_tiles(int nf, int lev, int seg) {
   const int dp = 1 << (lev - 1);
   int tx, ty;
-  lev_tile_grid(nf, dp, &tx, &ty);
+  lev_tile_grid(nf, dp, seg, &tx, &ty);
   return dp * dp * tx * ty;
 }
 int lowpass_blocks(int nf) { return nf; }
 
+// level kernel of a segment height (32 rows: FP64 only)
+template <typename T, typename TZ, bool TOP>
+const void* lev_kernel(int seg) {
+  if (seg == 4) return (const void*)k_frame_lev<T, TZ, TOP, 4>;
+  if (seg == 8) return (const void*)k_frame_lev<T, TZ, TOP, 8>;
+  if constexpr (sizeof(T) == 8)
+    if (seg == 32) return (const void*)k_frame_lev<T, TZ, TOP, 32>;
+  return (const void*)k_frame_lev<T, TZ, TOP, 16>;
+}
+
 template <typename T, typename TZ>
 void launch_frame_levels(const Prob* probs, State* states, const int2* items, const int* sec,
-                         int levels, int u_slot, int f_slot, const void* zin, void* zout,
+                         int levels, int seg, int u_slot, int f_slot, const void* zin, void* zout,
                          double op_mu, cudaStream_t s) {
   // sec: (offset, count) of the fold, low-pass and level-L .. level-1 sections
   if (u_slot < 0 && sec[1] > 0) launch_vec<T>(VEC_FOLD, probs, states, items + sec[0], sec[1], 0, s);
@@ -931,15 +969,14 @@ void launch_frame_levels(const Prob* probs, State* states, const int2* items, co
     for (int l = 1; l < levels; ++l)
       k_lowpass<T><<<sec[3], LP_THREADS, 0, s>>>(probs, states, items + sec[2], l, u_slot);
   for (int k = 0; k < levels; ++k) {
-    const int lev = levels - k, off = sec[4 + 2 * k], cnt = sec[5 + 2 * k];
+    int lev = levels - k;
+    const int off = sec[4 + 2 * k], cnt = sec[5 + 2 * k];
     if (cnt <= 0) continue;
     const int2* it = items + off;
-    if (lev == levels)
-      k_frame_lev<T, TZ, true><<<cnt, 32 * LV_NWR, lev_smem_bytes<T>(), s>>>(
-          probs, states, it, lev, u_slot, f_slot, zin, zout, op_mu);
-    else
-      k_frame_lev<T, TZ, false><<<cnt, 32 * LV_NWR, lev_smem_bytes<T>(), s>>>(
-          probs, states, it, lev, u_slot, f_slot, zin, zout, op_mu);
+    void* args[] = {&probs, &states, &it, &lev, &u_slot, &f_slot, &zin, &zout, &op_mu};
+    const size_t sm = (size_t)LV<32>::CW * (seg + 4) * sizeof(T);
+    cudaLaunchKernel(lev == levels ? lev_kernel<T, TZ, true>(seg) : lev_kernel<T, TZ, false>(seg), dim3(cnt),
+                     dim3(32), args, sm, s);
   }
 }
 
@@ -998,13 +1035,13 @@ void launch_z_layout(void* dst, const void* src, int levels, int nf, int elem_by
 template <typename T, typename TZ, int L>
 const void* frame3_kernel(int shape) {
   if constexpr (sizeof(T) == 8) {
-    return (const void*)k_frame3<T, TZ, L, 2, 2, 0>;
+    return (const void*)k_frame3<T, TZ, L, 2, 1, 0>;
   } else {
     switch (shape) {
 #define X(S, NWR, PF, RING) case S: return (const void*)k_frame3<T, TZ, L, NWR, PF, RING>;
       F3_SHAPE_CASES(X)
 #undef X
-      default: return (const void*)k_frame3<T, TZ, L, 2, 2, 0>;
+      default: return (const void*)k_frame3<T, TZ, L, 2, 1, 0>;
     }
   }
 }
@@ -1028,7 +1065,7 @@ void launch_frame3_shape(int shape, int seg, const Prob* probs, State* states, c
   if (seg < F3_SEG) {
     auto go = [&](auto sg) {
       constexpr int SG = decltype(sg)::value;
-      k_frame3<T, TZ, L, F3_SEG_NWR, 2, 0, SG>
+      k_frame3<T, TZ, L, F3_SEG_NWR, 1, 0, SG>
           <<<nitems, 32 * F3_SEG_NWR, frame3_smem_bytes<T, TZ, L, F3_SEG_NWR, 0, SG>(), s>>>(
               probs, states, items, u_slot, f_slot, zin, zout, op_mu);
     };
@@ -1038,7 +1075,7 @@ void launch_frame3_shape(int shape, int seg, const Prob* probs, State* states, c
     return;
   }
   if constexpr (sizeof(T) == 8) {
-    k_frame3<T, TZ, L, 2, 2, 0><<<nitems, 64, frame3_smem_bytes<T, TZ, L, 2, 0>(), s>>>(
+    k_frame3<T, TZ, L, 2, 1, 0><<<nitems, 64, frame3_smem_bytes<T, TZ, L, 2, 0>(), s>>>(
         probs, states, items, u_slot, f_slot, zin, zout, op_mu);
   } else {
     switch (shape) {
@@ -1050,7 +1087,7 @@ void launch_frame3_shape(int shape, int seg, const Prob* probs, State* states, c
       F3_SHAPE_CASES(X)
 #undef X
       default:
-        k_frame3<T, TZ, L, 2, 2, 0><<<nitems, 64, frame3_smem_bytes<T, TZ, L, 2, 0>(), s>>>(
+        k_frame3<T, TZ, L, 2, 1, 0><<<nitems, 64, frame3_smem_bytes<T, TZ, L, 2, 0>(), s>>>(
             probs, states, items, u_slot, f_slot, zin, zout, op_mu);
     }
   }
@@ -1066,16 +1103,7 @@ void launch_frame(const Prob* probs, State* states, const int2* items, int nitem
   else if (levels == 2)
     launch_frame3_shape<T, TZ, 2>(shape, seg, probs, states, items, nitems, u_slot, f_slot, zin, zout, op_mu, s);
   else
-    launch_frame_levels<T, TZ>(probs, states, items, sec, levels, u_slot, f_slot, zin, zout, op_mu, s);
-}
-
-// the level kernels of one precision (below the top level, the top level)
-// and the low-pass chain kernel
-template <typename T, typename TZ>
-const void* const* lev_kernels() {
-  static const void* const k[] = {(const void*)k_frame_lev<T, TZ, false>,
-                                  (const void*)k_frame_lev<T, TZ, true>, (const void*)k_lowpass<T>};
-  return k;
+    launch_frame_levels<T, TZ>(probs, states, items, sec, levels, seg, u_slot, f_slot, zin, zout, op_mu, s);
 }
 
 template <typename T, typename TZ>
@@ -1089,17 +1117,11 @@ cudaError_t frame_set_smem() {
                              (int)frame3_smem<T, TZ, 2>(sh));
     if (e != cudaSuccess) return e;
   }
-  for (int k = 0; k < 2; ++k) {
-    const cudaError_t e = cudaFuncSetAttribute(lev_kernels<T, TZ>()[k],
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)lev_smem_bytes<T>());
-    if (e != cudaSuccess) return e;
-  }
   return cudaSuccess;
 }
 
 template <typename T, typename TZ, int L, int SG>
-const void* frame3_seg_kernel() { return (const void*)k_frame3<T, TZ, L, F3_SEG_NWR, 2, 0, SG>; }
+const void* frame3_seg_kernel() { return (const void*)k_frame3<T, TZ, L, F3_SEG_NWR, 1, 0, SG>; }
 
 bool is_frame_kernel(const void* func) {
   for (int sh = 0; sh < FRAME_SHAPES; ++sh) {
@@ -1117,10 +1139,13 @@ bool is_frame_kernel(const void* func) {
     if (f == func) return true;
   X(16) X(8) X(4)
 #undef X
-  for (int k = 0; k < 3; ++k)
-    if (func == lev_kernels<float, float>()[k] || func == lev_kernels<float, __nv_bfloat16>()[k] ||
-        func == lev_kernels<double, double>()[k])
-      return true;
+  for (int sg = 4; sg <= 32; sg *= 2)
+    for (const void* f : {lev_kernel<float, float, false>(sg), lev_kernel<float, float, true>(sg),
+                          lev_kernel<float, __nv_bfloat16, false>(sg),
+                          lev_kernel<float, __nv_bfloat16, true>(sg),
+                          lev_kernel<double, double, false>(sg), lev_kernel<double, double, true>(sg)})
+      if (f == func) return true;
+  if (func == (const void*)k_lowpass<float> || func == (const void*)k_lowpass<double>) return true;
   return false;
 }
 

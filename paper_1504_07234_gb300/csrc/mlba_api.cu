@@ -83,7 +83,7 @@ void add_frame_items(const Prob& pd, int i, int levels, int shape, int seg,
   if (levels <= 2) { add(fs[0], frame_tiles(pd.nf, levels, shape, seg)); return; }
   if (pd.use_adj && pd.bc != BC_RECT && pd.bc != BC_AR && !pd.balanced) add(fs[0], pd.nblk_vec);
   add(fs[1], lowpass_blocks(pd.nf));
-  for (int k = 0; k < levels; ++k) add(fs[2 + k], lev_tiles(pd.nf, levels - k));
+  for (int k = 0; k < levels; ++k) add(fs[2 + k], lev_tiles(pd.nf, levels - k, seg));
 }
 
 // parts of a step: a = residual and stop rule, then the preconditioner;
@@ -986,22 +986,25 @@ int time_frame_shape(mlba_batch* B, int shape, float* us) {
   return MLBA_OK;
 }
 
-// Rows a warp of the fused framelet sweep owns (L <= 2, built-in shape).  A
-// warp's sweep is one chain of rows (72 of them for 32 owned rows at L = 2),
-// so a launch with few warps lasts as long as that chain while most of the
-// chip idles; shorter segments give more and shorter chains at the price of
-// recomputed halo rows (2.25 swept rows per owned row at 32, 2.5 at 16, 3 at
-// 8, 4 at 4).  Halve while the doubled number of warps is resident at once:
-// about 20 FP32 warps per SM; in FP64 one warp per scheduler, because the
+// Rows a warp of a framelet sweep owns (L <= 2: the built-in shape).  A warp's
+// sweep is one chain of rows (72 of them for 32 owned rows at L = 2), so a
+// launch with few warps lasts as long as that chain while most of the chip
+// idles; shorter segments give more and shorter chains at the price of
+// recomputed halo rows (L = 2: 2.25 swept rows per owned row at 32, 2.5 at 16,
+// 3 at 8, 4 at 4).  Halve while the doubled number of warps is resident at
+// once: about 20 FP32 warps per SM; in FP64 one warp per scheduler, because the
 // FP64 pipe is already full with one.  Measured per launch, 32 rows against
 // the choice: 256^2 FP32 32 -> 10 us (4 rows), 72^2 FP64 L = 1 150 -> 27 us (4);
 // 1044^2 BF16 z 45 -> 39 us (16; 8: 44, 4: 54); the 64-problem batch stays at
-// 32 (16: +0.5 %, 8: +10 %).
+// 32 (16: +0.5 %, 8: +10 %).  L >= 3 starts at 16 in FP32 (a step at 4096^2:
+// as 32; at 2048^2: 470 us, 32: 486, 8: 527; at 1024^2: 194, 32: 218, 8: 209;
+// at 512^2 the choice is 4: 119, 32: 169).
 int frame_segment(const mlba_batch* B) {
   const double resident = B->dtype == MLBA_F64 ? 608.0 : 3040.0;
-  for (int seg = 32;; seg /= 2) {
+  for (int seg = (B->levels > 2 && B->dtype == MLBA_F32) ? 16 : 32;; seg /= 2) {
     double warps = 0.0;      // at half the segment
-    for (const HostProb& h : B->hp) warps += 2.0 * frame_tiles(h.pd.nf, B->levels, 0, seg / 2);
+    for (const HostProb& h : B->hp)
+      warps += B->levels > 2 ? lev_tiles(h.pd.nf, 1, seg / 2) : 2.0 * frame_tiles(h.pd.nf, B->levels, 0, seg / 2);
     if (seg == 4 || warps > resident) return seg;
   }
 }
@@ -1011,7 +1014,7 @@ int choose_frame_shape(mlba_batch* B, const mlba_opts& o) {
   B->frame_tuned = 0;
   // (a forced or measured shape, and the persistent schedule, keep 32 rows)
   B->frame_seg = 32;
-  if (B->levels <= 2 && o.frame_shape < 0 && !o.autotune && !o.persistent) B->frame_seg = frame_segment(B);
+  if (B->levels > 2 || (o.frame_shape < 0 && !o.autotune && !o.persistent)) B->frame_seg = frame_segment(B);
   const bool shaped = B->levels <= 2 && B->dtype != MLBA_F64;   // FP64: one shape
   if (!shaped) return MLBA_OK;
   if (o.frame_shape >= 0) {

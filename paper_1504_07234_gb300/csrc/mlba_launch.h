@@ -51,7 +51,6 @@ constexpr int VEC_THREADS = 256;
 constexpr int VEC_PER_THREAD = 8;
 constexpr int TR_CAP = 4096;          // complex values held by one transform CTA
 constexpr int FRAME_SHAPES = 8;      // tile shapes of the L <= 2 framelet kernel (k_frame.cu)
-constexpr int LV_NWR = 1;            // warps per CTA of the per-level framelet kernel (L >= 3; 1, 2, 4 measured)
 constexpr int LP_THREADS = 256, LP_PER = 4;   // low-pass chain kernel (L >= 3)
 constexpr int FRAME_SECTIONS = 2 + 4;         // fold, low-pass, up to four levels
 constexpr int SPEC_THREADS = 256;    // alpha_n solve (k_fft.cu)
@@ -98,7 +97,7 @@ void launch_frame(const Prob* probs, State* states, const int2* items, int nitem
                   int u_slot, int f_slot, const void* zin, void* zout, double op_mu, int levels,
                   int shape, int seg, cudaStream_t s);
 int frame_tiles(int nf, int levels, int shape, int seg);   // CTAs of the fused sweep for one problem (L <= 2)
-int lev_tiles(int nf, int lev);                   // CTAs of one level kernel (L >= 3)
+int lev_tiles(int nf, int lev, int seg);                   // CTAs of one level kernel (L >= 3)
 int lowpass_blocks(int nf);                       // CTAs of one low-pass launch (L >= 3)
 void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch);
 bool is_frame_kernel(const void* func);  // func is one of the framelet-update kernels

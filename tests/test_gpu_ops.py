@@ -262,3 +262,24 @@ def test_frame_segments_give_the_same_iterates(M, dtype, zs, levels):
         for a, c in zip(ref, out):
             np.testing.assert_array_equal(a, c)
     assert seen == {8, 16, 32, 64}, seen
+
+
+@pytest.mark.parametrize("dtype,zs", [("f32", "f32"), ("f32", "bf16"), ("f64", "f64")])
+@pytest.mark.parametrize("n", [31, 50])
+def test_level_segments_give_the_same_iterates(M, dtype, zs, n):
+    """L = 3: the rows a warp of the per-level sweep owns follow from the number
+    of warps of the batch (4, 8, 16, in FP64 also 32); every height computes the
+    same values, so batches of 1 to 260 copies end with the same bits."""
+    h = I.psf_gaussian(0.8, 5)
+    f = I.true_image(n + 4, n)
+    g, delta = I.observe(f, h, 0.02, n)
+    desc = dict(psf=h, g=g.astype(np.float64 if dtype == "f64" else np.float32), delta=delta,
+                bc="reflective", precond="none")
+    ref = None
+    for count in (1, 40, 90, 260):
+        b = M.Batch([desc] * count, dtype=dtype, z_store=zs, levels=3, stop=False, max_iter=3)
+        b.iterate(2)
+        out = b.result(count - 1)
+        b.close()
+        ref = out if ref is None else ref
+        np.testing.assert_array_equal(ref, out)
