@@ -298,8 +298,8 @@ struct F3Ring {
 template <typename T, typename TZ, int LEV, int L, int F3_PF, int RING>
 __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ cin, int cpitch,
                                          int cy0, int cx0, const TZ* __restrict__ zin,
-                                         TZ* __restrict__ zout, int ty0, int tx0, int seg_lo,
-                                         int seg_hi, T mu, T* __restrict__ f2s,
+                                         TZ* __restrict__ zout, bool fresh, int ty0, int tx0,
+                                         int seg_lo, int seg_hi, T mu, T* __restrict__ f2s,
                                          T* __restrict__ fout, F3Ring<TZ>& rg) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int D = 1 << (LEV - 1);
@@ -364,6 +364,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
   // the length): nothing moves.  Deeper queues are unrolled by the queue's
   // length and shift the rings by one row per step (phase 0 always).
   constexpr int RL = 2 * D + 1;
+  constexpr int RINGD = RING > 0 ? RING : 1;
   constexpr bool STATIC_RING = F3_PF == 1 && RING == 0;
   constexpr int UNR = STATIC_RING ? RL : F3_PF;
 #pragma unroll
@@ -383,6 +384,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     const int q = f3_refl(y, nf, &par) * nf + zc;
     zqo[k] = q;
     zqm[k] = par ? (int)0x80000000 : 0;
+    if (fresh) return;                 // z_in = 0: the queue keeps its zeros
     if constexpr (RING == 0) {
       const uint4* src = reinterpret_cast<const uint4*>(zin + (gbase + 8 * q));
 #pragma unroll
@@ -391,7 +393,12 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     if (TOP) zl[k] = zin[lbase + q];
   };
 #pragma unroll
-  for (int k = 0; k < F3_PF; ++k) zload(yc0 + k, k);
+  for (int k = 0; k < F3_PF; ++k) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) zq[RING > 0 ? 0 : k].v[v] = make_uint4(0, 0, 0, 0);
+    zl[k] = TZ(0.0f);
+    zload(yc0 + k, k);
+  }
   // ring: rows are issued RING ahead of the sweep.  Bulk path when the warp's
   // 32 columns lie inside the image (one contiguous run of 32 groups per row),
   // else per-lane 16-byte asynchronous copies of the mirrored columns.
@@ -428,7 +435,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     // the ring may hold rows an earlier level wrote with per-lane copies:
     // order those writes before this level's bulk copies
     if (bulk && lane == 0) fence_proxy_async();
-    for (int i = 0; i < RING; ++i) {
+    for (int i = 0; i < RING && !fresh; ++i) {
       if (i < nrows) issue(i);
       else if (!bulk) cp_commit();          // empty group: one group per row slot
     }
@@ -445,21 +452,21 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
   auto step = [&](int y, int k) {
     const int kq = STATIC_RING ? 0 : k, ph = STATIC_RING ? k : 0;
     const int ia = ph, ib = (ph + D) % RL, ic = (ph + 2 * D) % RL;   // rows y - D, y, y + D
-    if constexpr (RING > 0) {
+    if (RING > 0 && !fresh) {
       // this row's groups from the ring, then the slot is refilled with row y + RING
       const int i = y - yc0;
       if (bulk) {
         const int g = seq0 + i;
-        if (!rg.bad && !mbar_wait(rg.bar + g % RING, (unsigned)(g / RING) & 1u)) {
+        if (!rg.bad && !mbar_wait(rg.bar + g % RINGD, (unsigned)(g / RINGD) & 1u)) {
           rg.bad = true;
           first_bad = i;
         }
-        const uint4* sv = reinterpret_cast<const uint4*>(rg.buf + (g % RING) * 256 + 8 * lane);
+        const uint4* sv = reinterpret_cast<const uint4*>(rg.buf + (g % RINGD) * 256 + 8 * lane);
 #pragma unroll
         for (int v = 0; v < NV; ++v) zq[0].v[v] = sv[v];
       } else {
-        cp_wait<RING - 1>();
-        const uint4* sv = reinterpret_cast<const uint4*>(rg.buf + (i % RING) * 256 + 8 * lane);
+        cp_wait<RINGD - 1>();
+        const uint4* sv = reinterpret_cast<const uint4*>(rg.buf + (i % RINGD) * 256 + 8 * lane);
 #pragma unroll
         for (int v = 0; v < NV; ++v) zq[0].v[v] = sv[v];
       }
@@ -483,7 +490,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
       if (TOP) zout[lbase + zwo] = zlo;
     }
     if (y + F3_PF < yc1) zload(y + F3_PF, kq);
-    if constexpr (RING == 0) {
+    if (RING == 0 && !fresh) {
       // the z lines of a row further ahead into L2 (no registers held): the
       // register queue then finds them there
       const int ya = y + F3_PF + Z_L2_AHEAD;
@@ -530,14 +537,14 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     for (int k = 0; k < UNR; ++k)
       if (y + k < yc1) step(y + k, k);
   }
-  if constexpr (RING > 0) {
+  if (RING > 0 && !fresh) {
     if (bulk) {
       if (rg.bad) {
         // a wait gave up: wait (bounded) for the copies this level issued
         // from that row on, so none lands after the CTA has gone
         for (int i = first_bad; i < n_issued; ++i) {
           const int g = seq0 + i;
-          mbar_wait(rg.bar + g % RING, (unsigned)(g / RING) & 1u);
+          mbar_wait(rg.bar + g % RINGD, (unsigned)(g / RINGD) & 1u);
         }
       }
       rg.seq = seq0 + nrows;
@@ -546,6 +553,13 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     }
     __syncwarp();
   }
+}
+
+// No z to read: the first update after a reset (z^0 = 0), and every step of the
+// balanced formulation.  (Storing the zeros cost a memset of all of z per
+// reset and their read in the first step: 4096^2, L = 2: 181 + 190 us.)
+__device__ __forceinline__ bool frame_fresh(const Prob& pd, const State& st, const void* zin_op) {
+  return !zin_op && (pd.balanced || (st.zfresh && st.iter == 1));
 }
 
 // One framelet tile on the thread group `blk` of 32 F3_NWR threads with its
@@ -571,9 +585,10 @@ __device__ __forceinline__ void frame3_body(const int2 item, const Prob* __restr
     zin = static_cast<const TZ*>(zin_op);
     zout = static_cast<TZ*>(zout_op);
   } else {
-    zin = static_cast<const TZ*>(pd.z0 ? pd.z0 : pd.z[(st.iter - 1) & 1]);
+    zin = static_cast<const TZ*>(pd.z[(st.iter - 1) & 1]);
     zout = static_cast<TZ*>(pd.z[st.iter & 1]);
   }
+  const bool fresh = frame_fresh(pd, st, zin_op);
   T* su = reinterpret_cast<T*>(smraw);            // u on rows ty0 - C0.., cols tx0 - C0..
   T* sf2 = su + Gm::UW * Gm::UH;                  // level-2 part of f on the tile (L = 2)
   constexpr int C0 = Gm::C0;
@@ -644,12 +659,12 @@ __device__ __forceinline__ void frame3_body(const int2 item, const Prob* __restr
     __syncwarp();
   }
   if (L == 2) {
-    f3_level<T, TZ, 2, L, F3_PF, RING>(pd, su, Gm::UW, ty0 - C0, tx0 - C0, zin, zout, ty0, tx0,
+    f3_level<T, TZ, 2, L, F3_PF, RING>(pd, su, Gm::UW, ty0 - C0, tx0 - C0, zin, zout, fresh, ty0, tx0,
                                        seg_lo, seg_hi, mu, sf2, f, rg);
     __syncwarp();
   }
   if (!rg.bad)
-    f3_level<T, TZ, 1, L, F3_PF, RING>(pd, su, Gm::UW, ty0 - C0, tx0 - C0, zin, zout, ty0, tx0,
+    f3_level<T, TZ, 1, L, F3_PF, RING>(pd, su, Gm::UW, ty0 - C0, tx0 - C0, zin, zout, fresh, ty0, tx0,
                                        seg_lo, seg_hi, mu, sf2, f, rg);
   if (rg.bad && (tid & 31) == 0) {
     // a bounded wait gave up: the problem stops with a timeout status
@@ -817,9 +832,10 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
     zin = static_cast<const TZ*>(zin_op);
     zout = static_cast<TZ*>(zout_op);
   } else {
-    zin = static_cast<const TZ*>(pd.z0 ? pd.z0 : pd.z[(st.iter - 1) & 1]);
+    zin = static_cast<const TZ*>(pd.z[(st.iter - 1) & 1]);
     zout = static_cast<TZ*>(pd.z[st.iter & 1]);
   }
+  const bool fresh = frame_fresh(pd, st, zin_op);
   // position of the local coordinate m of a sub-lattice in the level's order
   // (mirrored into the image first)
   auto cpos = [&](int m, int off, bool* par) { return P.pos(f3_refl(off + dp * m, nf, par)); };
@@ -869,14 +885,20 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
     const int q = cpos(y, sb, &par) * nf + zc;
     zqo[k] = q;
     zqm[k] = par ? (int)0x80000000 : 0;
+    if (!TOP) sq[k] = sin[q];                // s_l at (y, mx), mirrored like z
+    if (fresh) return;                       // z_in = 0: the queue keeps its zeros
     const uint4* src = reinterpret_cast<const uint4*>(zin + (gbase + 8 * q));
 #pragma unroll
     for (int v = 0; v < NV; ++v) zq[k].v[v] = src[v];
     if (TOP) zl[k] = zin[lbase + q];
-    else sq[k] = sin[q];                     // s_l at (y, mx), mirrored like z
   };
 #pragma unroll
-  for (int k = 0; k < PF; ++k) zload(yc0 + k, k);
+  for (int k = 0; k < PF; ++k) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) zq[k].v[v] = make_uint4(0, 0, 0, 0);
+    zl[k] = TZ(0.0f);
+    zload(yc0 + k, k);
+  }
   cp_wait<0>();
   __syncwarp();
   auto hrow = [&](int y, T (&h)[3]) {
@@ -916,9 +938,11 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
       if (ya < yc1) {
         bool par;
         const int qa = cpos(ya, sb, &par) * nf + zc;
-        prefetch_l2(zin + (gbase + 8 * qa));
-        if (TOP) prefetch_l2(zin + (lbase + qa));
-        else prefetch_l2(sin + qa);
+        if (!fresh) {
+          prefetch_l2(zin + (gbase + 8 * qa));
+          if (TOP) prefetch_l2(zin + (lbase + qa));
+        }
+        if (!TOP) prefetch_l2(sin + qa);
       }
     }
     // row y - 1 is complete

@@ -102,7 +102,7 @@ struct mlba_batch {
   State* d_opstates = nullptr;
   unsigned char* arena = nullptr;
   size_t arena_bytes = 0;
-  size_t zero_bytes = 0;        // [arena, arena + zero_bytes): every problem's f and z^0
+  size_t zero_bytes = 0;        // [arena, arena + zero_bytes): every problem's f
   // item lists
   ItemList blur, corr, reblur, corr_kry, blur_kry, rows_spec, cols_stat, cols_ns, spec, rows_kry,
       cols_kry, vec_kry, vec_kry_bc, frame, corr_all, rows_all, cols_all, spec_all, vec_all,
@@ -119,6 +119,7 @@ struct mlba_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool has_data = false;
+  bool z0_given = false;        // a loaded state brought its own z at iteration 0
   int any_krylov = 0, any_spec = 0, any_ns = 0, any_stat = 0, any_ar = 0;
   // Two-group schedule (batches of two or more problems): group 1 runs half a
   // step behind group 0 on a second stream, so that one group's framelet
@@ -280,6 +281,7 @@ State initial_state(const Prob& pd) {
   s.stop_iter = -1;
   s.alpha_n = pd.alpha;
   s.nb = 0.0;
+  s.zfresh = 1;
   return s;
 }
 
@@ -1030,8 +1032,7 @@ int choose_frame_shape(mlba_batch* B, const mlba_opts& o) {
     B->frame_shape = sh; B->frame_tuned = 2; B->frame_us = us;
     return MLBA_OK;
   }
-  // the first step reads z^0 = 0 from z[0] and writes z[1]; the timed
-  // launches read z[1] and write z[0], which the reset after create clears
+  // (the timed launches, at iteration 0, read z[1] and write z[0])
   for (const HostProb& hp : B->hp)
     CK(cudaMemsetAsync(hp.pd.z[1], 0, (size_t)hp.pd.nbands * hp.pd.nf * hp.pd.nf * zsize(B->z_store),
                        B->stream));
@@ -1276,7 +1277,6 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
         (pd.ns ? nspec : 1) * ts,              // 4-NS weighted power
         (pd.levels >= 3 ? (size_t)(pd.levels - 1) * nf2 : 1) * ts,   // low-pass chain (L >= 3)
         (pd.levels >= 3 ? (size_t)(pd.levels - 1) * nf2 : 1) * ts,   // synthesis partials
-        pd.balanced ? (size_t)pd.nbands * nf2 * zs : zs,             // zeros (balanced z_in)
         spec ? (size_t)pd.nfft * 2 * ts : ts,  // tw
         spec ? (size_t)pd.n * 2 * ts : ts,     // dtw
         (size_t)pd.nruns * 16, 2 * (size_t)pd.nrw * ts,   // tap runs and weights (both orders)
@@ -1285,19 +1285,18 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
         (size_t)(pd.max_iter + 2) * 8, (size_t)(pd.max_iter + 2) * 8, (size_t)(pd.max_iter + 2) * 4};
     szs[i] = sz;
   }
-  // f and z^0 of every problem come first, side by side, so that a reset
-  // clears all of them with one memset of [arena, arena + zero_bytes); the
-  // other buffers follow, problem by problem
-  const size_t kF = SL_F, kZ0 = NSLOT;
+  // f of every problem comes first, side by side, so that a reset clears all
+  // of them with one memset of [arena, arena + zero_bytes) (z^0 = 0 is never
+  // stored, State::zfresh); the other buffers follow, problem by problem
+  const size_t kF = SL_F;
   for (int i = 0; i < count; ++i) {
     offs[i].assign(szs[i].size(), 0);
     offs[i][kF] = total; total += al(szs[i][kF]);
-    offs[i][kZ0] = total; total += al(szs[i][kZ0]);
   }
   B->zero_bytes = total;
   for (int i = 0; i < count; ++i)
     for (size_t k = 0; k < szs[i].size(); ++k)
-      if (k != kF && k != kZ0) { offs[i][k] = total; total += al(szs[i][k]); }
+      if (k != kF) { offs[i][k] = total; total += al(szs[i][k]); }
   // convolution entries: X, Y, the spectrum work array, the two spectra, a
   // zero |lambda|^2 and the twiddles, shared by the pair of one problem (the
   // forward pass and the adjoint pass of a step never overlap)
@@ -1333,9 +1332,6 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
     pd.pw = base + of[k++];
     pd.lp = base + of[k++];
     pd.sy = base + of[k++];
-    pd.z0 = base + of[k++];
-    if (pd.balanced) CK(cudaMemset(pd.z0, 0, (size_t)pd.nbands * pd.nf * pd.nf * zs));
-    else pd.z0 = nullptr;
     pd.tw = base + of[k++];
     pd.dtw = base + of[k++];
     pd.tap_runs = reinterpret_cast<int4*>(base + of[k++]);
@@ -1548,7 +1544,8 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
 
 int reset_batch(mlba_batch* B) {
   std::vector<State> st_h(B->hp.size());
-  // f and z^0 of every problem: one region at the start of the arena
+  B->z0_given = false;
+  // f of every problem: one region at the start of the arena
   CK(cudaMemsetAsync(B->arena, 0, B->zero_bytes, B->stream));
   for (size_t i = 0; i < B->hp.size(); ++i) st_h[i] = initial_state(B->hp[i].pd);
   CK(cudaMemcpyAsync(B->d_states, st_h.data(), st_h.size() * sizeof(State), cudaMemcpyHostToDevice,
@@ -1958,8 +1955,13 @@ int mlba_get_z(mlba_ctx* c, void* z_out, int on_device) {
   const Prob& pd = B->hp[0].pd;
   const size_t es = zsize(B->z_store), plane = (size_t)pd.nf * pd.nf;
   const size_t zbytes = (size_t)pd.nbands * plane * es;
-  if (!z_grouped(pd.levels)) return copy_out(B, z_out, pd.z[s.iter & 1], zbytes, on_device);
   if (!z_out) return MLBA_E_INVAL;
+  if (s.iter == 0 && !c->b->z0_given) {           // z^0 = 0 is not stored
+    if (!on_device) std::memset(z_out, 0, zbytes);
+    else CK(cudaMemsetAsync(z_out, 0, zbytes, B->stream));
+    return MLBA_OK;
+  }
+  if (!z_grouped(pd.levels)) return copy_out(B, z_out, pd.z[s.iter & 1], zbytes, on_device);
   // the library keeps z in its internal order (z_index); the caller gets band-major planes
   if (on_device) {
     launch_z_layout(z_out, pd.z[s.iter & 1], pd.levels, pd.nf, (int)es, 0, B->stream);
@@ -2104,6 +2106,8 @@ int mlba_set_state(mlba_ctx* c, const void* blob, size_t bytes) {
   st.iter = h.iter; st.stopped = h.stopped; st.stop_iter = h.stop_iter; st.status = h.status;
   st.nres = h.nres; st.beta_last = h.beta_last;
   st.resnorm = h.resnorm; st.alpha_n = h.alpha_n; st.nb = h.nb; st.qn = h.qn;
+  st.zfresh = 0;
+  B->z0_given = true;
   CK(cudaMemcpy(&B->d_states[0], &st, sizeof(State), cudaMemcpyHostToDevice));
   return MLBA_OK;
 }

@@ -43,7 +43,7 @@ struct Prob {
   int fc;            // problem: 1 = A and A^T by FFT convolution (the entries below)
   int fc_sh[2];      // problem: table indices of its forward / adjoint convolution entries
   int balanced;      // 1: the balanced formulation, x = S_mu(W (f + u)): u is replaced by
-                     // f + u before the framelet step and z_in by zeros (z0)
+                     // f + u before the framelet step, which reads no z
   int bc, precond, transform, levels, nbands;
   int ns;            // nonstationary alpha (4-NS)
   int use_adj;       // 1: u = A^T t ; 0: u = t (Algorithm 4 forms)
@@ -66,7 +66,6 @@ struct Prob {
   double mu, alpha, gamma, delta, q, rho, tau, pcg_tol;
   void* buf[NSLOT];
   void* z[2];        // ping-pong Bregman variable
-  void* z0;          // balanced formulation: zeros read in place of z_in
   void* w;           // |lambda|^2 in T precision, column-blocked like S
   void* pw;          // 4-NS: weighted power |orthonormal coefficient of r|^2 per
                      // spectral value, T, blocked like S (0 on padding); written by
@@ -98,6 +97,7 @@ struct State {
   int nphase;        // 4-NS: 0 = bracketing pass pending, 1 = Newton
   int pdone, psteps; // PCG
   int beta_last;
+  int zfresh;        // z^0 = 0 is not stored: the update of iteration 1 reads no z
   double resnorm, alpha_n, qn;
   double nb, nb_lo, nb_hi;     // Newton on log(alpha)
   double ea;                   // exp(nb), set with nb (before the rectangular floor)

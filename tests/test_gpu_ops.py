@@ -283,3 +283,35 @@ def test_level_segments_give_the_same_iterates(M, dtype, zs, n):
         b.close()
         ref = out if ref is None else ref
         np.testing.assert_array_equal(ref, out)
+
+
+@pytest.mark.parametrize("dtype,zs,levels,shape", [("f32", "f32", 2, -1), ("f32", "bf16", 1, 5), ("f32", "f32", 2, 6),
+                                                   ("f32", "f32", 3, -1), ("f64", "f64", 2, -1), ("f64", "f64", 4, -1)])
+@pytest.mark.parametrize("formulation", ["synthesis", "balanced"])
+def test_restart_reads_no_old_z(M, dtype, zs, levels, shape, formulation):
+    """z^0 = 0 is not stored: after a reset (set_data) over used buffers, get_z
+    gives zeros, the iterates are those of a new context bit for bit, and a state
+    saved at iteration 0 resumes to the same iterates."""
+    h = I.psf_gaussian(0.8, 5)
+    f = I.true_image(44, 5)
+    g, delta = I.observe(f, h, 0.02, 5)
+    kw = dict(dtype=dtype, z_store=zs, levels=levels, max_iter=9, stop=False, frame_shape=shape,
+              formulation=formulation)
+    a, b = (M.Context(h, g.shape[0], "reflective", "bccb", alpha=0.3, **kw) for _ in range(2))
+    a.set_data(g, delta)
+    a.iterate(5)
+    a.set_data(g, delta)
+    assert not a.get_z().any()
+    blob = a.get_state()
+    a.iterate(3)
+    b.set_data(g, delta)
+    b.iterate(3)
+    ref = b.result()
+    np.testing.assert_array_equal(a.result(), ref)
+    assert np.array_equal(a.get_z().float().cpu().numpy(), b.get_z().float().cpu().numpy())
+    b.set_data(g, delta)
+    b.set_state(blob)
+    b.iterate(3)
+    np.testing.assert_array_equal(b.result(), ref)
+    a.close()
+    b.close()
