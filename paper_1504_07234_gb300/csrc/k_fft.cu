@@ -1776,20 +1776,20 @@ void launch_spectrum_setup(int transform, int n, int p, int half, int cb, const 
   k_spectrum<<<blocks, 256, 0, s>>>(transform, n, p, half, cb, q_dev, tab_dev, lam, sigT, is_double);
 }
 template <typename T>
-cudaError_t fft_set_smem(size_t bytes) {
-  cudaError_t e = cudaFuncSetAttribute(k_rows_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+cudaError_t fft_set_smem() {
+  cudaError_t e = cudaFuncSetAttribute(k_rows_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
   if (e != cudaSuccess) return e;
   for (const void* f : {(const void*)k_cols<T, COL_FUSED>, (const void*)k_cols<T, COL_FWD>,
                         (const void*)k_cols<T, COL_NS_INV>, (const void*)k_cols<T, COL_OP>}) {
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
   }
   for (const void* f : {(const void*)k_ar_rows<T, false>, (const void*)k_ar_rows<T, true>,
                         (const void*)k_ar_cols<T, COL_FUSED>, (const void*)k_ar_cols<T, COL_OP>}) {
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
   }
-  return cudaFuncSetAttribute(k_rows_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return cudaFuncSetAttribute(k_rows_inv<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
 }
 
 #define INST(T)                                                                                   \
@@ -1799,7 +1799,7 @@ cudaError_t fft_set_smem(size_t bytes) {
   template void launch_spec<T>(const Prob*, State*, const int2*, int, int, cudaStream_t);         \
   template void launch_ar_rows<T>(const Prob*, State*, const int2*, int, int, int, int, size_t, cudaStream_t); \
   template void launch_ar_cols<T>(const Prob*, State*, const int2*, int, int, int, double, int, size_t, cudaStream_t); \
-  template cudaError_t fft_set_smem<T>(size_t);
+  template cudaError_t fft_set_smem<T>();
 INST(float)
 INST(double)
 #undef INST

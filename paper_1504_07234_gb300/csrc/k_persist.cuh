@@ -15,6 +15,7 @@
 // FP32 z, k_persist_bf16.cu for bf16 z (two units compiled in parallel).
 #pragma once
 #define MLBA_BODIES_ONLY
+#include <type_traits>
 #include "k_stencil.cu"
 #include "k_fft.cu"
 #include "k_frame.cu"
@@ -108,12 +109,20 @@ k_persist(const Prob* __restrict__ probs, State* __restrict__ states, int nprob,
             if (i >= cnt) continue;
             unsigned char* sm = smraw + (size_t)sub2 * stencil_slot;
             const BlkSub<STENCIL_THREADS> b{1 + sub2};
-            if (sg.kind == PS_RESID)
-              stencil_body<T, ST_FWD_RESID>(it[i], probs, states, SL_F, SL_R, SL_G, 0, sm, red[sub2], &flag[sub2], b);
-            else if (sg.kind == PS_CORR)
-              stencil_body<T, ST_CORR>(it[i], probs, states, -1, SL_V, SL_V, 0, sm, red[sub2], &flag[sub2], b);
-            else
-              stencil_body<T, ST_REBLUR>(it[i], probs, states, -1, -1, SL_U, 0, sm, red[sub2], &flag[sub2], b);
+            // (the rows per thread of the graph schedule: the norm's partial
+            // sums then add up in the same order)
+            auto tile = [&](auto rc) {
+              constexpr int R = decltype(rc)::value;
+              if (sg.kind == PS_RESID)
+                stencil_body<T, ST_FWD_RESID, R>(it[i], probs, states, SL_F, SL_R, SL_G, 0, sm, red[sub2], &flag[sub2], b);
+              else if (sg.kind == PS_CORR)
+                stencil_body<T, ST_CORR, R>(it[i], probs, states, -1, SL_V, SL_V, 0, sm, red[sub2], &flag[sub2], b);
+              else
+                stencil_body<T, ST_REBLUR, R>(it[i], probs, states, -1, -1, SL_U, 0, sm, red[sub2], &flag[sub2], b);
+            };
+            if (sg.rows == 2) tile(std::integral_constant<int, 2>{});
+            else if (sg.rows == 4) tile(std::integral_constant<int, 4>{});
+            else tile(std::integral_constant<int, 8>{});
             b.sync();   // the next item's tile loads overwrite this one's shared memory
           }
           break;

@@ -53,66 +53,6 @@ __device__ __forceinline__ bool skip(const State& st, int pcg) {
   return st.stopped || (pcg && st.pdone);
 }
 
-// The last R (1..7) taps t .. t + R - 1 of a run from the aligned window
-// (slot j holds v[t + j]): v[t + 8 .. t + R + 6] go to R - 1 more registers and
-// every index is static, so no value moves and no work is predicated off.
-template <int R, typename V, typename W, typename LD, typename FMA>
-__device__ __forceinline__ void window_tail(V (&acc)[8], const V (&win)[8], const W* __restrict__ w,
-                                            int t, LD ld, FMA fma2) {
-  V ext[R > 1 ? R - 1 : 1];
-#pragma unroll
-  for (int i = 0; i < R - 1; ++i) ext[i] = ld(t + 8 + i);
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const W wt = w[t + u];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int sidx = j + u;
-      acc[j] = fma2(sidx < 8 ? win[sidx] : ext[sidx - 8 < R - 1 ? sidx - 8 : 0], wt, acc[j]);
-    }
-  }
-}
-template <typename V, typename W, typename LD, typename FMA>
-__device__ __forceinline__ void window_tails(V (&acc)[8], const V (&win)[8], const W* __restrict__ w,
-                                             int t, int r, LD ld, FMA fma2) {
-  switch (r) {
-    case 1: window_tail<1>(acc, win, w, t, ld, fma2); break;
-    case 2: window_tail<2>(acc, win, w, t, ld, fma2); break;
-    case 3: window_tail<3>(acc, win, w, t, ld, fma2); break;
-    case 4: window_tail<4>(acc, win, w, t, ld, fma2); break;
-    case 5: window_tail<5>(acc, win, w, t, ld, fma2); break;
-    case 6: window_tail<6>(acc, win, w, t, ld, fma2); break;
-    case 7: window_tail<7>(acc, win, w, t, ld, fma2); break;
-    default: break;
-  }
-}
-
-// acc[j] += sum_t w[t] v[t + j] over a run of len taps, v[i] = base[i * stride]:
-// an 8-value window of v.  Whole groups of 8 taps keep the window as a ring
-// (slot (i & 7) holds v[i]) so every register index is static and no value
-// moves; after them the ring is aligned again (slot j holds v[t + j]) and the
-// last len % 8 taps go through window_tail.
-template <typename T>
-__device__ __forceinline__ void window_run(T (&acc)[8], const T* __restrict__ base, int stride,
-                                           const T* __restrict__ w, int len) {
-  T win[8];
-#pragma unroll
-  for (int j = 0; j < 8; ++j) win[j] = base[j * stride];
-  int t = 0;
-  for (; t + 8 <= len; t += 8) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const T wt = w[t + u];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] += wt * win[(j + u) & 7];
-      // slot u held v[t + u], needed by no later tap: refill with v[t + u + 8]
-      if (t + u + 1 < len) win[u] = base[(t + u + 8) * stride];
-    }
-  }
-  window_tails(acc, win, w, t, len - t, [&](int i) { return base[i * stride]; },
-               [](T v, T wt, T a) { return a + wt * v; });
-}
-
 // asynchronous global -> shared copy of a B-byte chunk (B = 8 or 16, both
 // addresses B-aligned) of which the first nbytes come from global memory and
 // the rest are zero-filled
@@ -150,90 +90,135 @@ __device__ __forceinline__ int bc_map_near(int e, int n, int bc) {
   return bc_map(e, n, bc);
 }
 
-// Pairs of FP32 values: the paired FP32 instructions of sm_100+ do two
-// multiply-adds in one; FP64 falls back to two scalar ones.
+// Pairs of values: the paired FP32 instructions of sm_100+ do two
+// multiply-adds in one (the weight is kept twice in shared memory, so a pair
+// is one load); FP64 falls back to two scalar ones.
 template <typename T> struct Pair;
 template <> struct Pair<float> {
   using type = float2;
-  static __device__ __forceinline__ float2 fma(float2 a, float w, float2 acc) {
-    return __ffma2_rn(a, make_float2(w, w), acc);
-  }
+  using weight = float2;
+  static __device__ __forceinline__ float2 w(float v) { return make_float2(v, v); }
+  static __device__ __forceinline__ float2 fma(float2 a, float2 w, float2 acc) { return __ffma2_rn(a, w, acc); }
 };
 template <> struct Pair<double> {
   using type = double2;
+  using weight = double;
+  static __device__ __forceinline__ double w(double v) { return v; }
   static __device__ __forceinline__ double2 fma(double2 a, double w, double2 acc) {
     return make_double2(::fma(a.x, w, acc.x), ::fma(a.y, w, acc.y));
   }
 };
 
-// acc[j] += sum_t w[t] v[t + j] over a run of len taps for pairs of
-// neighbouring columns, v[i] = (base[i stride], base[i stride + 1]) (one
-// 8-byte or 16-byte load when `aligned`, else two): the same ring / shifting
-// window as window_run, on pairs.
-template <typename T>
-__device__ __forceinline__ void window_run2(typename Pair<T>::type (&acc)[8], const T* __restrict__ base,
-                                            int stride, const T* __restrict__ w, int len,
-                                            bool aligned) {
-  using T2 = typename Pair<T>::type;
-  auto ld = [&](int i) -> T2 {
-    const T* q = base + i * stride;
-    if (aligned) return *reinterpret_cast<const T2*>(q);
-    T2 v; v.x = q[0]; v.y = q[1]; return v;
-  };
-  T2 win[8];
+// B taps t .. t + B - 1 of a run for R outputs: acc[j] += w[t + u] v[t + u + j].
+// The window is a ring: slot (ROT + j) % R holds v[t + j] on entry, slot
+// (ROT + B + j) % R holds v[t + B + j] on exit, so every register index is static
+// and no value moves (copying the window cost 400 of 2700 instructions per warp
+// at 31 taps).  The value past the last tap's reach is not loaded.
+template <typename T, int R, int B, int ROT, typename LD>
+__device__ __forceinline__ void window_taps(typename Pair<T>::type (&acc)[R], typename Pair<T>::type (&win)[R],
+                                            const typename Pair<T>::weight* __restrict__ w, int t, int len,
+                                            LD ld) {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) win[j] = ld(j);
-  int t = 0;
-  for (; t + 8 <= len; t += 8) {
+  for (int u = 0; u < B; ++u) {
+    const typename Pair<T>::weight wt = w[t + u];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const T wt = w[t + u];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = Pair<T>::fma(win[(j + u) & 7], wt, acc[j]);
-      if (t + u + 1 < len) win[u] = ld(t + u + 8);
-    }
+    for (int j = 0; j < R; ++j) acc[j] = Pair<T>::fma(win[(ROT + u + j) % R], wt, acc[j]);
+    if (u + 1 < B || t + B < len) win[(ROT + u) % R] = ld(t + u + R);
   }
-  window_tails(acc, win, w, t, len - t, ld, [](T2 v, T wt, T2 a) { return Pair<T>::fma(v, wt, a); });
+}
+template <typename T, int R, int ROT, typename LD>
+__device__ __forceinline__ void window_tail3(typename Pair<T>::type (&acc)[R], typename Pair<T>::type (&win)[R],
+                                             const typename Pair<T>::weight* __restrict__ w, int t, int len,
+                                             LD ld) {
+  if (t + 2 <= len) {
+    window_taps<T, R, 2, ROT>(acc, win, w, t, len, ld);
+    if (t + 2 < len) window_taps<T, R, 1, ROT + 2>(acc, win, w, t + 2, len, ld);
+  } else if (t < len) {
+    window_taps<T, R, 1, ROT>(acc, win, w, t, len, ld);
+  }
 }
 
-// Stencil tile geometry: 64 x 32 outputs per CTA of 128 threads; a thread
-// owns two neighbouring columns over 8 rows (16 outputs in registers).  The
-// input tile (32 + p - 1) x (64 + p - 1) lives in shared memory with an even
-// row pitch (pairs of columns are one 8-byte word when the column is even).
-constexpr int ST_TX = 64, ST_TY = 32;
+// acc[j] += sum_t w[t] v[t + j], j < R, over a run of len taps, v[i] = ld(i)
+// pairs of values: blocks of 8 (R = 8) or 4 taps, then the rest by halves.
+template <typename T, int R, typename LD>
+__device__ __forceinline__ void window_run(typename Pair<T>::type (&acc)[R],
+                                           const typename Pair<T>::weight* __restrict__ w, int len, LD ld) {
+  constexpr int B0 = R >= 8 ? 8 : 4;       // a multiple of R: the ring is aligned after a block
+  typename Pair<T>::type win[R];
+#pragma unroll
+  for (int j = 0; j < R; ++j) win[j] = ld(j);
+  int t = 0;
+#pragma unroll 1
+  for (; t + B0 <= len; t += B0) window_taps<T, R, B0, 0>(acc, win, w, t, len, ld);
+  if constexpr (B0 == 8) {
+    if (t + 4 <= len) {
+      window_taps<T, R, 4, 0>(acc, win, w, t, len, ld);
+      window_tail3<T, R, 4>(acc, win, w, t + 4, len, ld);
+      return;
+    }
+  }
+  window_tail3<T, R, 0>(acc, win, w, t, len, ld);
+}
+
+// Stencil tile geometry: 64 x 4 R outputs per CTA of 128 threads; a thread
+// owns two neighbouring columns over R rows.  The input tile (4 R + p - 1) x
+// (64 + p - 1) lives in shared memory with an even row pitch (pairs of columns
+// are one 8-byte word when the column is even).  R = 8 reuses each loaded value
+// most; small images take fewer rows per thread (the host's stencil_rows).
+constexpr int ST_TX = 64;
 // row pitch of the input tile: a multiple of 16 bytes with room for the
 // shift (< 16 bytes) that aligns a row's source to 16 bytes
 __host__ __device__ constexpr int st_pitch(int RX, int elem) {
   return (RX + 16 / elem - 1 + 16 / elem - 1) / (16 / elem) * (16 / elem);
 }
-constexpr int ST_TP = ST_TX + 2;      // row-pass tile pitch (rank-one PSF, p > 33)
-constexpr int ST_ROW_ITEMS = 4;       // row-pass items a thread holds in registers (8 RY <= 4 x 128)
+// rank-one PSF: pitch in pairs of the column-pass result (row pairs x columns),
+// odd so that the lanes of the row pass (one row pair each) hit different banks
+__host__ __device__ constexpr int st_tpitch(int RX, int elem) { return (st_pitch(RX, elem) + 2) | 1; }
+// shared memory of a tile: weights, runs (general PSF), the source rows
+// and columns of the tile, input tile (which the
+// column-pass result and the output tile of a rank-one PSF overwrite)
+__host__ __device__ constexpr size_t st_smem(int R, int p, int sep, int nrw, int nruns, int elem) {
+  const int RY = 4 * R + p - 1, RX = ST_TX + p - 1;
+  const int nw = sep ? 2 * p : nrw, we = elem == 4 ? 2 : 1;
+  const size_t in = (size_t)RY * st_pitch(RX, elem), tmp = sep ? (size_t)4 * R * st_tpitch(RX, elem) : 0;
+  return (((size_t)nw * we + 3) / 4 * 4 + (in > tmp ? in : tmp)) * elem + (sep ? 0 : (size_t)nruns * 16) +
+         (size_t)((RY + RX + 3) / 4 * 4) * 4;
+}
 
 #ifndef MLBA_BODIES_ONLY
-int stencil_tiles(int outN) { return ((outN + ST_TX - 1) / ST_TX) * ((outN + ST_TY - 1) / ST_TY); }
+int stencil_tiles(int outN, int R) { return ((outN + ST_TX - 1) / ST_TX) * ((outN + 4 * R - 1) / (4 * R)); }
+size_t stencil_smem(int R, int p, int sep, int nrw, int nruns, int elem) {
+  return st_smem(R, p, sep, nrw, nruns, elem);
+}
 #endif
 
 // Blur A (Eq. 2 with the Table 1 boundary conditions, or the valid part for
 // rectangular A) and the full correlation that A^T is built from, as
 // register-window stencils:
 //  - general PSF: the taps are grouped by PSF column b into dense runs
-//    [lo_b, hi_b] of rows; a thread slides an 8-row window of two input
+//    [lo_b, hi_b] of rows; a thread slides an R-row window of two input
 //    columns down the run, so each tap costs one (or two) shared loads, one
-//    broadcast weight and 8 paired FMAs for 16 outputs;
-//  - rank-one PSF (h = hy hx^T): a horizontal pass with an 8-value window along
-//    the rows into shared memory, then a vertical pass with paired windows.
+//    broadcast weight and R paired FMAs for 2 R outputs;
+//  - rank-one PSF (h = hy hx^T): a column pass first (pairs of columns, R-row
+//    windows, over the tile's 64 + p - 1 columns), kept in registers and written
+//    over the input tile as pairs of rows, then the row pass on the row pairs
+//    (R-column windows): both passes are paired FMAs on conflict-free loads.
+//    The row-first order did 32 + p - 1 rows for 32 with scalar FMAs from
+//    four-way conflicting loads.
 // Forward (A f)(y, x) = sum_{a,b} H[a][b] f_ext(y + c - a, x + c - b); the
 // correlation (ne x ne) is sum_{a,b} H[a][b] t(y - 2c + a, x - 2c + b).
 // (FP32: 8 CTAs per SM, 64 registers; the tile of the largest PSF of a batch
 // decides how many fit in shared memory)
 // One stencil item (tile) on the thread group `blk` of STENCIL_THREADS threads,
 // with its shared memory at smraw, 32 doubles of reduction space and one int.
-template <typename T, int MODE, typename BLK>
+template <typename T, int MODE, int R, typename BLK>
 __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __restrict__ probs,
                                              State* __restrict__ states, int src_slot, int dst_slot,
                                              int aux_slot, int pcg, unsigned char* smraw,
                                              double* red, int* flag, BLK blk) {
   using T2 = typename Pair<T>::type;
+  using TW = typename Pair<T>::weight;
+  constexpr int ST_TY = 4 * R;
   const int tid = blk.tid();
   const Prob& pd = probs[item.x];
   State& st = states[item.x];
@@ -256,10 +241,11 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   // shared memory: weights, column runs (general PSF), input tile, row-pass
   // tile (rank-one PSF)
   const int nw = sep ? 2 * p : pd.nrw;
-  T* s_w = reinterpret_cast<T*>(smraw);
-  int4* s_runs = reinterpret_cast<int4*>(s_w + ((nw + 3) & ~3));
-  T* s_in = reinterpret_cast<T*>(s_runs + (sep ? 0 : pd.nruns));
-  T* s_tmp = s_in + RY * RP;
+  TW* s_w = reinterpret_cast<TW*>(smraw);
+  constexpr int WE = (int)(sizeof(TW) / sizeof(T));
+  int4* s_runs = reinterpret_cast<int4*>(reinterpret_cast<T*>(smraw) + ((nw * WE + 3) & ~3));
+  int* s_map = reinterpret_cast<int*>(s_runs + (sep ? 0 : pd.nruns));     // RY + RX entries
+  T* s_in = reinterpret_cast<T*>(s_map + ((RY + RX + 3) & ~3));
 
   // src_slot < 0: the per-problem default operand (t, or r for P = I, in the
   // correlation; A^T p for the PCG product: V for rectangular A, U otherwise)
@@ -273,32 +259,32 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
     const T* hy = static_cast<const T*>(pd.hy);
     const T* hx = static_cast<const T*>(pd.hx);
     for (int k = tid; k < p; k += NT) {
-      s_w[k] = CORR ? hx[k] : hx[p - 1 - k];
-      s_w[p + k] = CORR ? hy[k] : hy[p - 1 - k];
+      s_w[k] = Pair<T>::w(CORR ? hx[k] : hx[p - 1 - k]);
+      s_w[p + k] = Pair<T>::w(CORR ? hy[k] : hy[p - 1 - k]);
     }
   } else {
     // the weights are stored in both orders: one flat, coalesced copy
     const T* tw = static_cast<const T*>(pd.tap_w) + (CORR ? 0 : pd.nrw);
     for (int k = tid; k < pd.nruns; k += NT) s_runs[k] = pd.tap_runs[k];
-    for (int k = tid; k < pd.nrw; k += NT) s_w[k] = tw[k];
+    for (int k = tid; k < pd.nrw; k += NT) s_w[k] = Pair<T>::w(tw[k]);
   }
   // input region
   const int oy0 = ZPAD ? ty0 - 2 * c : ty0 - c;
   const int ox0 = ZPAD ? tx0 - 2 * c : tx0 - c;
   // asynchronous copies straight into shared memory (no registers held, all
   // of a thread's copies in flight together); positions outside the source
-  // are zero-filled by a copy of 0 source bytes.  One warp per row, lanes
-  // along the row (RX <= 64 + MLBA_MAX_P - 1 = 128: four column passes at
-  // most); the row's source index is mapped once.
+  // are zero-filled by a copy of 0 source bytes.  The source row (and, where
+  // copied by elements, column) of every tile row (column) is mapped once, into a
+  // table: mapping every copy was a third of the kernel's instructions.
   // When the tile's columns lie inside the source, every tile row is one
   // contiguous source run: it is copied in 16-byte (or 8-byte) chunks from a
   // chunk-aligned start, the tile sitting xs elements into its shared-memory
   // row (xs = the start's offset from the chunk boundary; the same for every
-  // row when the source pitch is a multiple of the chunk); bytes past the
-  // source row are zero-filled.  Other tiles map every element.
+  // row when the source pitch is a multiple of the chunk), a thread keeping its
+  // chunk column and stepping down the rows; bytes past the source row are
+  // zero-filled.  Other tiles are walked flat, element by element.
   int xs = 0;
   {
-    const int lane = tid & 31;
     const int pitch = (!ZPAD && pd.bc == BC_RECT) ? pd.nf : n;
     const int sx0 = (!ZPAD && pd.bc == BC_RECT) ? ox0 + c : ox0;
     const bool colin = sx0 >= 0 && sx0 + RX <= pitch;
@@ -333,102 +319,119 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
           for (int b = 0; b < nx; ++b) v += wy[a] * wx[b] * src[(size_t)iy[a] * n + ix[b]];
         s_in[ry * RP + rx] = v;
       }
-    } else if (ce > 0) {
-      xs = sx0 % ce;
-      const int gs = sx0 - xs;
-      const int nch = (xs + RX + ce - 1) / ce;      // <= 65 (8-byte chunks of <= 129 values): three passes
-      for (int ry = tid >> 5; ry < RY; ry += NT / 32) {
-        const int ey = oy0 + ry;
-        int sy;
-        if (ZPAD) sy = (ey >= 0 && ey < n) ? ey : -1;
-        else if (pd.bc == BC_RECT) sy = (ey + c >= 0 && ey + c < pd.nf) ? ey + c : -1;
-        else sy = bc_map_near(ey, n, pd.bc);
-        const T* row = src + (size_t)(sy < 0 ? 0 : sy) * pitch;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int ch = lane + 32 * k;
-          if (ch < nch) {
-            const int g0 = gs + ch * ce;
-            int nv = pitch - g0;
-            nv = nv < 0 ? 0 : (nv > ce ? ce : nv);
-            if (sy < 0) nv = 0;
-            T* d = s_in + ry * RP + ch * ce;
-            const T* g = row + (nv > 0 ? g0 : 0);
-            if (ce * (int)sizeof(T) == 16) cp_async_bytes<16>(d, g, nv * (int)sizeof(T));
-            else cp_async_bytes<8>(d, g, nv * (int)sizeof(T));
+    } else {
+      const bool rect = !ZPAD && pd.bc == BC_RECT;
+      // source index of an extended index (-1: zero)
+      auto mapped = [&](int e) -> int {
+        if (ZPAD || rect) { const int q = e + (rect ? c : 0); return (q >= 0 && q < pitch) ? q : -1; }
+        return bc_map_near(e, n, pd.bc);
+      };
+      for (int k = tid; k < RY; k += NT) s_map[k] = mapped(oy0 + k);
+      if (ce == 0)
+        for (int k = tid; k < RX; k += NT) s_map[RY + k] = mapped(ox0 + k);
+      blk.sync();
+      if (ce > 0) {
+        xs = sx0 % ce;
+        const int gs = sx0 - xs;
+        const int nch = (xs + RX + ce - 1) / ce;       // <= 65 (8-byte chunks of <= 129 values)
+        const int lw = nch <= 32 ? 5 : nch <= 64 ? 6 : 7;   // threads per row: 32, 64 or 128
+        const int ch = tid & ((1 << lw) - 1), x = ch * ce;
+        int nv = pitch - gs - x;
+        nv = (nv < 0 ? 0 : (nv > ce ? ce : nv)) * (int)sizeof(T);
+        const T* g0 = src + (nv > 0 ? gs + x : 0);
+        if (ch < nch) {
+          const int dr = NT >> lw;
+          T* d = s_in + (tid >> lw) * RP + x;
+#pragma unroll 4
+          for (int ry = tid >> lw; ry < RY; ry += dr, d += dr * RP) {
+            const int sy = s_map[ry];
+            const T* g = g0 + (size_t)(sy < 0 ? 0 : sy) * pitch;
+            const int nb = sy < 0 ? 0 : nv;
+            if (ce * (int)sizeof(T) == 16) cp_async_bytes<16>(d, g, nb);
+            else cp_async_bytes<8>(d, g, nb);
           }
         }
-      }
-    } else {
-      for (int ry = tid >> 5; ry < RY; ry += NT / 32) {
-        const int ey = oy0 + ry;
-        int sy;
-        if (ZPAD) sy = (ey >= 0 && ey < n) ? ey : -1;
-        else if (pd.bc == BC_RECT) sy = (ey + c >= 0 && ey + c < pd.nf) ? ey + c : -1;
-        else sy = bc_map_near(ey, n, pd.bc);
-        const T* row = src + (size_t)(sy < 0 ? 0 : sy) * pitch;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int rx = lane + 32 * k;
-          if (rx < RX) {
-            const int ex = ox0 + rx;
-            int sx;
-            if (ZPAD) sx = (ex >= 0 && ex < n) ? ex : -1;
-            else if (pd.bc == BC_RECT) sx = (ex + c >= 0 && ex + c < pd.nf) ? ex + c : -1;
-            else sx = bc_map_near(ex, n, pd.bc);
-            const bool ok = sy >= 0 && sx >= 0;
-            cp_async_zfill<sizeof(T)>(s_in + ry * RP + rx, row + (ok ? sx : 0), ok);
-          }
+      } else {
+        const FastDiv frx(RX);
+        for (int idx = tid; idx < RY * RX; idx += NT) {
+          const int ry = frx.div(idx), rx = idx - ry * RX;
+          const int sy = s_map[ry], sx = s_map[RY + rx];
+          const bool ok = (sy | sx) >= 0;
+          cp_async_zfill<sizeof(T)>(s_in + ry * RP + rx, src + (ok ? (size_t)sy * pitch + sx : 0), ok);
         }
       }
     }
     cp_async_wait_all();
   }
   blk.sync();
-  // this thread's outputs: columns x2, x2 + 1, rows y8 .. y8 + 7 of the tile
-  const int x2 = 2 * (tid & 31), y8 = (tid >> 5) * 8;
-  T2 acc[8];
+  // this thread's outputs: columns x2, x2 + 1, rows y8 .. y8 + R - 1 of the tile
+  const int x2 = 2 * (tid & 31), y8 = (tid >> 5) * R;
+  T2 acc[R];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) { acc[j].x = T(0); acc[j].y = T(0); }
-  if (sep && 8 * RY <= ST_ROW_ITEMS * NT) {
-    // row pass over all RY rows, tmp(ry, xx) = sum_t wx[t] in(ry, xx + t): every
-    // thread first holds all of its (row, 8 columns) items in registers, then,
-    // after a barrier, writes them over the input tile (row ry of tmp at the
-    // start of input row ry), so no second tile is needed
-    T h[ST_ROW_ITEMS][8];
+  for (int j = 0; j < R; ++j) { acc[j].x = T(0); acc[j].y = T(0); }
+  if (sep) {
+    // column pass: tmp(y, c) = sum_t wy[t] in(y + t, c) for the tile's columns
+    // in pairs, an item being R rows of a pair.  Pairs are aligned in shared
+    // memory where the tile's shifted columns fit 64 pairs (else they start at
+    // the tile's first column); columns outside the tile give values nobody reads.
+    constexpr int RND = 2;                       // items per thread: 4 groups x 64 pairs = 2 x 128
+    const bool al = xs + RX <= 128;
+    const int c0 = al ? 0 : xs;                  // shared column of pair 0
+    const int np = al ? (xs + RX + 1) / 2 : (RX + 1) / 2;
+    const FastDiv fnp(np);
+    T2 tv[RND][R];
 #pragma unroll
-    for (int i = 0; i < ST_ROW_ITEMS; ++i) {
-      const int idx = tid + i * NT;
+    for (int i = 0; i < RND; ++i) {
+      const int it = tid + i * NT;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) h[i][j] = T(0);
-      if (idx < 8 * RY) window_run<T>(h[i], s_in + (idx >> 3) * RP + xs + (idx & 7) * 8, 1, s_w, p);
-    }
-    blk.sync();
-#pragma unroll
-    for (int i = 0; i < ST_ROW_ITEMS; ++i) {
-      const int idx = tid + i * NT;
-      if (idx < 8 * RY) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) s_in[(idx >> 3) * RP + (idx & 7) * 8 + j] = h[i][j];
+      for (int j = 0; j < R; ++j) { tv[i][j].x = T(0); tv[i][j].y = T(0); }
+      if (it < 4 * np) {
+        const int gr = fnp.div(it), cp = it - gr * np;
+        const T* base = s_in + (gr * R) * RP + c0 + 2 * cp;
+        if (al)
+          window_run<T, R>(tv[i], s_w + p, p, [&](int q) { return *reinterpret_cast<const T2*>(base + q * RP); });
+        else
+          window_run<T, R>(tv[i], s_w + p, p, [&](int q) { T2 v; v.x = base[q * RP]; v.y = base[q * RP + 1]; return v; });
       }
     }
     blk.sync();
-    // column pass: out(y, x) = sum_t wy[t] tmp(y + t, x)
-    window_run2<T>(acc, s_in + y8 * RP + x2, RP, s_w + p, p, true);
-  } else if (sep) {
-    // (taller tiles, p > 33) the row pass into a second tile
-    for (int idx = tid; idx < 8 * RY; idx += NT) {
-      const int ry = idx >> 3, x8 = (idx & 7) * 8;
-      T h[8];
+    // as row pairs over the input tile: element (y / 2, c) = (tmp(y, c), tmp(y + 1, c))
+    T2* tmp = reinterpret_cast<T2*>(s_in);
+    const int TP = st_tpitch(RX, (int)sizeof(T));
 #pragma unroll
-      for (int j = 0; j < 8; ++j) h[j] = T(0);
-      window_run<T>(h, s_in + ry * RP + xs + x8, 1, s_w, p);
+    for (int i = 0; i < RND; ++i) {
+      const int it = tid + i * NT;
+      if (it < 4 * np) {
+        const int gr = fnp.div(it), cp = it - gr * np;
+        T2* d = tmp + (gr * (R / 2)) * TP + 2 * cp;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) s_tmp[ry * ST_TP + x8 + j] = h[j];
+        for (int j = 0; j < R; j += 2) {
+          T2 lo, hi;
+          lo.x = tv[i][j].x; lo.y = tv[i][j + 1].x;
+          hi.x = tv[i][j].y; hi.y = tv[i][j + 1].y;
+          d[(j / 2) * TP] = lo;
+          d[(j / 2) * TP + 1] = hi;
+        }
+      }
     }
     blk.sync();
-    // column pass: out(y, x) = sum_t wy[t] tmp(y + t, x)
-    window_run2<T>(acc, s_tmp + y8 * ST_TP + x2, ST_TP, s_w + p, p, true);
+    // row pass: a thread does R columns of one row pair, out(y, x) = sum_t wx[t] tmp(y, x + t)
+    constexpr int NRP = ST_TY / 2;               // row pairs of the tile; 64 / R column groups
+    const int rp = tid % NRP, xg = (tid / NRP) * R;
+    const T2* hb = tmp + rp * TP + (xs - c0) + xg;
+    window_run<T, R>(acc, s_w, p, [&](int q) { return hb[q]; });
+    blk.sync();
+    // to the epilogue's layout (two columns x R rows) through shared memory
+    constexpr int OP = ST_TX + 2;
+    T* ot = s_in;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+      ot[(2 * rp) * OP + xg + j] = acc[j].x;
+      ot[(2 * rp + 1) * OP + xg + j] = acc[j].y;
+    }
+    blk.sync();
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[j] = *reinterpret_cast<const T2*>(ot + (y8 + j) * OP + x2);
   } else {
     // runs of PSF column b over rows lo..hi: input columns x + (CORR ? b : 2c - b),
     // window rows from y8 + (CORR ? lo : 2c - hi)
@@ -437,7 +440,13 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
       const int len = rn.z - rn.y + 1;
       const int col = CORR ? x2 + rn.x : x2 + 2 * c - rn.x;
       const int r0 = CORR ? y8 + rn.y : y8 + 2 * c - rn.z;
-      window_run2<T>(acc, s_in + r0 * RP + xs + col, RP, s_w + rn.w, len, ((xs + col) & 1) == 0);
+      const T* base = s_in + r0 * RP + xs + col;
+      const bool aligned = ((xs + col) & 1) == 0;
+      window_run<T, R>(acc, s_w + rn.w, len, [&](int q) -> T2 {
+        const T* v = base + q * RP;
+        if (aligned) return *reinterpret_cast<const T2*>(v);
+        T2 o; o.x = v[0]; o.y = v[1]; return o;
+      });
     }
   }
   T* dst = static_cast<T*>(pd.buf[dst_slot]);
@@ -458,11 +467,11 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
       dst[o] = a;
     }
   };
-  // the second operand (g or p) for all 16 outputs first, then the stores
-  T2 av[8];
+  // the second operand (g or p) for all outputs first, then the stores
+  T2 av[R];
   if (MODE == ST_FWD_RESID || MODE == ST_FWD_PCGQ) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < R; ++j) {
       const int gy = ty0 + y8 + j;
       const size_t o = (size_t)gy * outN + gx;
       av[j].x = (gy < outN && gx < outN) ? aux[o] : T(0);
@@ -470,7 +479,7 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
     }
   }
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
+  for (int j = 0; j < R; ++j) {
     const int gy = ty0 + y8 + j;
     if (gy < outN) {
       const size_t o = (size_t)gy * outN + gx;
@@ -479,7 +488,7 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
     }
   }
   if (MODE == ST_FWD_RESID || MODE == ST_FWD_PCGQ) {
-    // each thread's 16 terms in T; from the warp sum on, FP64 (an FP32
+    // each thread's 2 R terms in T; from the warp sum on, FP64 (an FP32
     // partial of 16 squares is within 16 u = 1e-6 of its exact value)
     double dl = (double)lacc;
     for (int o = 16; o > 0; o >>= 1) dl += __shfl_xor_sync(0xffffffffu, dl, o);
@@ -502,14 +511,14 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   }
 }
 
-template <typename T, int MODE>
+template <typename T, int MODE, int R>
 __global__ void __launch_bounds__(STENCIL_THREADS, sizeof(T) == 4 ? 8 : 4)
 k_stencil(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __restrict__ items,
           int src_slot, int dst_slot, int aux_slot, int pcg) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double red[32];
   __shared__ int flag;
-  stencil_body<T, MODE>(items[blockIdx.x], probs, states, src_slot, dst_slot, aux_slot, pcg, smraw,
+  stencil_body<T, MODE, R>(items[blockIdx.x], probs, states, src_slot, dst_slot, aux_slot, pcg, smraw,
                         red, &flag, BlkFull{});
 }
 
@@ -760,32 +769,37 @@ void launch_fc_out(const Prob* probs, State* states, const int2* items, int nite
 }
 
 // ---------------------------------------------------------------------------
-template <typename T>
-void launch_stencil(int mode, const Prob* probs, State* states, const int2* items, int nitems,
-                    int src, int dst, int aux, int pcg, size_t smem, cudaStream_t s) {
-  if (nitems <= 0) return;
-  dim3 g(nitems), b(STENCIL_THREADS);
+// the stencil kernel of a mode and of the rows per thread
+template <typename T, int R>
+auto stencil_kernel_r(int mode) {
   switch (mode) {
-    case ST_FWD_RESID: k_stencil<T, ST_FWD_RESID><<<g, b, smem, s>>>(probs, states, items, src, dst, aux, pcg); break;
-    case ST_FWD_STORE: k_stencil<T, ST_FWD_STORE><<<g, b, smem, s>>>(probs, states, items, src, dst, aux, pcg); break;
-    case ST_FWD_PCGQ: k_stencil<T, ST_FWD_PCGQ><<<g, b, smem, s>>>(probs, states, items, src, dst, aux, pcg); break;
-    case ST_REBLUR: k_stencil<T, ST_REBLUR><<<g, b, smem, s>>>(probs, states, items, src, dst, aux, pcg); break;
-    default: k_stencil<T, ST_CORR><<<g, b, smem, s>>>(probs, states, items, src, dst, aux, pcg); break;
+    case ST_FWD_RESID: return k_stencil<T, ST_FWD_RESID, R>;
+    case ST_FWD_STORE: return k_stencil<T, ST_FWD_STORE, R>;
+    case ST_FWD_PCGQ: return k_stencil<T, ST_FWD_PCGQ, R>;
+    case ST_REBLUR: return k_stencil<T, ST_REBLUR, R>;
+    default: return k_stencil<T, ST_CORR, R>;
   }
+}
+template <typename T>
+auto stencil_kernel(int mode, int R) {
+  return R == 2 ? stencil_kernel_r<T, 2>(mode) : R == 4 ? stencil_kernel_r<T, 4>(mode) : stencil_kernel_r<T, 8>(mode);
 }
 
 template <typename T>
-cudaError_t stencil_set_smem(size_t bytes) {
-  cudaError_t e = cudaSuccess;
-  e = cudaFuncSetAttribute(k_stencil<T, ST_FWD_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_stencil<T, ST_FWD_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_stencil<T, ST_FWD_PCGQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_stencil<T, ST_REBLUR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_stencil<T, ST_CORR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+void launch_stencil(int mode, const Prob* probs, State* states, const int2* items, int nitems,
+                    int src, int dst, int aux, int pcg, int rows, size_t smem, cudaStream_t s) {
+  if (nitems <= 0) return;
+  stencil_kernel<T>(mode, rows)<<<nitems, STENCIL_THREADS, smem, s>>>(probs, states, items, src, dst, aux, pcg);
+}
+
+template <typename T>
+cudaError_t stencil_set_smem(int rows) {
+  for (int mode : {(int)ST_FWD_RESID, (int)ST_FWD_STORE, (int)ST_FWD_PCGQ, (int)ST_REBLUR, (int)ST_CORR}) {
+    const cudaError_t e = cudaFuncSetAttribute((const void*)stencil_kernel<T>(mode, rows),
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 template <typename T>
@@ -804,10 +818,10 @@ void launch_vec(int mode, const Prob* probs, State* states, const int2* items, i
   }
 }
 
-template void launch_stencil<float>(int, const Prob*, State*, const int2*, int, int, int, int, int, size_t, cudaStream_t);
-template void launch_stencil<double>(int, const Prob*, State*, const int2*, int, int, int, int, int, size_t, cudaStream_t);
-template cudaError_t stencil_set_smem<float>(size_t);
-template cudaError_t stencil_set_smem<double>(size_t);
+template void launch_stencil<float>(int, const Prob*, State*, const int2*, int, int, int, int, int, int, size_t, cudaStream_t);
+template void launch_stencil<double>(int, const Prob*, State*, const int2*, int, int, int, int, int, int, size_t, cudaStream_t);
+template cudaError_t stencil_set_smem<float>(int);
+template cudaError_t stencil_set_smem<double>(int);
 template void launch_balance<float>(const Prob*, State*, const int2*, int, cudaStream_t);
 template void launch_balance<double>(const Prob*, State*, const int2*, int, cudaStream_t);
 template void launch_fc_pad<float>(const Prob*, State*, const int2*, int, int, int, cudaStream_t);

@@ -116,6 +116,7 @@ struct mlba_batch {
   int formulation = 0;
   std::vector<int2*> allocs;
   size_t smem_stencil = 0, smem_fft = 0;
+  int st_rows = 8;              // stencils: rows per thread (stencil_rows)
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool has_data = false;
@@ -291,8 +292,7 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
   State* S = B->d_states;
   if (part & PART_A) {
     // a2: r = g - A f with ||r||^2 and the stop rule
-    launch_stencil<T>(ST_FWD_RESID, P, S, L.blur.dev, L.blur.count, SL_F, SL_R, SL_G, 0,
-                      B->smem_stencil, s);
+    launch_stencil<T>(ST_FWD_RESID, P, S, L.blur.dev, L.blur.count, SL_F, SL_R, SL_G, 0, B->st_rows, B->smem_stencil, s);
     // (FFT blur path: f extended by the BCs, A f by convolution with the PSF)
     if (L.fc_out_r.count) {
       launch_fc_pad<T>(P, S, L.fc_pad_f.dev, L.fc_pad_f.count, 0, -1, s);
@@ -360,11 +360,9 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
       launch_rows_inv<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PZ, 1, B->smem_fft, s);
       launch_vec<T>(VEC_PCG_RHO0, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
       for (int k = 0; k < maxs; ++k) {
-        launch_stencil<T>(ST_CORR, P, S, L.corr_kry.dev, L.corr_kry.count, SL_PP, SL_V, SL_V, 1,
-                          B->smem_stencil, s);
+        launch_stencil<T>(ST_CORR, P, S, L.corr_kry.dev, L.corr_kry.count, SL_PP, SL_V, SL_V, 1, B->st_rows, B->smem_stencil, s);
         launch_vec<T>(VEC_FOLD, P, S, L.vec_kry_bc.dev, L.vec_kry_bc.count, 1, s);
-        launch_stencil<T>(ST_FWD_PCGQ, P, S, L.blur_kry.dev, L.blur_kry.count, -1, SL_PQ, SL_PP, 1,
-                          B->smem_stencil, s);
+        launch_stencil<T>(ST_FWD_PCGQ, P, S, L.blur_kry.dev, L.blur_kry.count, -1, SL_PQ, SL_PP, 1, B->st_rows, B->smem_stencil, s);
         launch_vec<T>(VEC_PCG_AXPY, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
         launch_rows_fwd<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PRES, 1, B->smem_fft, s);
         launch_cols<T>(P, S, L.cols_kry.dev, L.cols_kry.count, COL_FUSED, 1, 0.0, 0, B->smem_fft, s);
@@ -378,8 +376,8 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
   if (part & PART_B) {
     // a6: full correlation of t (A^T up to the BC fold); antireflective BCs:
     // the reblurring A' t into U
-    launch_stencil<T>(ST_CORR, P, S, L.corr.dev, L.corr.count, -1, SL_V, SL_V, 0, B->smem_stencil, s);
-    launch_stencil<T>(ST_REBLUR, P, S, L.reblur.dev, L.reblur.count, -1, -1, SL_U, 0, B->smem_stencil, s);
+    launch_stencil<T>(ST_CORR, P, S, L.corr.dev, L.corr.count, -1, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, s);
+    launch_stencil<T>(ST_REBLUR, P, S, L.reblur.dev, L.reblur.count, -1, -1, SL_U, 0, B->st_rows, B->smem_stencil, s);
     // (FFT blur path: t placed at (c, c), or extended antireflectively, and
     // correlated with the PSF)
     if (L.fc_pad_a.count) {
@@ -571,12 +569,12 @@ int build_split(mlba_batch* B) {
 
 int set_smem_attrs(mlba_batch* B) {
   if (B->dtype == MLBA_F64) {
-    CK(stencil_set_smem<double>(B->smem_stencil));
-    CK(fft_set_smem<double>(B->smem_fft));
+    CK(stencil_set_smem<double>(B->st_rows));
+    CK(fft_set_smem<double>());
     CK((frame_set_smem<double, double>()));
   } else {
-    CK(stencil_set_smem<float>(B->smem_stencil));
-    CK(fft_set_smem<float>(B->smem_fft));
+    CK(stencil_set_smem<float>(B->st_rows));
+    CK(fft_set_smem<float>());
     if (B->z_store == MLBA_BF16) CK((frame_set_smem<float, __nv_bfloat16>()));
     else CK((frame_set_smem<float, float>()));
   }
@@ -612,6 +610,23 @@ void destroy_batch(mlba_batch* B) {
   if (B->d_ctl) cudaFree(B->d_ctl);
   if (B->own_stream && B->stream) cudaStreamDestroy(B->stream);
   delete B;
+}
+
+// Rows per thread of the stencils (a tile is 64 x 4 rows-per-thread outputs).
+// 8 rows reuse every loaded value 8 times and win wherever the tiles fill the
+// chip; with fewer than about two tiles per SM a launch lasts as long as one
+// tile, and in FP64, whose pipe one warp per scheduler fills, as long as the
+// fullest scheduler: then the smallest height whose tiles still fit, down to 2
+// rows.  A step, 8 / 4 / 2 rows: 64^2 FP64 114 / 96 / 88 us; 256^2 FP64 L = 4
+// 387 / 308 / 284; 256^2 FP32 83 / 81 / 82; 226^2 FP32 100 / 96 / 95; 512^2 FP32
+// 68 / 68 / 69; 1024^2 FP32 (Algorithm 2) 576 / 593 / 670; 4096^2 1190 / 1258 / 1470.
+int stencil_rows(const mlba_batch* B) {
+  const double resident = B->dtype == MLBA_F64 ? 152.0 : 304.0;
+  for (int rows = 8;; rows /= 2) {
+    double tiles = 0.0;      // at half the rows
+    for (const HostProb& h : B->hp) tiles += stencil_tiles(h.pd.n, rows / 2);
+    if (rows == 2 || tiles > resident) return rows;
+  }
 }
 
 // Complex values per transform CTA for a set of problems whose passes run as
@@ -790,9 +805,6 @@ int setup_problem(const mlba_problem& in, const mlba_opts& o, HostProb& h) {
     }
   }
   pd.sep = rank_one(h.psf, p, h.hy, h.hx) && p > 1 ? 1 : 0;
-  // launch geometry
-  pd.nblk_blur = stencil_tiles(n);
-  pd.nblk_corr = stencil_tiles(pd.ne);
   // the frame kernel indexes a z array (all bands) with 32-bit offsets
   if ((double)pd.nbands * pd.nf * pd.nf >= 2147483647.0) return MLBA_E_UNSUPPORTED;
   pd.nblk_vec = vec_blocks((size_t)n * n);
@@ -1074,7 +1086,7 @@ int time_blur_paths(mlba_batch* B, int i, float* t_dir, float* t_fft) {
   State* S = B->d_opstates;
   cudaStream_t s = B->stream;
   auto direct = [&] {
-    launch_stencil<T>(ST_FWD_STORE, P, S, L[0].dev, L[0].count, SL_F, SL_AUX1, SL_AUX1, 0, B->smem_stencil, s);
+    launch_stencil<T>(ST_FWD_STORE, P, S, L[0].dev, L[0].count, SL_F, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, s);
   };
   auto fft = [&] {
     launch_fc_pad<T>(P, S, L[1].dev, L[1].count, 0, SL_F, s);
@@ -1127,9 +1139,9 @@ int choose_blur_paths(mlba_batch* B) {
 int build_persist(mlba_batch* B) {
   const StepLists L = all_lists(B);
   std::vector<std::vector<PersistStage>> groups;
-  auto st = [](int kind, const ItemList& l) {
+  auto st = [B](int kind, const ItemList& l) {
     PersistStage p;
-    p.kind = kind; p.count = l.count; p.items = l.dev; p.sync = 0; p.pad = 0;
+    p.kind = kind; p.count = l.count; p.items = l.dev; p.sync = 0; p.rows = B->st_rows;
     return p;
   };
   groups.push_back({st(PS_RESID, L.blur)});
@@ -1233,6 +1245,11 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
       B->fc.push_back(sa);
       h.pd.fc = (o.blur_path == 1) ? 1 : 0;       // 2: measured below
     }
+  }
+  B->st_rows = stencil_rows(B);
+  for (HostProb& h : B->hp) {
+    h.pd.nblk_blur = stencil_tiles(h.pd.n, B->st_rows);
+    h.pd.nblk_corr = stencil_tiles(h.pd.ne, B->st_rows);
   }
   // transforms per CTA: as many as fit, or fewer so that the batch's row and
   // column passes have about two CTAs per SM
@@ -1423,14 +1440,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
     size_t smem_st = 0, smem_fft = 0;
     for (int i = 0; i < count; ++i) {
       const Prob& pd = B->hp[i].pd;
-      // stencil: weights (padded to 16 bytes), runs, input tile, row-pass tile
-      const size_t RY = 32 + pd.p - 1, RX = 64 + pd.p - 1;
-      const size_t ce = 16 / ts;                  // input-tile pitch as in k_stencil.cu (st_pitch)
-      const size_t RP = (RX + 2 * (ce - 1)) / ce * ce;
-      const size_t nw = pd.sep ? 2 * pd.p : pd.nrw;
-      // (a second row-pass tile only for rank-one PSFs with 8 RY > 4 x 128, see k_stencil.cu)
-      const size_t st_b = (((nw + 3) & ~(size_t)3) + RY * RP + (pd.sep && 8 * RY > 4 * 128 ? RY * 66 : 0)) * ts +
-                          (pd.sep ? 0 : (size_t)pd.nruns * 16);
+      const size_t st_b = stencil_smem(B->st_rows, pd.p, pd.sep, pd.nrw, pd.nruns, (int)ts);
       smem_st = std::max(smem_st, st_b);
       if (pd.transform != TR_NONE) {
         // (antireflective columns also keep two weighted end values per transform)
@@ -1780,7 +1790,7 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
     if (stage == 0) {
       CK(cudaGraphLaunch(B->exec, s));
     } else if (B->dtype == MLBA_F64) {
-      if (stage == 1) launch_stencil<double>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->smem_stencil, s);
+      if (stage == 1) launch_stencil<double>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->st_rows, B->smem_stencil, s);
       if (stage == 2) {
         launch_rows_fwd<double>(P, S, B->rows_spec.dev, B->rows_spec.count, SL_R, 0, B->smem_fft, s);
         launch_cols<double>(P, S, B->cols_stat.dev, B->cols_stat.count, COL_FUSED, 0, 0.0, 0, B->smem_fft, s);
@@ -1792,12 +1802,12 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
         launch_ar_rows<double>(P, S, B->ar_rows.dev, B->ar_rows.count, SL_T, 1, 0, B->smem_fft, s);
       }
       if (stage == 3) {
-        launch_stencil<double>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->smem_stencil, s);
-        launch_stencil<double>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->smem_stencil, s);
+        launch_stencil<double>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, s);
+        launch_stencil<double>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->st_rows, B->smem_stencil, s);
       }
       if (stage == 4) launch_frame<double, double>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, B->frame_seg, s);
     } else {
-      if (stage == 1) launch_stencil<float>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->smem_stencil, s);
+      if (stage == 1) launch_stencil<float>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->st_rows, B->smem_stencil, s);
       if (stage == 2) {
         launch_rows_fwd<float>(P, S, B->rows_spec.dev, B->rows_spec.count, SL_R, 0, B->smem_fft, s);
         launch_cols<float>(P, S, B->cols_stat.dev, B->cols_stat.count, COL_FUSED, 0, 0.0, 0, B->smem_fft, s);
@@ -1809,8 +1819,8 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
         launch_ar_rows<float>(P, S, B->ar_rows.dev, B->ar_rows.count, SL_T, 1, 0, B->smem_fft, s);
       }
       if (stage == 3) {
-        launch_stencil<float>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->smem_stencil, s);
-        launch_stencil<float>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->smem_stencil, s);
+        launch_stencil<float>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, s);
+        launch_stencil<float>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->st_rows, B->smem_stencil, s);
       }
       if (stage == 4) {
         if (B->z_store == MLBA_BF16)
@@ -2160,10 +2170,10 @@ int mlba_op_blur(mlba_ctx* c, const void* f, void* out, int on_device) {
   }
   if (B->dtype == MLBA_F64)
     launch_stencil<double>(ST_FWD_STORE, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                           SL_AUX0, SL_AUX1, SL_AUX1, 0, B->smem_stencil, B->stream);
+                           SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
   else
     launch_stencil<float>(ST_FWD_STORE, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                          SL_AUX0, SL_AUX1, SL_AUX1, 0, B->smem_stencil, B->stream);
+                          SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
   CK(cudaGetLastError());
   return copy_out(B, out, pd.buf[SL_AUX1], (size_t)pd.n * pd.n * ts, on_device);
 }
@@ -2192,20 +2202,20 @@ int mlba_op_blur_adjoint(mlba_ctx* c, const void* t, void* out, int on_device) {
     // the reblurring matrix A' (Section 2.2), n x n
     if (B->dtype == MLBA_F64)
       launch_stencil<double>(ST_REBLUR, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                             SL_AUX0, SL_AUX1, SL_AUX1, 0, B->smem_stencil, B->stream);
+                             SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
     else
       launch_stencil<float>(ST_REBLUR, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                            SL_AUX0, SL_AUX1, SL_AUX1, 0, B->smem_stencil, B->stream);
+                            SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
     CK(cudaGetLastError());
     return copy_out(B, out, pd.buf[SL_AUX1], (size_t)pd.n * pd.n * ts, on_device);
   }
   if (B->dtype == MLBA_F64) {
     launch_stencil<double>(ST_CORR, B->d_probs, B->d_opstates, B->corr_all.dev, B->corr_all.count,
-                           SL_AUX0, SL_V, SL_V, 0, B->smem_stencil, B->stream);
+                           SL_AUX0, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, B->stream);
     if (pd.bc != BC_RECT) launch_vec<double>(VEC_FOLD, B->d_probs, B->d_opstates, B->vec_all.dev, B->vec_all.count, 0, B->stream);
   } else {
     launch_stencil<float>(ST_CORR, B->d_probs, B->d_opstates, B->corr_all.dev, B->corr_all.count,
-                          SL_AUX0, SL_V, SL_V, 0, B->smem_stencil, B->stream);
+                          SL_AUX0, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, B->stream);
     if (pd.bc != BC_RECT) launch_vec<float>(VEC_FOLD, B->d_probs, B->d_opstates, B->vec_all.dev, B->vec_all.count, 0, B->stream);
   }
   CK(cudaGetLastError());

@@ -46,6 +46,11 @@ enum {
 };
 enum { W_INV = 0, W_TIKH = 1 };
 
+// Dynamic shared memory every stencil and transform kernel may be launched with.
+// The limit belongs to the function, not to a batch: a fixed one, so that
+// creating a batch with small tiles leaves the launches of an earlier batch
+// with larger ones valid (227 KB per CTA less the kernels' static arrays).
+constexpr int SMEM_LIMIT = 220 * 1024;
 constexpr int STENCIL_THREADS = 128;
 constexpr int VEC_THREADS = 256;
 constexpr int VEC_PER_THREAD = 8;
@@ -59,7 +64,7 @@ constexpr int SPEC_SUMS = 17;        // block sums of the bracketing pass (2 x 8
 
 template <typename T>
 void launch_stencil(int mode, const Prob* probs, State* states, const int2* items, int nitems,
-                    int src, int dst, int aux, int pcg, size_t smem, cudaStream_t s);
+                    int src, int dst, int aux, int pcg, int rows, size_t smem, cudaStream_t s);
 template <typename T>
 void launch_vec(int mode, const Prob* probs, State* states, const int2* items, int nitems,
                 int pcg, cudaStream_t s);
@@ -101,7 +106,8 @@ int lev_tiles(int nf, int lev, int seg);                   // CTAs of one level 
 int lowpass_blocks(int nf);                       // CTAs of one low-pass launch (L >= 3)
 void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch);
 bool is_frame_kernel(const void* func);  // func is one of the framelet-update kernels
-int stencil_tiles(int outN);             // CTAs of the stencil for an outN x outN output
+int stencil_tiles(int outN, int R);      // CTAs of the stencil (R rows per thread) for an outN x outN output
+size_t stencil_smem(int R, int p, int sep, int nrw, int nruns, int elem);   // its shared memory
 // z layout: the 8 high-pass bands of a level contiguous per position, in
 // the polyphase order of the level's dilation for L >= 3 (z_index);
 // conversion to / from band-major planes
@@ -118,7 +124,7 @@ struct PersistStage {
   int kind, count;
   const int2* items;
   int sync;            // 1: a grid barrier follows (the next stage reads what this one wrote)
-  int pad;
+  int rows;            // stencil stages: rows per thread
 };
 size_t persist_smem(int dtype_bytes, int zs_bytes, int levels, size_t smem_stencil, size_t smem_fft,
                     int* stencil_slot, int* frame_slot);
@@ -134,8 +140,8 @@ cudaError_t persist_graph_set_k(cudaGraphExec_t x, cudaGraphNode_t knode, int zs
 size_t persist_ctl_bytes();
 int persist_threads();
 template <typename T>
-cudaError_t stencil_set_smem(size_t bytes);
+cudaError_t stencil_set_smem(int rows);
 template <typename T>
-cudaError_t fft_set_smem(size_t bytes);
+cudaError_t fft_set_smem();
 
 }  // namespace mlba

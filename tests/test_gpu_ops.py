@@ -315,3 +315,54 @@ def test_restart_reads_no_old_z(M, dtype, zs, levels, shape, formulation):
     np.testing.assert_array_equal(b.result(), ref)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("bc", ["zero", "periodic", "reflective", "rect", "antireflective"])
+@pytest.mark.parametrize("psf,n", [("gauss31", 300), ("gauss41", 260), ("disk17", 1030), ("motion7", 517),
+                                   ("gauss9", 1025), ("gauss65", 130), ("wide65", 131)])
+def test_blur_over_rows_per_thread(M, dtype, bc, psf, n):
+    """The stencils' rows per thread follow from the number of tiles (2, 4 and 8
+    over these sizes, 2 for the small operator tests): ragged tiles, odd and even
+    pitches (element, 8- and 16-byte tile copies), the largest PSF, rank-one and
+    general, against the oracle."""
+    extra = {"gauss65": I.psf_gaussian(9.0, 65), "wide65": I.psf_disk(31)}
+    h = extra[psf] if psf in extra else PSFS[psf]
+    ctx = M.Context(h, n, bc, "none", dtype=dtype)
+    rng = np.random.default_rng(n)
+    f = rng.standard_normal((ctx.nf, ctx.nf))
+    t = rng.standard_normal((n, n))
+    from scipy.signal import fftconvolve
+    c = (h.shape[0] - 1) // 2
+    ext = f if bc == "rect" else O.extend(f, c, bc)
+    assert rel_err(ctx.blur(f), fftconvolve(ext, h, mode="valid")) <= TOL[dtype]
+    if bc == "antireflective":
+        ref = fftconvolve(O.extend(t, c, bc), h[::-1, ::-1], mode="valid")
+    else:
+        v = fftconvolve(t, h[::-1, ::-1], mode="full")
+        if bc != "rect":
+            idx = O.bc_index(np.arange(-c, n + c), n, bc)
+            ok = idx >= 0
+            rows = np.zeros((n, n + 2 * c))
+            np.add.at(rows, idx[ok], v[ok, :])
+            u = np.zeros((n, n))
+            np.add.at(u.T, idx[ok], rows.T[ok, :])
+            v = u
+        ref = v
+    assert rel_err(ctx.blur_adjoint(t), ref) <= TOL[dtype]
+    ctx.close()
+
+
+def test_contexts_with_other_tile_sizes_stay_usable(M):
+    """Creating a context with a small PSF and transform leaves the launches of
+    an earlier context with larger shared-memory tiles valid."""
+    rng = np.random.default_rng(3)
+    big = M.Context(PSFS["disk17"], 72, "zero", "none", dtype="f64")
+    pre = M.Context(PSFS["gauss9"], 256, "periodic", "bccb", dtype="f64")
+    small_psf = M.Context(PSFS["asym3"], 17, "zero", "bccb", dtype="f64")
+    f = rng.standard_normal((72, 72))
+    assert rel_err(big.blur(f), O.blur(f, PSFS["disk17"], "zero")) <= TOL["f64"]
+    r = rng.standard_normal((256, 256))
+    assert rel_err(pre.precond(r, 0.1), O.SpectralPrecond(PSFS["gauss9"], 256, "dft").inv(r, 0.1)) <= TOL["f64"]
+    for x in (big, pre, small_psf):
+        x.close()
