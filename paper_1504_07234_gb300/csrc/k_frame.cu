@@ -20,6 +20,7 @@
 // u comes from (per problem): the full correlation V folded by the BC
 // transpose (A^T t for imposed boundary conditions), V itself (rectangular
 // A), or t (Algorithm 4 forms, where C^T is already applied).
+#include <algorithm>
 #include <type_traits>
 #include "mlba_internal.cuh"
 #include "mlba_launch.h"
@@ -1016,39 +1017,62 @@ void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch) {
   *prefetch = F3_SHAPES[shape].ring > 0 ? F3_SHAPES[shape].ring : F3_SHAPES[shape].pf;
 }
 
-// Planar (band-major) <-> internal z layout (z_index), element size E bytes.
-template <typename E>
-__global__ void k_zlayout(E* __restrict__ dst, const E* __restrict__ src, int levels, int nf,
-                          int to_internal) {
-  const size_t plane = (size_t)nf * nf;
-  const size_t tot = (size_t)(8 * levels + 1) * plane;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < tot;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int b = (int)(i / plane);
-    const int q = (int)(i - (size_t)b * plane);
+// Planar (band-major) <-> internal z layout (z_index), elements E of 2, 4 or 8
+// bytes.  A thread moves one pixel's 8 bands of a level: its accesses to the
+// planes are consecutive along the warp, its group is one or more 16-byte
+// words (a whole sector or more for 4- and 8-byte elements wherever the
+// polyphase order puts it); then the low-pass plane.  HBM-bound: 751^2, L = 2,
+// FP32: 13 us a direction (2 x 38 MB); element by element it took 42.
+template <typename E, bool TO_INTERNAL>
+__global__ void __launch_bounds__(256)
+k_zlayout(E* __restrict__ dst, const E* __restrict__ src, int levels, int nf) {
+  union Group {
+    uint4 v[8 * sizeof(E) / 16];
+    E e[8];
+  };
+  const int plane = nf * nf;                       // nbands nf^2 < 2^31
+  const int tot = (levels + 1) * plane;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < tot; i += gridDim.x * 256) {
+    const int l = i / plane, q = i - l * plane;    // level l + 1; l = levels: the low-pass plane
     const int y = q / nf, x = q - y * nf;
-    const size_t g = z_index(b, y, x, levels, nf);
-    if (to_internal) dst[g] = src[i]; else dst[i] = src[g];
+    const int lev = l < levels ? l : levels - 1;
+    const Poly P(nf, levels >= 3 ? 1 << lev : 1);
+    const int p = P.pos(y) * nf + P.pos(x);
+    if (l == levels) {
+      const int o = 8 * levels * plane;
+      if (TO_INTERNAL) dst[o + p] = src[o + q]; else dst[o + q] = src[o + p];
+      continue;
+    }
+    const int pb = 8 * l * plane + q, gb = 8 * l * plane + 8 * p;
+    Group g;
+    if (TO_INTERNAL) {
+#pragma unroll
+      for (int b = 0; b < 8; ++b) g.e[b] = src[pb + b * plane];
+#pragma unroll
+      for (int v = 0; v < (int)(8 * sizeof(E) / 16); ++v) reinterpret_cast<uint4*>(dst + gb)[v] = g.v[v];
+    } else {
+#pragma unroll
+      for (int v = 0; v < (int)(8 * sizeof(E) / 16); ++v) g.v[v] = reinterpret_cast<const uint4*>(src + gb)[v];
+#pragma unroll
+      for (int b = 0; b < 8; ++b) dst[pb + b * plane] = g.e[b];
+    }
   }
 }
 
-bool z_grouped(int levels) { (void)levels; return true; }
-
 void launch_z_layout(void* dst, const void* src, int levels, int nf, int elem_bytes,
                      int to_grouped, cudaStream_t s) {
-  const int nbands = 8 * levels + 1;
-  const size_t tot = (size_t)nbands * nf * nf;
-  int blocks = (int)((tot + 255) / 256);
-  if (blocks > 152 * 32) blocks = 152 * 32;
-  if (elem_bytes == 8)
-    k_zlayout<unsigned long long><<<blocks, 256, 0, s>>>(static_cast<unsigned long long*>(dst),
-        static_cast<const unsigned long long*>(src), levels, nf, to_grouped);
-  else if (elem_bytes == 4)
-    k_zlayout<unsigned int><<<blocks, 256, 0, s>>>(static_cast<unsigned int*>(dst),
-        static_cast<const unsigned int*>(src), levels, nf, to_grouped);
-  else
-    k_zlayout<unsigned short><<<blocks, 256, 0, s>>>(static_cast<unsigned short*>(dst),
-        static_cast<const unsigned short*>(src), levels, nf, to_grouped);
+  const size_t tot = (size_t)(levels + 1) * nf * nf;
+  const int blocks = (int)std::min<size_t>((tot + 255) / 256, 152 * 16);
+  auto go = [&](auto e) {
+    using E = decltype(e);
+    if (to_grouped)
+      k_zlayout<E, true><<<blocks, 256, 0, s>>>(static_cast<E*>(dst), static_cast<const E*>(src), levels, nf);
+    else
+      k_zlayout<E, false><<<blocks, 256, 0, s>>>(static_cast<E*>(dst), static_cast<const E*>(src), levels, nf);
+  };
+  if (elem_bytes == 8) go((unsigned long long)0);
+  else if (elem_bytes == 4) go((unsigned int)0);
+  else go((unsigned short)0);
 }
 
 // the kernel of one tile shape, its shared memory and its launch (FP64 has

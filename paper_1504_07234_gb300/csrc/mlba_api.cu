@@ -115,6 +115,7 @@ struct mlba_batch {
   ItemList balance;
   int formulation = 0;
   std::vector<int2*> allocs;
+  void* op_z[2] = {nullptr, nullptr};   // mlba_op_frame: z in the internal order (first call)
   size_t smem_stencil = 0, smem_fft = 0;
   int st_rows = 8;              // stencils: rows per thread (stencil_rows)
   cudaGraph_t graph = nullptr;
@@ -608,6 +609,7 @@ void destroy_batch(mlba_batch* B) {
   if (B->p_graph) cudaGraphDestroy(B->p_graph);
   if (B->d_stages) cudaFree(B->d_stages);
   if (B->d_ctl) cudaFree(B->d_ctl);
+  for (void* p : B->op_z) if (p) cudaFree(p);
   if (B->own_stream && B->stream) cudaStreamDestroy(B->stream);
   delete B;
 }
@@ -1971,7 +1973,6 @@ int mlba_get_z(mlba_ctx* c, void* z_out, int on_device) {
     else CK(cudaMemsetAsync(z_out, 0, zbytes, B->stream));
     return MLBA_OK;
   }
-  if (!z_grouped(pd.levels)) return copy_out(B, z_out, pd.z[s.iter & 1], zbytes, on_device);
   // the library keeps z in its internal order (z_index); the caller gets band-major planes
   if (on_device) {
     launch_z_layout(z_out, pd.z[s.iter & 1], pd.levels, pd.nf, (int)es, 0, B->stream);
@@ -2102,9 +2103,7 @@ int mlba_set_state(mlba_ctx* c, const void* blob, size_t bytes) {
   const size_t es = zsize(B->z_store);
   const size_t zbytes = (size_t)pd.nbands * plane * es;
   void* zdst = pd.z[h.iter & 1];
-  if (!z_grouped(pd.levels)) {
-    CK(cudaMemcpy(zdst, in + L.z, zbytes, cudaMemcpyHostToDevice));
-  } else {
+  {
     std::vector<unsigned char> g(zbytes);
     for (int b = 0; b < pd.nbands; ++b)
       for (size_t q = 0; q < plane; ++q)
@@ -2273,18 +2272,20 @@ int mlba_op_frame(mlba_ctx* c, const void* z_in, const void* u, void* z_out, voi
     CK(cudaMalloc(&dzo, zbytes));
     CK(cudaMemcpyAsync(dzi, z_in, zbytes, cudaMemcpyHostToDevice, B->stream));
   }
-  // the kernel works on grouped z (L <= 2): convert the caller's band-major
-  // planes into scratch copies and back
-  const bool grouped = z_grouped(pd.levels);
+  // the kernels work on the internal order of z: convert the caller's
+  // band-major planes into scratch copies and back (allocated by the first call
+  // and kept with the context: two allocations and frees cost more than the
+  // step itself)
   const int es = (int)zsize(B->z_store);
-  void *gzi = nullptr, *gzo = nullptr;
-  if (grouped) {
-    CK(cudaMalloc(&gzi, zbytes));
-    CK(cudaMalloc(&gzo, zbytes));
-    launch_z_layout(gzi, dzi, pd.levels, pd.nf, es, 1, B->stream);
-  }
-  void* kzi = grouped ? gzi : dzi;
-  void* kzo = grouped ? gzo : dzo;
+  for (void** p : {&B->op_z[0], &B->op_z[1]})
+    if (!*p && cudaMalloc(p, zbytes) != cudaSuccess) {
+      (void)cudaGetLastError();
+      *p = nullptr;
+      if (!on_device) { cudaFree(dzi); cudaFree(dzo); }
+      return MLBA_E_NOMEM;
+    }
+  void *kzi = B->op_z[0], *kzo = B->op_z[1];
+  launch_z_layout(kzi, dzi, pd.levels, pd.nf, es, 1, B->stream);
   int rc = copy_in(B, pd.buf[SL_AUX0], u, fbytes, on_device);
   if (rc != MLBA_OK) return rc;
   if (reset_opstates(B) != MLBA_OK) return MLBA_E_CUDA;
@@ -2295,13 +2296,8 @@ int mlba_op_frame(mlba_ctx* c, const void* z_in, const void* u, void* z_out, voi
   else
     launch_frame<float, float>(B->d_probs, B->d_opstates, B->frame.dev, B->frame.count, B->frame.sec, SL_AUX0, SL_AUX1, kzi, kzo, mu, B->levels, B->frame_shape, B->frame_seg, B->stream);
   CK(cudaGetLastError());
-  if (grouped) {
-    launch_z_layout(dzo, gzo, pd.levels, pd.nf, es, 0, B->stream);
-    CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(B->stream));
-    cudaFree(gzi);
-    cudaFree(gzo);
-  }
+  launch_z_layout(dzo, kzo, pd.levels, pd.nf, es, 0, B->stream);
+  CK(cudaGetLastError());
   rc = copy_out(B, f, pd.buf[SL_AUX1], fbytes, on_device);
   if (rc != MLBA_OK) return rc;
   if (!on_device) {

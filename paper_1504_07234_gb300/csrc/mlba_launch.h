@@ -111,7 +111,6 @@ size_t stencil_smem(int R, int p, int sep, int nrw, int nruns, int elem);   // i
 // z layout: the 8 high-pass bands of a level contiguous per position, in
 // the polyphase order of the level's dilation for L >= 3 (z_index);
 // conversion to / from band-major planes
-bool z_grouped(int levels);
 void launch_z_layout(void* dst, const void* src, int levels, int nf, int elem_bytes,
                      int to_grouped, cudaStream_t s);
 template <typename T, typename TZ>

@@ -366,3 +366,37 @@ def test_contexts_with_other_tile_sizes_stay_usable(M):
     assert rel_err(pre.precond(r, 0.1), O.SpectralPrecond(PSFS["gauss9"], 256, "dft").inv(r, 0.1)) <= TOL["f64"]
     for x in (big, pre, small_psf):
         x.close()
+
+
+@pytest.mark.parametrize("dtype,zs", [("f32", "f32"), ("f32", "bf16"), ("f64", "f64")])
+@pytest.mark.parametrize("levels,n", [(1, 7), (2, 53), (3, 21), (4, 75)])
+def test_frame_call_repeats_and_leaves_the_state_alone(M, dtype, zs, levels, n):
+    """The framelet operator keeps its scratch between calls: a second call on
+    other data gives what a new context gives, caller tensors at odd element
+    offsets are accepted, and the context's own iterates do not change."""
+    import torch
+    h = PSFS["asym3"]
+    rng = np.random.default_rng(n)
+    ctx = M.Context(h, n, "reflective", "none", dtype=dtype, z_store=zs, levels=levels, max_iter=9, stop=False)
+    g = rng.standard_normal((n, n))
+    ctx.set_data(g, 0.1)
+    ctx.iterate(2)
+    f0, z0 = ctx.result(), ctx.get_z().float().cpu().numpy()
+    zdt = {"f32": torch.float32, "bf16": torch.bfloat16, "f64": torch.float64}[zs]
+    shape = (8 * levels + 1, n, n)
+    for k in range(2):
+        flat = torch.empty(int(np.prod(shape)) + 1, dtype=zdt, device="cuda")
+        zi = flat[1:].view(shape)
+        zi.copy_(torch.from_numpy(0.05 * rng.standard_normal(shape)))
+        u = 0.1 * rng.standard_normal((n, n))
+        zo, f = ctx.frame(zi, u, 0.03)
+        other = M.Context(h, n, "reflective", "none", dtype=dtype, z_store=zs, levels=levels)
+        zr, fr = other.frame(zi.clone(), u, 0.03)
+        assert torch.equal(zo, zr) and torch.equal(f, fr)
+        other.close()
+        zin = zi.double().cpu().numpy()
+        z_ref = zin + O.framelet_analysis(u, levels)
+        assert rel_err(zo.double().cpu().numpy(), z_ref) <= {"f64": 1e-12, "f32": 2e-6, "bf16": 1e-2}[zs]
+    np.testing.assert_array_equal(ctx.result(), f0)
+    np.testing.assert_array_equal(ctx.get_z().float().cpu().numpy(), z0)
+    ctx.close()
