@@ -197,6 +197,22 @@ bool fft_plan(Prob& pd) {
   return m == 1;
 }
 
+// The twiddles in the order of the radix passes (Prob::ptw), from the table tw
+// of exp(-2 pi i m/nfft); the direct-sum passes keep tw.
+std::vector<double> pass_twiddles(const Prob& pd, const std::vector<double>& tw) {
+  std::vector<double> o(tw.size(), 0.0);
+  for (int s = 0, Ns = 1; s < pd.nstage; Ns *= pd.radix[s], ++s) {
+    const int R = pd.radix[s], step = pd.nfft / (Ns * R);
+    for (int r = 1; r < R; ++r)
+      for (int k = 0; k < Ns; ++k) {
+        const size_t d = (size_t)Ns - 1 + (size_t)(r - 1) * Ns + k, m = (size_t)r * k * step;
+        o[2 * d] = tw[2 * m];
+        o[2 * d + 1] = tw[2 * m + 1];
+      }
+  }
+  return o;
+}
+
 bool quad_symmetric(const std::vector<double>& h, int p) {
   double mx = 0;
   for (double v : h) mx = std::max(mx, std::fabs(v));
@@ -669,6 +685,10 @@ void transform_geometry(Prob& pd, int fill) {
     const int units = dct ? pairs : pd.half;           // complex columns to transform
     const int nb = (units + cap - 1) / cap;
     pd.col_g = std::max(1, (units + nb - 1) / nb);
+    // DFT: an even number of complex columns where two fit a CTA, so that the
+    // passes move them in pairs (16-byte words)
+    if (!dct && (pd.col_g & 1) && std::min(TR_CAP, 2 * fill) / std::max(pd.nfft, n) >= 2)
+      pd.col_g += pd.col_g == 1 || (pd.col_g + 1) * std::max(pd.nfft, n) <= TR_CAP ? 1 : -1;
     pd.cb = dct ? 2 * pd.col_g : pd.col_g;
     pd.nblk_cols = ((dct ? n : pd.half) + pd.cb - 1) / pd.cb;
   }
@@ -1297,6 +1317,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
         (pd.levels >= 3 ? (size_t)(pd.levels - 1) * nf2 : 1) * ts,   // low-pass chain (L >= 3)
         (pd.levels >= 3 ? (size_t)(pd.levels - 1) * nf2 : 1) * ts,   // synthesis partials
         spec ? (size_t)pd.nfft * 2 * ts : ts,  // tw
+        spec ? (size_t)pd.nfft * 2 * ts : ts,  // ptw
         spec ? (size_t)pd.n * 2 * ts : ts,     // dtw
         (size_t)pd.nruns * 16, 2 * (size_t)pd.nrw * ts,   // tap runs and weights (both orders)
         (size_t)pd.p * ts, (size_t)pd.p * ts,  // hy, hx
@@ -1325,7 +1346,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
     const Prob& sf = B->fc[2 * k].pd;
     const size_t M2 = (size_t)sf.n * sf.n, nspec = spec_elems(sf);
     std::vector<size_t> sz = {M2 * ts, M2 * ts, nspec * 2 * ts, nspec * 2 * ts, nspec * 2 * ts,
-                              nspec * ts, (size_t)sf.nfft * 2 * ts};
+                              nspec * ts, (size_t)sf.nfft * 2 * ts, (size_t)sf.nfft * 2 * ts};
     foffs[k].resize(sz.size());
     for (size_t q = 0; q < sz.size(); ++q) { foffs[k][q] = total; total += al(sz[q]); }
   }
@@ -1352,6 +1373,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
     pd.lp = base + of[k++];
     pd.sy = base + of[k++];
     pd.tw = base + of[k++];
+    pd.ptw = base + of[k++];
     pd.dtw = base + of[k++];
     pd.tap_runs = reinterpret_cast<int4*>(base + of[k++]);
     pd.tap_w = base + of[k++];
@@ -1386,7 +1408,8 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
         const double b = M_PI * (double)m / (2.0 * (double)pd.n);
         dtw[2 * m] = std::cos(b); dtw[2 * m + 1] = -std::sin(b);
       }
-      if (upload(pd.tw, tw) != MLBA_OK || upload(pd.dtw, dtw) != MLBA_OK) {
+      if (upload(pd.tw, tw) != MLBA_OK || upload(pd.ptw, pass_twiddles(pd, tw)) != MLBA_OK ||
+          upload(pd.dtw, dtw) != MLBA_OK) {
         destroy_batch(B); return MLBA_E_CUDA;
       }
       const int rc = build_spectrum(B, h);
@@ -1404,6 +1427,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
       pd.lam = base + of[3 + a];
       pd.w = base + of[5];
       pd.tw = pd.dtw = base + of[6];
+      pd.ptw = base + of[7];
     }
     const Prob& sf = B->fc[2 * k].pd;
     std::vector<double> tw(2 * (size_t)sf.nfft);
@@ -1412,9 +1436,12 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
       tw[2 * m] = std::cos(a); tw[2 * m + 1] = -std::sin(a);
     }
     std::vector<unsigned char> tmp(tw.size() * ts);
-    if (ts == 8) put<double>(tmp.data(), 0, tw); else put<float>(tmp.data(), 0, tw);
-    if (cudaMemcpy(sf.tw, tmp.data(), tmp.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
-      destroy_batch(B); return MLBA_E_CUDA;
+    const std::vector<double> pt = pass_twiddles(sf, tw);
+    for (const std::vector<double>* v : {static_cast<const std::vector<double>*>(&tw), &pt}) {
+      if (ts == 8) put<double>(tmp.data(), 0, *v); else put<float>(tmp.data(), 0, *v);
+      if (cudaMemcpy(v == &tw ? sf.tw : sf.ptw, tmp.data(), tmp.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+        destroy_batch(B); return MLBA_E_CUDA;
+      }
     }
     for (int a = 0; a < 2; ++a) {
       const int rc = build_spectrum(B, B->fc[2 * k + a]);

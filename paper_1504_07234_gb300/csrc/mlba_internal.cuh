@@ -73,7 +73,10 @@ struct Prob {
   void* lam;         // spectrum of C (real for DCT, complex half for DFT), T, blocked
   void* lp;          // L >= 3: low-pass chain c_1 .. c_{L-1} (nf x nf planes, T)
   void* sy;          // L >= 3: synthesis partials s_1 .. s_{L-1} (nf x nf planes, T)
-  void* tw;          // exp(-2 pi i k/nfft), k < nfft   (T2)
+  void* tw;          // exp(-2 pi i k/nfft), k < nfft   (T2): direct-sum passes
+  void* ptw;         // the same values in the order the radix passes read them: the pass
+                     // that joins transforms of length Ns has its radix R's twiddles
+                     // exp(-2 pi i r k/(Ns R)) at Ns - 1 + (r - 1) Ns + k (1 <= r < R, k < Ns)
   void* dtw;         // exp(-i pi k/(2n)), k < n  (T2)
   int4* tap_runs;     // per nonzero PSF column b: (b, lo, hi, offset of H[lo..hi][b] in tap_w)
   void* tap_w;        // packed run weights, T precision: nrw in PSF order, then nrw with
@@ -116,6 +119,9 @@ __host__ __device__ __forceinline__ T2 mk2(T a, T b) { T2 r; r.x = a; r.y = b; r
 
 template <typename T2> __device__ __forceinline__ T2 cadd(T2 a, T2 b) { a.x += b.x; a.y += b.y; return a; }
 template <typename T2> __device__ __forceinline__ T2 csub(T2 a, T2 b) { a.x -= b.x; a.y -= b.y; return a; }
+// FP32: one paired instruction each (a - b as the exact a + (-1) b)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 template <typename T2> __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
   T2 r; r.x = a.x * b.x - a.y * b.y; r.y = a.x * b.y + a.y * b.x; return r;
 }

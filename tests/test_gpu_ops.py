@@ -400,3 +400,22 @@ def test_frame_call_repeats_and_leaves_the_state_alone(M, dtype, zs, levels, n):
     np.testing.assert_array_equal(ctx.result(), f0)
     np.testing.assert_array_equal(ctx.get_z().float().cpu().numpy(), z0)
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("transform", ["dft", "dct"])
+@pytest.mark.parametrize("n", [2, 3, 5, 9, 16, 17, 32, 81, 125, 144, 240, 375, 512, 750, 768, 1000, 1024, 1200])
+def test_transform_lengths(M, dtype, transform, n):
+    """Every first radix (16, 8, 4, 2, 3, 5, a prime) and the strides that are and
+    are not multiples of 16 in later passes, one and several columns per block:
+    the preconditioner against the oracle."""
+    p = 3 if n >= 3 else 1
+    h = I.psf_gaussian(0.7, p) if p > 1 else np.ones((1, 1))
+    ctx = M.Context(h, n, "periodic" if transform == "dft" else "reflective", "bccb", dtype=dtype,
+                    transform=transform)
+    pre = O.SpectralPrecond(h, n, transform)
+    r = np.random.default_rng(n).standard_normal((n, n))
+    for which in ("inv", "tikh"):
+        ref = pre.inv(r, 0.05) if which == "inv" else pre.tikh(r, 0.05)
+        assert rel_err(ctx.precond(r, 0.05, which), ref) <= (1e-11 if dtype == "f64" else 2e-5)
+    ctx.close()
