@@ -830,6 +830,32 @@ __device__ __forceinline__ void rows_fwd_body(const int2 item, const Prob* __res
     // columns in pairs (c, c + 1): one 8-byte (DCT) or 16-byte (DFT) store
     const int H = cb / 2;
     const FastDiv frh(R2 * H), fh(H);
+    if (R2 * H <= NT) {
+      // a thread keeps its row and column pair and steps through the blocks
+      // (mapping every pair took a seventh of the kernel's instructions)
+      const int nbk = frh.div(NT), q = frh.div(threadIdx.x), rem = threadIdx.x - q * (R2 * H);
+      const int rl = fh.div(rem), c = 2 * (rem - rl * H), row = row0 + rl;
+      if (q >= nbk || row >= N) return;
+      const T2* tb = sm + (rl >> 1) * TSg;
+      size_t o = (size_t)q * N * cb + (size_t)row * cb + c;
+      const size_t od = (size_t)nbk * N * cb;
+      for (int k = q * cb + c; k < W; k += nbk * cb, o += od) {
+        const bool two = k + 1 < W;
+        if (dct) {
+          // (k is even: k + 1 is the next slot)
+          const T* v = reinterpret_cast<const T*>(tb + fpad(k)) + (rl & 1);
+          T* S = static_cast<T*>(pd.buf[SL_S]);
+          if (two) *reinterpret_cast<T2*>(S + o) = mk2<T2>(v[0], v[2]);
+          else S[o] = v[0];
+        } else {
+          T2* S = static_cast<T2*>(pd.buf[SL_S]);
+          const T2 x0 = spec_val(tb, rl, k);
+          if (two) stc2(S + o, x0, spec_val(tb, rl, k + 1));
+          else S[o] = x0;
+        }
+      }
+      return;
+    }
     for (int e = threadIdx.x; e < nb * R2 * H; e += NT) {
       const int b = frh.div(e), rem = e - b * (R2 * H);
       const int rl = fh.div(rem), c = 2 * (rem - rl * H);
@@ -1215,6 +1241,51 @@ __device__ __forceinline__ void rows_inv_body(const int2 item, const Prob* __res
     const int H = cb / 2;
     const int tot2 = nb * G * H;
     const FastDiv fgh(G * H), fh(H);
+    if (G * H <= NT) {
+      // a thread keeps its row pair and column pair and steps through the blocks
+      const int nbk = fgh.div(NT), q = fgh.div(threadIdx.x), rem = threadIdx.x - q * (G * H);
+      const int g = fh.div(rem), c = 2 * (rem - g * H), ra = row0 + 2 * g;
+      T2* tb = sm + g * TSg;
+      const bool rb = ra + 1 < N;
+      const int dk = nbk * cb;
+      const size_t od = (size_t)nbk * N * cb;
+      size_t o = (size_t)q * N * cb + (size_t)ra * cb + c;
+      if (q < nbk && ra < N) {
+        for (int k = q * cb + c; k < W; k += BATCH2 * dk, o += BATCH2 * od) {
+          T2 a0[BATCH2], a1[BATCH2], b0[BATCH2], b1[BATCH2];
+#pragma unroll
+          for (int u = 0; u < BATCH2; ++u) {
+            a0[u].x = a0[u].y = a1[u].x = a1[u].y = T(0);
+            b0[u] = a0[u]; b1[u] = a0[u];
+            if (k + u * dk < W) {
+              if (dct) {
+                const T* S = static_cast<const T*>(pd.buf[SL_S]) + (o + u * od);
+                a0[u] = *reinterpret_cast<const T2*>(S);                  // row ra, columns c, c + 1
+                if (rb) b0[u] = *reinterpret_cast<const T2*>(S + cb);
+              } else {
+                const T2* S = static_cast<const T2*>(pd.buf[SL_S]) + (o + u * od);
+                ldc2(S, a0[u], a1[u]);
+                if (rb) ldc2(S + cb, b0[u], b1[u]);
+              }
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < BATCH2; ++u) {
+            const int kk = k + u * dk;
+            if (kk >= W) continue;
+            const bool two = kk + 1 < W;
+            if (dct) {
+              T2* d = tb + fpad(kk);                 // (kk is even: kk + 1 is the next slot)
+              d[0] = mk2<T2>(a0[u].x, b0[u].x);
+              if (two) d[1] = mk2<T2>(a0[u].y, b0[u].y);
+            } else {
+              put_dft(tb, kk, a0[u], b0[u]);
+              if (two) put_dft(tb, kk + 1, a1[u], b1[u]);
+            }
+          }
+        }
+      }
+    } else
     for (int e0 = threadIdx.x; e0 < tot2; e0 += BATCH2 * NT) {
       T2 a0[BATCH2], a1[BATCH2], b0[BATCH2], b1[BATCH2];
       int kq[BATCH2];
