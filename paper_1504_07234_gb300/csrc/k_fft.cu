@@ -1200,15 +1200,21 @@ k_cols(const Prob* __restrict__ probs, State* __restrict__ states, const int2* _
   cols_body<T, mode>(items[blockIdx.x], probs, states, pcg, op_alpha, op_kind);
 }
 
-// Pass 3: inverse transform of row pairs: S -> dst (n x n real)
-template <typename T>
-__device__ __forceinline__ void rows_inv_body(const int2 item, const Prob* __restrict__ probs, State* __restrict__ states, int dst_slot, int pcg) {
+// Pass 3: inverse transform of row pairs: S -> dst (n x n real).  epi stores the
+// values at element i of dst (and may use them); false when the problem is skipped.
+template <typename T> struct RowStore {
+  __device__ __forceinline__ void four(T* dst, size_t i, T a, T b, T c, T d) { st4(dst + i, a, b, c, d); }
+  __device__ __forceinline__ void one(T* dst, size_t i, T a) { dst[i] = a; }
+  __device__ __forceinline__ void flush() {}
+};
+template <typename T, typename EPI>
+__device__ __forceinline__ bool rows_inv_body(const int2 item, const Prob* __restrict__ probs, State* __restrict__ states, int dst_slot, int pcg, EPI& epi) {
   using T2 = typename Vec2<T>::type;
   constexpr int NT = tr_nt(sizeof(T));
   extern __shared__ __align__(16) unsigned char smraw[];
   T2* sm = reinterpret_cast<T2*>(smraw);
   const Prob& pd = probs[item.x];
-  if (tr_skip(states[pd.sidx], pcg)) return;
+  if (tr_skip(states[pd.sidx], pcg)) return false;
   const int N = pd.n, G = pd.row_g, TSg = fpad(N) + 1;
   const int row0 = 2 * item.y * G;
   const bool dct = (pd.transform == TR_DCT);
@@ -1414,24 +1420,126 @@ __device__ __forceinline__ void rows_inv_body(const int2 item, const Prob* __res
       const int p0 = dct ? 2 * xq : 4 * xq, p1 = dct ? N - 1 - 2 * xq : 4 * xq + 1;
       const int p2 = dct ? 2 * xq + 1 : 4 * xq + 2, p3 = dct ? N - 2 - 2 * xq : 4 * xq + 3;
       const T2 v0 = tb[fpad(p0)], v1 = tb[fpad(p1)], v2 = tb[fpad(p2)], v3 = tb[fpad(p3)];
-      T* r = dst + (size_t)ra * N + 4 * xq;
-      if (ra < N) st4(r, v0.x, v1.x, v2.x, v3.x);
-      if (ra + 1 < N) st4(r + N, v0.y, v1.y, v2.y, v3.y);
+      const size_t i = (size_t)ra * N + 4 * xq;
+      if (ra < N) epi.four(dst, i, v0.x, v1.x, v2.x, v3.x);
+      if (ra + 1 < N) epi.four(dst, i + N, v0.y, v1.y, v2.y, v3.y);
+      epi.flush();
     }
-    return;
+    return true;
   }
   for (int e = threadIdx.x; e < G * N; e += NT) {
     const int g = fN.div(e), x = e - g * N;
     const int ra = row0 + 2 * g, rb = ra + 1;
     const T2 v = sm[g * TSg + fpad(dct ? dct_pos(x, N) : x)];
-    if (ra < N) dst[(size_t)ra * N + x] = v.x;
-    if (rb < N) dst[(size_t)rb * N + x] = v.y;
+    if (ra < N) epi.one(dst, (size_t)ra * N + x, v.x);
+    if (rb < N) epi.one(dst, (size_t)rb * N + x, v.y);
+    epi.flush();
   }
+  return true;
 }
 template <typename T>
 __global__ void __launch_bounds__(tr_nt(sizeof(T)), tr_minb(sizeof(T)))
 k_rows_inv(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __restrict__ items, int dst_slot, int pcg) {
-  rows_inv_body<T>(items[blockIdx.x], probs, states, dst_slot, pcg);
+  RowStore<T> st;
+  rows_inv_body<T>(items[blockIdx.x], probs, states, dst_slot, pcg, st);
+}
+
+// ---------------------------------------------------------------------------
+// Algorithm 2: the vector operations of a PCG step that the transform passes
+// can do on the rows they hold (a launch each for the update, the inner
+// product and the start vectors took 16 us of the 52 us of a step at 1024^2).
+// First: the first step, whose vectors are x = 0, res = r (not stored).
+//
+// Forward rows: x += a p, res -= a q on this CTA's rows, then the transform of
+// res.  The CTA's own writes are ordered for its loads by the barrier.
+template <typename T, bool FIRST>
+__global__ void __launch_bounds__(tr_nt(sizeof(T)), tr_minb(sizeof(T)))
+k_rows_fwd_step(const Prob* __restrict__ probs, State* states, const int2* __restrict__ items) {
+  constexpr int NT = tr_nt(sizeof(T));
+  const int2 item = items[blockIdx.x];
+  const Prob& pd = probs[item.x];
+  const State& st = states[item.x];
+  if (tr_skip(st, 1)) return;
+  const int N = pd.n, row0 = 2 * item.y * pd.row_g;
+  const size_t beg = (size_t)row0 * N, end = (size_t)min(N, row0 + 2 * pd.row_g) * N;
+  T* __restrict__ px = static_cast<T*>(pd.buf[SL_PX]);
+  T* __restrict__ res = static_cast<T*>(pd.buf[SL_PRES]);
+  const T* __restrict__ r = static_cast<const T*>(pd.buf[SL_R]);
+  const T* __restrict__ pp = static_cast<const T*>(pd.buf[SL_PP]);
+  const T* __restrict__ pq = static_cast<const T*>(pd.buf[SL_PQ]);
+  const T a = T(st.pa);
+#pragma unroll 4
+  for (size_t i = beg + threadIdx.x; i < end; i += NT) {
+    px[i] = FIRST ? a * pp[i] : px[i] + a * pp[i];
+    res[i] = (FIRST ? r[i] : res[i]) - a * pq[i];
+  }
+  __syncthreads();
+  rows_fwd_body<T>(item, probs, states, SL_PRES, 1);
+}
+
+// Inverse rows: z = M res into PZ, rho = <res, z> (each thread's groups of 8
+// terms in T, FP64 from there on, fixed order), then the PCG scalars; First: rho_0
+// and p = z.
+template <typename T, bool FIRST>
+struct RowDot {
+  const T* res;
+  T* pp;
+  T part;
+  double acc;
+  __device__ __forceinline__ void four(T* dst, size_t i, T a, T b, T c, T d) {
+    T r[4];
+    ld4(res + i, r);
+    st4(dst + i, a, b, c, d);
+    if (FIRST) st4(pp + i, a, b, c, d);
+    part += r[0] * a + r[1] * b + r[2] * c + r[3] * d;
+  }
+  __device__ __forceinline__ void one(T* dst, size_t i, T a) {
+    const T r = res[i];
+    dst[i] = a;
+    if (FIRST) pp[i] = a;
+    part += r * a;
+  }
+  // at most 8 terms (two rows' groups of 4) are summed in T
+  __device__ __forceinline__ void flush() {
+    acc += (double)part;
+    part = T(0);
+  }
+};
+template <typename T, bool FIRST>
+__global__ void __launch_bounds__(tr_nt(sizeof(T)), tr_minb(sizeof(T)))
+k_rows_inv_dot(const Prob* __restrict__ probs, State* states, const int2* __restrict__ items) {
+  constexpr int NT = tr_nt(sizeof(T));
+  __shared__ double red[32];
+  const int2 item = items[blockIdx.x];
+  const Prob& pd = probs[item.x];
+  State& st = states[item.x];
+  RowDot<T, FIRST> dot;
+  dot.res = static_cast<const T*>(pd.buf[FIRST ? SL_R : SL_PRES]);
+  dot.pp = static_cast<T*>(pd.buf[SL_PP]);
+  dot.part = T(0);
+  dot.acc = 0.0;
+  if (!rows_inv_body<T>(item, probs, states, SL_PZ, FIRST ? 0 : 1, dot)) return;
+  double vals[1], tot[1];
+  vals[0] = block_sum<NT>(dot.acc, red);
+  if (last_block_reduce<NT, 1>(pd, st, item.y, pd.nblk_rows, vals, tot, red) && threadIdx.x == 0) {
+    const double rho = tot[0];
+    if (FIRST) {
+      st.prho = rho;
+      st.prho0 = rho;
+      st.psteps = 0;
+      st.pdone = (rho <= 0.0) ? 1 : 0;
+    } else {
+      st.psteps += 1;
+      // relative residual of the symmetric system (psys): sqrt(r_k^T M r_k / r_0^T M r_0)
+      const double rel = sqrt(fmax(rho, 0.0) / st.prho0);
+      if (rel <= pd.pcg_tol || st.psteps >= pd.pcg_max) {
+        st.pdone = 1;
+      } else {
+        st.pbeta = rho / st.prho;
+        st.prho = rho;
+      }
+    }
+  }
 }
 
 
@@ -1841,6 +1949,20 @@ void launch_rows_inv(const Prob* probs, State* states, const int2* items, int ni
   if (nitems > 0) k_rows_inv<T><<<nitems, tr_nt(sizeof(T)), smem, s>>>(probs, states, items, dst, pcg);
 }
 template <typename T>
+void launch_rows_fwd_step(const Prob* probs, State* states, const int2* items, int nitems, int first,
+                          size_t smem, cudaStream_t s) {
+  if (nitems <= 0) return;
+  if (first) k_rows_fwd_step<T, true><<<nitems, tr_nt(sizeof(T)), smem, s>>>(probs, states, items);
+  else k_rows_fwd_step<T, false><<<nitems, tr_nt(sizeof(T)), smem, s>>>(probs, states, items);
+}
+template <typename T>
+void launch_rows_inv_dot(const Prob* probs, State* states, const int2* items, int nitems, int first,
+                         size_t smem, cudaStream_t s) {
+  if (nitems <= 0) return;
+  if (first) k_rows_inv_dot<T, true><<<nitems, tr_nt(sizeof(T)), smem, s>>>(probs, states, items);
+  else k_rows_inv_dot<T, false><<<nitems, tr_nt(sizeof(T)), smem, s>>>(probs, states, items);
+}
+template <typename T>
 void launch_ar_rows(const Prob* probs, State* states, const int2* items, int nitems, int slot,
                     int inv, int pcg, size_t smem, cudaStream_t s) {
   if (nitems <= 0) return;
@@ -1882,7 +2004,9 @@ cudaError_t fft_set_smem() {
     if (e != cudaSuccess) return e;
   }
   for (const void* f : {(const void*)k_ar_rows<T, false>, (const void*)k_ar_rows<T, true>,
-                        (const void*)k_ar_cols<T, COL_FUSED>, (const void*)k_ar_cols<T, COL_OP>}) {
+                        (const void*)k_ar_cols<T, COL_FUSED>, (const void*)k_ar_cols<T, COL_OP>,
+                        (const void*)k_rows_fwd_step<T, false>, (const void*)k_rows_fwd_step<T, true>,
+                        (const void*)k_rows_inv_dot<T, false>, (const void*)k_rows_inv_dot<T, true>}) {
     e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
   }
@@ -1894,6 +2018,8 @@ cudaError_t fft_set_smem() {
   template void launch_cols<T>(const Prob*, State*, const int2*, int, int, int, double, int, size_t, cudaStream_t); \
   template void launch_rows_inv<T>(const Prob*, State*, const int2*, int, int, int, size_t, cudaStream_t); \
   template void launch_spec<T>(const Prob*, State*, const int2*, int, int, cudaStream_t);         \
+  template void launch_rows_fwd_step<T>(const Prob*, State*, const int2*, int, int, size_t, cudaStream_t); \
+  template void launch_rows_inv_dot<T>(const Prob*, State*, const int2*, int, int, size_t, cudaStream_t); \
   template void launch_ar_rows<T>(const Prob*, State*, const int2*, int, int, int, int, size_t, cudaStream_t); \
   template void launch_ar_cols<T>(const Prob*, State*, const int2*, int, int, int, double, int, size_t, cudaStream_t); \
   template cudaError_t fft_set_smem<T>();

@@ -153,7 +153,7 @@ k_persist(const Prob* __restrict__ probs, State* __restrict__ states, int nprob,
           for (int u = blockIdx.x; u < cnt; u += gridDim.x) { cols_body<T, COL_NS_INV>(it[u], probs, states, 0, 0.0, 0); __syncthreads(); }
           break;
         case PS_ROWS_INV:
-          for (int u = blockIdx.x; u < cnt; u += gridDim.x) { rows_inv_body<T>(it[u], probs, states, SL_T, 0); __syncthreads(); }
+          for (int u = blockIdx.x; u < cnt; u += gridDim.x) { RowStore<T> rs; rows_inv_body<T>(it[u], probs, states, SL_T, 0, rs); __syncthreads(); }
           break;
         case PS_BALANCE:
           for (int u = blockIdx.x; u < cnt; u += gridDim.x) { balance_body<T>(it[u], probs, states); __syncthreads(); }

@@ -526,74 +526,37 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(VEC_THREADS)
 k_vec(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __restrict__ items,
       int pcg) {
-  __shared__ double red[32];
   const int2 item = items[blockIdx.x];
   const Prob& pd = probs[item.x];
   State& st = states[item.x];
   if (st.stopped) return;
-  // INIT re-arms the PCG; FINISH always copies the solution out
-  if (pcg && st.pdone && MODE != VEC_PCG_INIT && MODE != VEC_PCG_FINISH) return;
-  if (MODE == VEC_PCG_INIT && item.y == 0 && threadIdx.x == 0) st.pdone = 0;
+  // FINISH always copies the solution out
+  if (pcg && st.pdone && MODE != VEC_PCG_FINISH) return;
   const int n = pd.n;
   const size_t nn = (size_t)n * n;
   const size_t chunk = (size_t)VEC_THREADS * VEC_PER_THREAD;
   const size_t beg = (size_t)item.y * chunk;
   const size_t end = beg + chunk < nn ? beg + chunk : nn;
-  T* U = static_cast<T*>(pd.buf[SL_U]);
-  T* PX = static_cast<T*>(pd.buf[SL_PX]);
-  T* PRES = static_cast<T*>(pd.buf[SL_PRES]);
-  T* PP = static_cast<T*>(pd.buf[SL_PP]);
-  T* PQ = static_cast<T*>(pd.buf[SL_PQ]);
-  T* PZ = static_cast<T*>(pd.buf[SL_PZ]);
-  double lacc = 0.0;
-  T tacc = T(0);
-  for (size_t i = beg + threadIdx.x; i < end; i += VEC_THREADS) {
+  // (distinct buffers: a thread's loads go out together)
+  T* __restrict__ U = static_cast<T*>(pd.buf[SL_U]);
+  T* __restrict__ PP = static_cast<T*>(pd.buf[SL_PP]);
+  T* __restrict__ TT = static_cast<T*>(pd.buf[SL_T]);
+  const T* __restrict__ V = static_cast<const T*>(pd.buf[SL_V]);
+  const T* __restrict__ PX = static_cast<const T*>(pd.buf[SL_PX]);
+  const T* __restrict__ PZ = static_cast<const T*>(pd.buf[SL_PZ]);
+  const T beta = MODE == VEC_PCG_PUPD ? T(st.pbeta) : T(0);
+  const bool any = MODE == VEC_PCG_FINISH && st.psteps > 0;
+#pragma unroll
+  for (int k = 0; k < VEC_PER_THREAD; ++k) {
+    const size_t i = beg + threadIdx.x + (size_t)k * VEC_THREADS;
+    if (i >= end) break;
     if (MODE == VEC_FOLD) {
       const int a = (int)(i / n), b = (int)(i - (size_t)a * n);
-      U[i] = fold_fetch<T>(pd, static_cast<const T*>(pd.buf[SL_V]), a, b);
-    } else if (MODE == VEC_PCG_INIT) {
-      PX[i] = T(0);
-      PRES[i] = static_cast<const T*>(pd.buf[SL_R])[i];
-    } else if (MODE == VEC_PCG_RHO0) {
-      const T zv = PZ[i];
-      tacc += PRES[i] * zv;
-      PP[i] = zv;
-    } else if (MODE == VEC_PCG_AXPY) {
-      const T a = T(st.pa);
-      PX[i] += a * PP[i];
-      PRES[i] -= a * PQ[i];
-    } else if (MODE == VEC_PCG_RHO) {
-      tacc += PRES[i] * PZ[i];
+      U[i] = fold_fetch<T>(pd, V, a, b);
     } else if (MODE == VEC_PCG_PUPD) {
-      PP[i] = PZ[i] + T(st.pbeta) * PP[i];
+      PP[i] = PZ[i] + beta * PP[i];
     } else if (MODE == VEC_PCG_FINISH) {
-      static_cast<T*>(pd.buf[SL_T])[i] = PX[i];
-    }
-  }
-  if (MODE == VEC_PCG_RHO0 || MODE == VEC_PCG_RHO) {
-    lacc = (double)tacc;
-    const double bs = block_sum<VEC_THREADS>(lacc, red);
-    double tot[1];
-    const double vals[1] = {bs};
-    if (last_block_reduce<VEC_THREADS, 1>(pd, st, item.y, pd.nblk_vec, vals, tot, red) &&
-        threadIdx.x == 0) {
-      const double rho = tot[0];
-      if (MODE == VEC_PCG_RHO0) {
-        st.prho = rho;
-        st.prho0 = rho;
-        st.psteps = 0;
-        st.pdone = (rho <= 0.0) ? 1 : 0;
-      } else {
-        st.psteps += 1;
-        // relative residual of the symmetric system (psys): sqrt(r_k^T M r_k / r_0^T M r_0)
-        const double rel = sqrt(fmax(rho, 0.0) / st.prho0);
-        if (rel <= pd.pcg_tol || st.psteps >= pd.pcg_max) {
-          st.pdone = 1;
-        } else {
-          st.pbeta = rho / st.prho;
-          st.prho = rho;
-        }
-      }
+      TT[i] = any ? PX[i] : T(0);
     }
   }
   if (MODE == VEC_PCG_FINISH && item.y == 0 && threadIdx.x == 0) {
@@ -809,10 +772,6 @@ void launch_vec(int mode, const Prob* probs, State* states, const int2* items, i
   dim3 g(nitems), b(VEC_THREADS);
   switch (mode) {
     case VEC_FOLD: k_vec<T, VEC_FOLD><<<g, b, 0, s>>>(probs, states, items, pcg); break;
-    case VEC_PCG_INIT: k_vec<T, VEC_PCG_INIT><<<g, b, 0, s>>>(probs, states, items, pcg); break;
-    case VEC_PCG_RHO0: k_vec<T, VEC_PCG_RHO0><<<g, b, 0, s>>>(probs, states, items, pcg); break;
-    case VEC_PCG_AXPY: k_vec<T, VEC_PCG_AXPY><<<g, b, 0, s>>>(probs, states, items, pcg); break;
-    case VEC_PCG_RHO: k_vec<T, VEC_PCG_RHO><<<g, b, 0, s>>>(probs, states, items, pcg); break;
     case VEC_PCG_PUPD: k_vec<T, VEC_PCG_PUPD><<<g, b, 0, s>>>(probs, states, items, pcg); break;
     default: k_vec<T, VEC_PCG_FINISH><<<g, b, 0, s>>>(probs, states, items, pcg); break;
   }

@@ -371,21 +371,18 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
     // a4': Algorithm 2, PCG on (A A^T + alpha I) t = r preconditioned by (CC^T + alpha I)^{-1}
     if (L.any_krylov) {
       const int maxs = L.pcg_max;
-      launch_vec<T>(VEC_PCG_INIT, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
-      launch_rows_fwd<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PRES, 1, B->smem_fft, s);
-      launch_cols<T>(P, S, L.cols_kry.dev, L.cols_kry.count, COL_FUSED, 1, 0.0, 0, B->smem_fft, s);
-      launch_rows_inv<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PZ, 1, B->smem_fft, s);
-      launch_vec<T>(VEC_PCG_RHO0, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
+      // (the first M r ignores pdone of the previous solve and sets it)
+      launch_rows_fwd<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_R, 0, B->smem_fft, s);
+      launch_cols<T>(P, S, L.cols_kry.dev, L.cols_kry.count, COL_FUSED, 0, 0.0, 0, B->smem_fft, s);
+      launch_rows_inv_dot<T>(P, S, L.rows_kry.dev, L.rows_kry.count, 1, B->smem_fft, s);
       for (int k = 0; k < maxs; ++k) {
         launch_stencil<T>(ST_CORR, P, S, L.corr_kry.dev, L.corr_kry.count, SL_PP, SL_V, SL_V, 1, B->st_rows, B->smem_stencil, s);
         launch_vec<T>(VEC_FOLD, P, S, L.vec_kry_bc.dev, L.vec_kry_bc.count, 1, s);
         launch_stencil<T>(ST_FWD_PCGQ, P, S, L.blur_kry.dev, L.blur_kry.count, -1, SL_PQ, SL_PP, 1, B->st_rows, B->smem_stencil, s);
-        launch_vec<T>(VEC_PCG_AXPY, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
-        launch_rows_fwd<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PRES, 1, B->smem_fft, s);
+        launch_rows_fwd_step<T>(P, S, L.rows_kry.dev, L.rows_kry.count, k == 0, B->smem_fft, s);
         launch_cols<T>(P, S, L.cols_kry.dev, L.cols_kry.count, COL_FUSED, 1, 0.0, 0, B->smem_fft, s);
-        launch_rows_inv<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PZ, 1, B->smem_fft, s);
-        launch_vec<T>(VEC_PCG_RHO, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
-        launch_vec<T>(VEC_PCG_PUPD, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
+        launch_rows_inv_dot<T>(P, S, L.rows_kry.dev, L.rows_kry.count, 0, B->smem_fft, s);
+        if (k + 1 < maxs) launch_vec<T>(VEC_PCG_PUPD, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
       }
       launch_vec<T>(VEC_PCG_FINISH, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
     }

@@ -30,12 +30,8 @@ void launch_balance(const Prob* probs, State* states, const int2* items, int nit
 // vector kernels (k_stencil.cu)
 enum {
   VEC_FOLD = 0,       // U = BC fold of V
-  VEC_PCG_INIT = 1,   // PX = 0, PRES = R
-  VEC_PCG_RHO0 = 2,   // rho0 = <PRES, PZ>, PP = PZ
-  VEC_PCG_AXPY = 3,   // PX += a PP, PRES -= a PQ
-  VEC_PCG_RHO = 4,    // rho = <PRES, PZ>, convergence test
-  VEC_PCG_PUPD = 5,   // PP = PZ + beta PP
-  VEC_PCG_FINISH = 6  // T = PX
+  VEC_PCG_PUPD = 1,   // PP = PZ + beta PP
+  VEC_PCG_FINISH = 2  // T = PX (0 when no step was taken), beta_n recorded
 };
 // column-pass modes (k_fft.cu)
 enum {
@@ -80,6 +76,15 @@ void launch_rows_inv(const Prob* probs, State* states, const int2* items, int ni
 template <typename T>
 void launch_spec(const Prob* probs, State* states, const int2* items, int nitems, int cand,
                  cudaStream_t s);
+// Algorithm 2 (k_fft.cu): the row passes of a PCG step with its vector
+// operations (x and res updated before the forward transform; <res, M res> and
+// the PCG scalars after the inverse one); first: the first ones of a solve
+template <typename T>
+void launch_rows_fwd_step(const Prob* probs, State* states, const int2* items, int nitems, int first,
+                          size_t smem, cudaStream_t s);
+template <typename T>
+void launch_rows_inv_dot(const Prob* probs, State* states, const int2* items, int nitems, int first,
+                         size_t smem, cudaStream_t s);
 // antireflective transform passes (k_fft.cu): rows (inv = 0: T^{-1} of
 // buf[slot] into S; inv = 1: T of S into buf[slot]) and the column pass
 // (T^{-1}, weight, T; mode COL_FUSED or COL_OP)

@@ -419,3 +419,31 @@ def test_transform_lengths(M, dtype, transform, n):
         ref = pre.inv(r, 0.05) if which == "inv" else pre.tikh(r, 0.05)
         assert rel_err(ctx.precond(r, 0.05, which), ref) <= (1e-11 if dtype == "f64" else 2e-5)
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("bc,transform,psf,n", [("rect", "dft", "motion7", 45), ("zero", "dft", "motion7", 97),
+                                                ("reflective", "dct", "gauss9", 64), ("periodic", "dft", "disk2", 130)])
+@pytest.mark.parametrize("tol,cap", [(1e-3, 1), (1e-3, 5), (1e-9, 7)])
+def test_pcg_steps_in_the_row_passes(M, dtype, bc, transform, psf, n, tol, cap):
+    """Algorithm 2 with its vector operations inside the row passes: one step,
+    the tolerance stop and a cap beyond it, odd sizes (element path) and sizes
+    that are multiples of 4, several iterations (the start vectors are formed
+    anew): step counts and iterates against the oracle.  (FP32 residuals do not
+    resolve 1e-9: FP64 only.)"""
+    if dtype == "f32" and tol < 1e-6:
+        pytest.skip("below FP32 resolution")
+    h = PSFS[psf]
+    f = I.true_image(n + h.shape[0] - 1, n)
+    g, delta = I.observe(f, h, 0.01, n)
+    alpha, iters = 0.05, 3
+    ctx = M.Context(h, n, bc, "krylov", dtype=dtype, alpha=alpha, levels=1, max_iter=iters, stop=False,
+                    transform=transform, pcg_tol=tol, pcg_max=cap)
+    ctx.set_data(g, delta)
+    ctx.run(iters)
+    out, (res, _, be) = ctx.result(), ctx.history()
+    ctx.close()
+    ref = O.mlba(g.astype(np.float32 if dtype == "f32" else np.float64).astype(np.float64), h, delta, bc, "krylov",
+                 10 / 255, alpha, 1, iters, stop=False, transform=transform, pcg_tol=tol, pcg_max=cap)
+    assert list(be) == ref["betas"]
+    assert rel_err(out, ref["f"]) <= (1e-9 if dtype == "f64" else 1e-4)
