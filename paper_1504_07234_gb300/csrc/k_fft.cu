@@ -304,7 +304,7 @@ __device__ __noinline__ void fft_pass_any(int G, int N, int TSg, int Ns, int R,
 
 // G transforms of length n held in the dynamic shared memory of the block
 // (transform g at g * (fpad(n) + 1)); all threads of the block call this
-// The passes run grouped by radix (16s, one 8/4/2, 3s, 5s) in straight-line
+// The passes run grouped by radix (16s or 4s, one 8/4/2, 3s, 5s) in straight-line
 // regions rather than as one loop over a radix switch: the compiler then
 // keeps each region's butterflies in registers (the switch form spilled).
 template <typename T2, bool INV>
@@ -315,6 +315,8 @@ __device__ __noinline__ void fft_smem(int G, const Prob& pd) {
   const int n16 = pd.nr16, r2 = pd.r2, n3 = pd.nr3, n5 = pd.nr5;
   int Ns = 1;
   for (int s = 0; s < n16; ++s) { fft_pass<T2, 16, INV>(G, N, TSg, Ns, tw); Ns *= 16; }
+  if constexpr (sizeof(T2) == 16)     // (radix-4 plans are FP64 only)
+    for (int s = 0; s < pd.nr4; ++s) { fft_pass<T2, 4, INV>(G, N, TSg, Ns, tw); Ns *= 4; }
   if (r2 == 8) { fft_pass<T2, 8, INV>(G, N, TSg, Ns, tw); Ns *= 8; }
   if (r2 == 4) { fft_pass<T2, 4, INV>(G, N, TSg, Ns, tw); Ns *= 4; }
   if (r2 == 2) { fft_pass<T2, 2, INV>(G, N, TSg, Ns, tw); Ns *= 2; }
@@ -423,9 +425,9 @@ __device__ __forceinline__ bool tr_skip(const State& st, int pcg) {
 // (FP32: 2 of the 3 in the step, FP64: 3 of 5 on the workloads' spectra)
 constexpr int NS_CAND = 8;
 constexpr double NS_CAND_STEP = 2.0;
-constexpr int NS_NT = SPEC_THREADS, NS_PT = SPEC_PER_THREAD;
+constexpr int NS_NT = SPEC_THREADS;        // (Prob::spec_pt values per thread)
 constexpr int NS_B = 8;                    // elements per thread with loads in flight together
-static_assert(NS_PT % NS_B == 0, "spectrum pass batches");
+static_assert(SPEC_PER_THREAD % NS_B == 0 && SPEC_PER_THREAD_MIN % NS_B == 0, "spectrum pass batches");
 static_assert(SPEC_SUMS == 2 * NS_CAND + 1, "partial buffer sized for the bracketing pass");
 
 __host__ __device__ constexpr double ns_tol(int elem_bytes) { return elem_bytes == 8 ? 1e-10 : 1e-5; }
@@ -433,7 +435,7 @@ __host__ __device__ constexpr double ns_tol(int elem_bytes) { return elem_bytes 
 // the step's cube) is far below tol; FP64 takes only steps below tol
 __host__ __device__ constexpr double ns_tol3(int elem_bytes) { return elem_bytes == 8 ? 1e-10 : 2.7e-3; }
 
-// element e (< NS_NT * NS_PT) of spectrum block `blk`, enumerated along the
+// element e (< NS_NT * spec_pt) of spectrum block `blk`, enumerated along the
 // column-blocked layout (contiguous reads): weighted power and |lambda|^2 in
 // T precision; false past the end or on padding
 template <typename T>
@@ -442,7 +444,7 @@ __device__ __forceinline__ bool spec_elem(const Prob& pd, int blk, int e, T& pw,
   const int N = pd.n, cb = pd.cb;
   const bool dct = (pd.transform == TR_DCT);
   const int W = dct ? N : pd.half;
-  const int L = blk * (NS_NT * NS_PT) + e;      // < 2^31: one spectrum holds < 2^25 elements
+  const int L = blk * (NS_NT * pd.spec_pt) + e;      // < 2^31: one spectrum holds < 2^25 elements
   const int blksz = N * cb;
   const int b = L / blksz;
   const int rem = L - b * blksz;
@@ -1565,7 +1567,7 @@ k_spec_cand(const Prob* __restrict__ probs, State* __restrict__ states, const in
   for (int j = 0; j < NS_CAND; ++j) { ci[j] = s_ci[j]; cF[j] = 0.f; cH[j] = 0.f; }
   T sP = T(0);
 #pragma unroll 1
-  for (int q0 = 0; q0 < NS_PT; q0 += NS_B) {
+  for (int q0 = 0; q0 < pd.spec_pt; q0 += NS_B) {
     T pw[NS_B], sg[NS_B];
     bool ok[NS_B];
 #pragma unroll
@@ -1573,7 +1575,7 @@ k_spec_cand(const Prob* __restrict__ probs, State* __restrict__ states, const in
       ok[q] = spec_elem<T>(pd, item.y, threadIdx.x + (q0 + q) * NS_NT, pw[q], sg[q]);
 #pragma unroll
     for (int q = 0; q < NS_B; ++q) {
-      const int L = item.y * (NS_NT * NS_PT) + threadIdx.x + (q0 + q) * NS_NT;
+      const int L = item.y * (NS_NT * pd.spec_pt) + threadIdx.x + (q0 + q) * NS_NT;
       if (L < pd.nblk_cols * pd.n * pd.cb) static_cast<T*>(pd.pw)[L] = ok[q] ? pw[q] : T(0);
       if (!ok[q]) continue;
       sP += pw[q];
@@ -1604,10 +1606,10 @@ __device__ __forceinline__ void spec_body(const int2 item, const Prob* __restric
   const int nel = pd.nblk_cols * pd.n * pd.cb;
   const T* P = static_cast<const T*>(pd.pw);
   const T* Sg = static_cast<const T*>(pd.w);
-  int L = item.y * (NS_NT * NS_PT) + threadIdx.x;
+  int L = item.y * (NS_NT * pd.spec_pt) + threadIdx.x;
   T sP = T(0), sF = T(0), sG1 = T(0), sG2 = T(0);
 #pragma unroll 1
-  for (int q0 = 0; q0 < NS_PT; q0 += NS_B) {
+  for (int q0 = 0; q0 < pd.spec_pt; q0 += NS_B) {
     T pw[NS_B], sg[NS_B];
 #pragma unroll
     for (int q = 0; q < NS_B; ++q) {

@@ -176,14 +176,35 @@ int vec_blocks(size_t elems) {
   return (int)((elems + VEC_THREADS * VEC_PER_THREAD - 1) / (VEC_THREADS * VEC_PER_THREAD));
 }
 
-// Radix passes of the length-n FFT: as many radix-16 passes as divide n, then
-// at most one of 8, 4 or 2 for the rest of the power of two, then 3s and 5s,
-// then every prime factor above 5 as a direct-sum pass (any n factors within
-// MAX_STAGES passes: n <= 4096 has at most 12 prime factors).
-bool fft_plan(Prob& pd) {
+// Spectral values per thread of an alpha_n pass: 32, or 8 (a quarter of the chain
+// of loads and sums) while the launch has at most one CTA per SM then.  A step
+// with 32 / 8: 256^2 FP32 83 / 81 us, 300^2 FP64 166 / 112; the 64-problem batch
+// 1.020 / 1.024 ms, 4096^2 1.09 / 1.16.
+void spec_geometry(std::vector<HostProb>& v) {
+  size_t ns = 0;
+  for (const HostProb& h : v) if (h.pd.ns) ns += spec_elems(h.pd);
+  for (HostProb& h : v) {
+    Prob& pd = h.pd;
+    const size_t tot = pd.ns ? ns : spec_elems(pd);       // (not 4-NS: the operator entry point)
+    pd.spec_pt = tot <= (size_t)152 * SPEC_THREADS * SPEC_PER_THREAD_MIN ? SPEC_PER_THREAD_MIN : SPEC_PER_THREAD;
+    pd.nblk_spec = (int)((spec_elems(pd) + SPEC_THREADS * pd.spec_pt - 1) / (SPEC_THREADS * pd.spec_pt));
+  }
+}
+
+// Radix passes of the length-n FFT: as many radix-16 passes (thin: radix-4) as
+// divide n, then at most one of 8, 4 or 2 for the rest of the power of two, then
+// 3s and 5s, then every prime factor above 5 as a direct-sum pass (any n factors
+// within MAX_STAGES passes: n <= 4096 has at most 12 prime factors).
+// thin: FP64 CTAs that hold few values.  A radix-16 pass of one 256-point
+// transform occupies half a warp, whose 200 FP64 instructions take the
+// scheduler's pipe 64 cycles each; radix 4 spreads them over two warps per pass
+// (a step at 64^2: 87 -> 75 us, at 256^2 with L = 4: 286 -> 251).  In FP32 the
+// additional passes cost more than they spread (256^2: +3 %, 1024^2: +4 %).
+bool fft_plan(Prob& pd, bool thin) {
   int m = pd.nfft, s = 0;
-  pd.nr16 = pd.r2 = pd.nr3 = pd.nr5 = pd.nrany = 0;
-  while (m % 16 == 0 && s < MAX_STAGES) { pd.radix[s++] = 16; m /= 16; ++pd.nr16; }
+  pd.nr16 = pd.nr4 = pd.r2 = pd.nr3 = pd.nr5 = pd.nrany = 0;
+  if (!thin) while (m % 16 == 0 && s < MAX_STAGES) { pd.radix[s++] = 16; m /= 16; ++pd.nr16; }
+  if (thin) while (m % 4 == 0 && s < MAX_STAGES) { pd.radix[s++] = 4; m /= 4; ++pd.nr4; }
   for (int r : {8, 4, 2})
     if (m % r == 0 && s < MAX_STAGES) { pd.radix[s++] = r; m /= r; pd.r2 = r; break; }
   while (m % 3 == 0 && s < MAX_STAGES) { pd.radix[s++] = 3; m /= 3; ++pd.nr3; }
@@ -666,7 +687,8 @@ int transform_fill(const std::vector<HostProb>& v, int launches) {
 // pd.nfft): transforms per CTA and the column blocking of the spectrum.
 // fill: complex values a CTA should hold (at least one transform, at most
 // TR_CAP).
-void transform_geometry(Prob& pd, int fill) {
+constexpr int TR_THIN = 1024;   // values per CTA up to which the plan is thin (fft_plan)
+void transform_geometry(Prob& pd, int fill, bool f64) {
   const int n = pd.n;
   const int cap = std::max(1, std::min(fill, TR_CAP) / std::max(pd.nfft, n));      // transforms per CTA
   const int pairs = (n + 1) / 2;
@@ -689,8 +711,8 @@ void transform_geometry(Prob& pd, int fill) {
     pd.cb = dct ? 2 * pd.col_g : pd.col_g;
     pd.nblk_cols = ((dct ? n : pd.half) + pd.cb - 1) / pd.cb;
   }
-  pd.nblk_spec = (int)((spec_elems(pd) + SPEC_THREADS * SPEC_PER_THREAD - 1) /
-                       (SPEC_THREADS * SPEC_PER_THREAD));
+  // the plan for CTAs of this size
+  if (pd.transform != TR_NONE) fft_plan(pd, f64 && std::max(pd.row_g, pd.col_g) * pd.nfft <= TR_THIN);
 }
 
 // smallest 2^a 3^b 5^c >= m (fast radix passes for the convolution size)
@@ -717,7 +739,7 @@ bool setup_conv_entry(const HostProb& own, int owner, int adj, HostProb& h) {
   pd.levels = op.levels; pd.nbands = op.nbands;
   pd.alpha = 1.0; pd.max_iter = -1; pd.sidx = owner;
   pd.nfft = M;
-  if (!fft_plan(pd)) return false;
+  if (!fft_plan(pd, false)) return false;
   pd.nblk_vec = vec_blocks((size_t)M * M);
   const int p = op.p;
   h.psf_pre.resize((size_t)p * p);
@@ -796,7 +818,7 @@ int setup_problem(const mlba_problem& in, const mlba_opts& o, HostProb& h) {
   if (pd.transform == TR_AR && (!ar_bc || ns || in.precond == MLBA_P_KRYLOV)) return MLBA_E_INVAL;
   pd.nfft = (pd.transform == TR_AR) ? 2 * (n - 1) : n;   // DST-I of n - 2 as a DFT of 2(n - 1)
   if (pd.transform != TR_NONE) {
-    if (!fft_plan(pd)) return MLBA_E_UNSUPPORTED;
+    if (!fft_plan(pd, false)) return MLBA_E_UNSUPPORTED;
     // one transform must fit the per-CTA value budget of the smem FFT
     if (pd.nfft > TR_CAP || (pd.transform == TR_AR && n < 3)) return MLBA_E_UNSUPPORTED;
   }
@@ -1274,8 +1296,9 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
   // column passes have about two CTAs per SM
   {
     const int fill = transform_fill(B->hp, 1), ffill = transform_fill(B->fc, 2);   // (forward, adjoint entries)
-    for (HostProb& h : B->hp) transform_geometry(h.pd, fill);
-    for (HostProb& h : B->fc) transform_geometry(h.pd, ffill);
+    for (HostProb& h : B->hp) transform_geometry(h.pd, fill, o.dtype == MLBA_F64);
+    spec_geometry(B->hp);
+    for (HostProb& h : B->fc) transform_geometry(h.pd, ffill, o.dtype == MLBA_F64);
   }
   if (o.stream) { B->stream = (cudaStream_t)o.stream; }
   else {

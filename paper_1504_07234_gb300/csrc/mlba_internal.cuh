@@ -54,11 +54,12 @@ struct Prob {
   int nfft;          // FFT length: n (DFT, DCT) or 2(n - 1) (antireflective transform)
   int nstage;        // FFT plan of length nfft
   int radix[MAX_STAGES];
-  int nr16, r2, nr3, nr5;   // the same plan: radix-16 passes, one 8/4/2 pass, 3s, 5s,
+  int nr16, nr4, r2, nr3, nr5;   // the same plan: radix-16 or radix-4 passes, one 8/4/2 pass, 3s, 5s,
   int nrany;                // then the prime factors above 5 (direct-sum passes)
   // per-list block counts (reductions need them)
   int nblk_blur, nblk_corr, nblk_rows, nblk_cols, nblk_spec, nblk_vec;
   int row_g, col_g;  // transforms per CTA in the row / column passes
+  int spec_pt;       // 4-NS: spectral values per thread of an alpha_n pass
   int cb;            // spectrum column block: col_g complex columns (DFT) or
                      // 2 col_g real columns (DCT); block j holds columns
                      // [j cb, (j+1) cb) as n rows of cb contiguous elements;

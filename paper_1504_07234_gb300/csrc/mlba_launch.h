@@ -55,7 +55,7 @@ constexpr int FRAME_SHAPES = 8;      // tile shapes of the L <= 2 framelet kerne
 constexpr int LP_THREADS = 256, LP_PER = 4;   // low-pass chain kernel (L >= 3)
 constexpr int FRAME_SECTIONS = 2 + 4;         // fold, low-pass, up to four levels
 constexpr int SPEC_THREADS = 256;    // alpha_n solve (k_fft.cu)
-constexpr int SPEC_PER_THREAD = 32;
+constexpr int SPEC_PER_THREAD = 32, SPEC_PER_THREAD_MIN = 8;   // spectral values per thread of a pass
 constexpr int SPEC_SUMS = 17;        // block sums of the bracketing pass (2 x 8 candidates + 1)
 
 template <typename T>

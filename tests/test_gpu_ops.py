@@ -447,3 +447,22 @@ def test_pcg_steps_in_the_row_passes(M, dtype, bc, transform, psf, n, tol, cap):
                  10 / 255, alpha, 1, iters, stop=False, transform=transform, pcg_tol=tol, pcg_max=cap)
     assert list(be) == ref["betas"]
     assert rel_err(out, ref["f"]) <= (1e-9 if dtype == "f64" else 1e-4)
+
+
+@pytest.mark.parametrize("n", [12, 64, 96, 250, 256, 320])
+@pytest.mark.parametrize("count", [1, 3])
+def test_fp64_thin_and_full_radix_plans(M, n, count):
+    """FP64 transforms whose CTAs hold few values run radix-4 passes, fuller ones
+    radix-16 (a batch of three takes the plan of its own CTA size): both against
+    the oracle's preconditioned first iterate, with the alpha_n solve whose passes
+    take 8 or 32 values per thread."""
+    h = I.psf_disk(2) if n > 12 else I.psf_gaussian(0.7, 3)
+    f = I.true_image(n + h.shape[0] - 1, n)
+    g, delta = I.observe(f, h, 0.02, n)
+    descs = [dict(psf=h, g=g, delta=delta, bc="reflective", precond="tikh_ns", transform="dct")] * count
+    b = M.Batch(descs, dtype="f64", levels=1, stop=False, max_iter=4)
+    b.iterate(2)
+    ref = O.mlba(g, h, delta, "reflective", "tikh_ns", 10 / 255, 0.05, 1, 2, stop=False, transform="dct")
+    for i in range(count):
+        assert rel_err(b.result(i), ref["f"]) <= 1e-9
+    b.close()
