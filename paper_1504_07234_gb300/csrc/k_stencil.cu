@@ -182,7 +182,7 @@ __host__ __device__ constexpr size_t st_smem(int R, int p, int sep, int nrw, int
   const int nw = sep ? 2 * p : nrw, we = elem == 4 ? 2 : 1;
   const size_t in = (size_t)RY * st_pitch(RX, elem), tmp = sep ? (size_t)4 * R * st_tpitch(RX, elem) : 0;
   return (((size_t)nw * we + 3) / 4 * 4 + (in > tmp ? in : tmp)) * elem + (sep ? 0 : (size_t)nruns * 16) +
-         (size_t)((RY + RX + 3) / 4 * 4) * 4;
+         (size_t)((2 * (RY + RX) + 3) / 4 * 4) * 4;
 }
 
 #ifndef MLBA_BODIES_ONLY
@@ -244,8 +244,8 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   TW* s_w = reinterpret_cast<TW*>(smraw);
   constexpr int WE = (int)(sizeof(TW) / sizeof(T));
   int4* s_runs = reinterpret_cast<int4*>(reinterpret_cast<T*>(smraw) + ((nw * WE + 3) & ~3));
-  int* s_map = reinterpret_cast<int*>(s_runs + (sep ? 0 : pd.nruns));     // RY + RX entries
-  T* s_in = reinterpret_cast<T*>(s_map + ((RY + RX + 3) & ~3));
+  int* s_map = reinterpret_cast<int*>(s_runs + (sep ? 0 : pd.nruns));     // 2 (RY + RX) entries
+  T* s_in = reinterpret_cast<T*>(s_map + ((2 * (RY + RX) + 3) & ~3));
 
   // src_slot < 0: the per-problem default operand (t, or r for P = I, in the
   // correlation; A^T p for the PCG product: V for rectangular A, U otherwise)
@@ -298,26 +298,43 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
     const int c16 = 16 / (int)sizeof(T);
     const int ce = !colin ? 0 : (pitch % c16 == 0 ? c16 : (sizeof(T) == 4 && pitch % 2 == 0 ? 2 : 0));
     if (ar_out) {
-      // 1-D antireflection of an extended index: up to two (index, weight)
-      // terms; 0 terms past the reach of any output of the image
-      auto ar_terms = [&](int e, int (&ix)[2], T (&wt)[2]) -> int {
-        if (e >= 0 && e < n) { ix[0] = e; wt[0] = T(1); return 1; }
+      // 1-D antireflection of an extended index: the pixel itself, or 2 x the
+      // edge minus the mirror pixel; nothing past the reach of any output of the
+      // image.  Tables of (first, second or -1) pixel per tile row and column.
+      auto terms = [&](int e, int* first, int* second) {
+        *first = e; *second = -1;
+        if (e >= 0 && e < n) return;
         const int k = e < 0 ? -e : e - (n - 1);          // distance outside the edge
-        if (k > n - 1) return 0;
-        ix[0] = e < 0 ? 0 : n - 1;
-        ix[1] = e < 0 ? k : n - 1 - k;
-        wt[0] = T(2); wt[1] = T(-1);
-        return 2;
+        *first = k > n - 1 ? -1 : (e < 0 ? 0 : n - 1);
+        *second = k > n - 1 ? -1 : (e < 0 ? k : n - 1 - k);
       };
+      int *r0 = s_map, *q0 = s_map + RY, *r1 = s_map + RY + RX, *q1 = r1 + RY;
+      for (int k = tid; k < RY; k += NT) terms(oy0 + k, r0 + k, r1 + k);
+      for (int k = tid; k < RX; k += NT) terms(ox0 + k, q0 + k, q1 + k);
+      blk.sync();
+      const FastDiv frx(RX);
       for (int idx = tid; idx < RY * RX; idx += NT) {
-        const int ry = idx / RX, rx = idx - ry * RX;
-        int iy[2], ix[2];
-        T wy[2], wx[2];
-        const int ny = ar_terms(oy0 + ry, iy, wy), nx = ar_terms(ox0 + rx, ix, wx);
-        T v = T(0);
-        for (int a = 0; a < ny; ++a)
-          for (int b = 0; b < nx; ++b) v += wy[a] * wx[b] * src[(size_t)iy[a] * n + ix[b]];
-        s_in[ry * RP + rx] = v;
+        const int ry = frx.div(idx), rx = idx - ry * RX;
+        const int i0 = r0[ry], i1 = r1[ry], j0 = q0[rx], j1 = q1[rx];
+        T* d = s_in + ry * RP + rx;
+        const bool ok = (i0 | j0) >= 0;
+        const T* g = src + (ok ? (size_t)i0 * n + j0 : 0);
+        if (i1 < 0 && j1 < 0) {
+          cp_async_zfill<sizeof(T)>(d, g, ok);           // one pixel (or none)
+        } else if (!ok) {
+          *d = T(0);
+        } else {
+          // up to four pixels, loaded together
+          const T wy = i1 < 0 ? T(1) : T(2), wx = j1 < 0 ? T(1) : T(2);
+          const T v00 = g[0], v01 = j1 < 0 ? T(0) : src[(size_t)i0 * n + j1];
+          const T v10 = i1 < 0 ? T(0) : src[(size_t)i1 * n + j0];
+          const T v11 = (i1 < 0 || j1 < 0) ? T(0) : src[(size_t)i1 * n + j1];
+          T v = wy * wx * v00;
+          if (j1 >= 0) v -= wy * v01;
+          if (i1 >= 0) v -= wx * v10;
+          if (i1 >= 0 && j1 >= 0) v += v11;
+          *d = v;
+        }
       }
     } else {
       const bool rect = !ZPAD && pd.bc == BC_RECT;
@@ -551,7 +568,7 @@ k_vec(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __
     const size_t i = beg + threadIdx.x + (size_t)k * VEC_THREADS;
     if (i >= end) break;
     if (MODE == VEC_FOLD) {
-      const int a = (int)(i / n), b = (int)(i - (size_t)a * n);
+      const int a = (int)((unsigned)i / (unsigned)n), b = (int)i - a * n;      // n^2 < 2^31
       U[i] = fold_fetch<T>(pd, V, a, b);
     } else if (MODE == VEC_PCG_PUPD) {
       PP[i] = PZ[i] + beta * PP[i];

@@ -352,6 +352,8 @@ __device__ bool last_block_reduce(const Prob& pd, State& st, int blk, int nblk,
 template <typename T>
 __device__ __forceinline__ T fold_fetch(const Prob& pd, const T* V, int a, int b) {
   const int n = pd.n, c = pd.c, ne = pd.ne;
+  // at least c pixels from every edge only the pixel itself copies (a, b)
+  if (pd.bc == BC_ZERO || (a >= c && a < n - c && b >= c && b < n - c)) return V[(size_t)(a + c) * ne + (b + c)];
   int cy[3], cx[3], ny = 1, nx = 1;
   cy[0] = a; cx[0] = b;
   if (pd.bc == BC_PERIODIC) {
