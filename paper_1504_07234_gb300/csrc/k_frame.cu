@@ -712,12 +712,16 @@ __device__ __forceinline__ const T* frame_u(const Prob& pd, int u_slot) {
 // c_lev = (b0 x b0) with dilation d = 2^(lev-1) applied to c_{lev-1}, half-
 // sample mirror at the border.  c_{lev-1} is read in the polyphase order of d
 // (u, lev = 1: plain) and c_lev is written in that of 2d, the order of the
-// kernels that read it.  The launch walks the input order: item.y = input
-// row; for each column sub-lattice a of d the threads stride along it, its
-// taps d apart being its neighbouring positions (contiguous reads), and its
-// even and odd positions land in the output sub-lattices a and a + d (two
-// contiguous runs of writes).
-template <typename T>
+// kernels that read it.  The launch walks the input order: item.y = (row
+// sub-lattice b of d, chunk of RB of its rows, which are neighbouring input
+// rows); for each column sub-lattice a of d the threads stride along it, its taps
+// d apart being its neighbouring positions (contiguous reads), and its even and
+// odd positions land in the output sub-lattices a and a + d (two contiguous runs
+// of writes).  A thread walks down the chunk's rows with the horizontally
+// filtered rows y - d, y, y + d in registers: 3 (RB + 2) / RB loads per output
+// instead of 9.  The kernel is bound by those loads (4126^2: 55 us a launch with
+// one row per CTA, 0.136 GB); small images keep one row per CTA (lowpass_rows).
+template <typename T, int RB>
 __global__ void __launch_bounds__(LP_THREADS)
 k_lowpass(const Prob* __restrict__ probs, const State* __restrict__ states,
           const int2* __restrict__ items, int lev, int u_slot) {
@@ -728,32 +732,38 @@ k_lowpass(const Prob* __restrict__ probs, const State* __restrict__ states,
   const size_t plane = (size_t)nf * nf;
   const int d = 1 << (lev - 1);
   const Poly pin(nf, d), pout(nf, 2 * d);
+  const int sb = item.y & (d - 1), m0 = (item.y >> (lev - 1)) * RB;
+  const int nr = min(RB, pin.count(sb) - m0);    // rows of this chunk
+  if (nr <= 0) return;
   const T* in = (lev == 1) ? frame_u<T>(pd, u_slot)
                            : static_cast<const T*>(pd.lp) + (size_t)(lev - 2) * plane;
-  const int iy = item.y;
-  const int y = pin.inv(iy);
+  T* out = static_cast<T*>(pd.lp) + (size_t)(lev - 1) * plane;
   bool par;
-  const T* rm = in + (size_t)pin.pos(f3_refl(y - d, nf, &par)) * nf;
-  const T* r0 = in + (size_t)iy * nf;
-  const T* rp = in + (size_t)pin.pos(f3_refl(y + d, nf, &par)) * nf;
-  T* out = static_cast<T*>(pd.lp) + (size_t)(lev - 1) * plane + (size_t)pout.pos(y) * nf;
-  // the three input rows into L2 first (the sweep below then finds them there)
-  prefetch_range(rm, (size_t)nf * sizeof(T), threadIdx.x, LP_THREADS);
-  prefetch_range(r0, (size_t)nf * sizeof(T), threadIdx.x, LP_THREADS);
-  prefetch_range(rp, (size_t)nf * sizeof(T), threadIdx.x, LP_THREADS);
+  // rows m0 - 1 .. m0 + RB of the sub-lattice (mirrored into the image; past the
+  // chunk's end the last row again) and the output rows
+  const T* row[RB + 2];
+  T* orow[RB];
+#pragma unroll
+  for (int k = 0; k < RB + 2; ++k)
+    row[k] = in + (size_t)pin.pos(f3_refl(sb + d * (m0 + min(k, nr + 1) - 1), nf, &par)) * nf;
+#pragma unroll
+  for (int k = 0; k < RB; ++k) orow[k] = out + (size_t)pout.pos(sb + d * (m0 + min(k, nr - 1))) * nf;
   for (int a = 0; a < d; ++a) {
     const int ma = pin.count(a), sa = pin.start(a);
     // output run starts of the even and odd positions of sub-lattice a
     const int oe = a < nf ? pout.pos(a) : 0, oo = (a + d < nf) ? pout.pos(a + d) : 0;
-#pragma unroll 4
     for (int m = threadIdx.x; m < ma; m += LP_THREADS) {
       const int ic = sa + m;
       int im = ic - 1, ip = ic + 1;             // neighbours inside the sub-lattice
       if (m == 0) im = pin.pos(f3_refl(a - d, nf, &par));
       if (m == ma - 1) ip = pin.pos(f3_refl(a + d * (m + 1), nf, &par));
-      auto row = [&](const T* q) { return T(0.25) * (q[im] + q[ip]) + T(0.5) * q[ic]; };
-      const T v = T(0.25) * (row(rm) + row(rp)) + T(0.5) * row(r0);
-      out[(m & 1) ? oo + (m >> 1) : oe + (m >> 1)] = v;
+      const int o = (m & 1) ? oo + (m >> 1) : oe + (m >> 1);
+      T h[RB + 2];
+#pragma unroll
+      for (int k = 0; k < RB + 2; ++k) h[k] = T(0.25) * (row[k][im] + row[k][ip]) + T(0.5) * row[k][ic];
+#pragma unroll
+      for (int k = 0; k < RB; ++k)
+        if (k < nr) orow[k][o] = T(0.25) * (h[k] + h[k + 2]) + T(0.5) * h[k + 1];
     }
   }
 }
@@ -972,7 +982,17 @@ int lev_tiles(int nf, int lev, int seg) {
   lev_tile_grid(nf, dp, seg, &tx, &ty);
   return dp * dp * tx * ty;
 }
-int lowpass_blocks(int nf) { return nf; }
+// rows per CTA of the low-pass chain: 8 where one row per CTA gives more CTAs than
+// fit the chip (8 of 256 threads per SM)
+int lowpass_rows(int nf) { return nf > 152 * 8 ? 8 : 1; }
+int lowpass_blocks(int nf, int levels) {
+  int most = 0;
+  for (int l = 1; l < levels; ++l) {
+    const int d = 1 << (l - 1), m = Poly(nf, d).count_max(), rb = lowpass_rows(nf);
+    most = std::max(most, d * ((m + rb - 1) / rb));
+  }
+  return most;
+}
 
 // level kernel of a segment height (32 rows: FP64 only)
 template <typename T, typename TZ, bool TOP>
@@ -990,9 +1010,12 @@ void launch_frame_levels(const Prob* probs, State* states, const int2* items, co
                          double op_mu, cudaStream_t s) {
   // sec: (offset, count) of the fold, low-pass and level-L .. level-1 sections
   if (u_slot < 0 && sec[1] > 0) launch_vec<T>(VEC_FOLD, probs, states, items + sec[0], sec[1], 0, s);
-  if (sec[3] > 0)
-    for (int l = 1; l < levels; ++l)
-      k_lowpass<T><<<sec[3], LP_THREADS, 0, s>>>(probs, states, items + sec[2], l, u_slot);
+  // low-pass chain: the problems with one row per CTA, then those with 8
+  for (int l = 1; l < levels; ++l) {
+    if (sec[3] > 0) k_lowpass<T, 1><<<sec[3], LP_THREADS, 0, s>>>(probs, states, items + sec[2], l, u_slot);
+    const int o8 = sec[2 * (FRAME_SECTIONS - 1)], n8 = sec[2 * (FRAME_SECTIONS - 1) + 1];
+    if (n8 > 0) k_lowpass<T, 8><<<n8, LP_THREADS, 0, s>>>(probs, states, items + o8, l, u_slot);
+  }
   for (int k = 0; k < levels; ++k) {
     int lev = levels - k;
     const int off = sec[4 + 2 * k], cnt = sec[5 + 2 * k];
@@ -1193,7 +1216,9 @@ bool is_frame_kernel(const void* func) {
                           lev_kernel<float, __nv_bfloat16, true>(sg),
                           lev_kernel<double, double, false>(sg), lev_kernel<double, double, true>(sg)})
       if (f == func) return true;
-  if (func == (const void*)k_lowpass<float> || func == (const void*)k_lowpass<double>) return true;
+  for (const void* f : {(const void*)k_lowpass<float, 1>, (const void*)k_lowpass<float, 8>,
+                        (const void*)k_lowpass<double, 1>, (const void*)k_lowpass<double, 8>})
+    if (f == func) return true;
   return false;
 }
 

@@ -82,7 +82,7 @@ void add_frame_items(const Prob& pd, int i, int levels, int shape, int seg,
   auto add = [&](std::vector<int2>& L, int nblk) { for (int k = 0; k < nblk; ++k) L.push_back(make_int2(i, k)); };
   if (levels <= 2) { add(fs[0], frame_tiles(pd.nf, levels, shape, seg)); return; }
   if (pd.use_adj && pd.bc != BC_RECT && pd.bc != BC_AR && !pd.balanced) add(fs[0], pd.nblk_vec);
-  add(fs[1], lowpass_blocks(pd.nf));
+  add(fs[lowpass_rows(pd.nf) == 1 ? 1 : FRAME_SECTIONS - 1], lowpass_blocks(pd.nf, levels));
   for (int k = 0; k < levels; ++k) add(fs[2 + k], lev_tiles(pd.nf, levels - k, seg));
 }
 
@@ -305,7 +305,7 @@ int build_frame_list(mlba_batch* B, ItemList& L, const std::vector<int2> (&fs)[F
                      int levels) {
   if (levels <= 2) return build_list(B, L, fs[0]);
   std::vector<int2> all;
-  for (int k = 0; k < 2 + levels; ++k) {
+  for (int k = 0; k < FRAME_SECTIONS; ++k) {
     L.sec[2 * k] = (int)all.size();
     L.sec[2 * k + 1] = (int)fs[k].size();
     all.insert(all.end(), fs[k].begin(), fs[k].end());

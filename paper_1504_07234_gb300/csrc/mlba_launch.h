@@ -52,8 +52,8 @@ constexpr int VEC_THREADS = 256;
 constexpr int VEC_PER_THREAD = 8;
 constexpr int TR_CAP = 4096;          // complex values held by one transform CTA
 constexpr int FRAME_SHAPES = 8;      // tile shapes of the L <= 2 framelet kernel (k_frame.cu)
-constexpr int LP_THREADS = 256, LP_PER = 4;   // low-pass chain kernel (L >= 3)
-constexpr int FRAME_SECTIONS = 2 + 4;         // fold, low-pass, up to four levels
+constexpr int LP_THREADS = 256;               // low-pass chain kernel (L >= 3)
+constexpr int FRAME_SECTIONS = 2 + 4 + 1;     // fold, low-pass (one row per CTA), up to four levels, low-pass (8 rows)
 constexpr int SPEC_THREADS = 256;    // alpha_n solve (k_fft.cu)
 constexpr int SPEC_PER_THREAD = 32, SPEC_PER_THREAD_MIN = 8;   // spectral values per thread of a pass
 constexpr int SPEC_SUMS = 17;        // block sums of the bracketing pass (2 x 8 candidates + 1)
@@ -108,7 +108,8 @@ void launch_frame(const Prob* probs, State* states, const int2* items, int nitem
                   int shape, int seg, cudaStream_t s);
 int frame_tiles(int nf, int levels, int shape, int seg);   // CTAs of the fused sweep for one problem (L <= 2)
 int lev_tiles(int nf, int lev, int seg);                   // CTAs of one level kernel (L >= 3)
-int lowpass_blocks(int nf);                       // CTAs of one low-pass launch (L >= 3)
+int lowpass_rows(int nf);                         // rows per CTA of a low-pass launch (L >= 3)
+int lowpass_blocks(int nf, int levels);           // CTAs of one low-pass launch
 void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch);
 bool is_frame_kernel(const void* func);  // func is one of the framelet-update kernels
 int stencil_tiles(int outN, int R);      // CTAs of the stencil (R rows per thread) for an outN x outN output

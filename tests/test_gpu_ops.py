@@ -466,3 +466,20 @@ def test_fp64_thin_and_full_radix_plans(M, n, count):
     for i in range(count):
         assert rel_err(b.result(i), ref["f"]) <= 1e-9
     b.close()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("levels", [3, 4])
+@pytest.mark.parametrize("n", [1217, 1220])
+def test_lowpass_chunks(M, dtype, levels, n):
+    """Images wider than 1216 run the low-pass chain 8 rows per CTA: ragged last
+    chunks and odd sub-lattice sizes, against the oracle's framelet step."""
+    ctx = M.Context(PSFS["asym3"], n, "reflective", "none", dtype=dtype, levels=levels)
+    rng = np.random.default_rng(n)
+    u = rng.standard_normal((n, n))
+    zo, f = ctx.frame(np.zeros((8 * levels + 1, n, n), dtype=np.float32), u, 0.03)
+    z_ref = O.framelet_analysis(u, levels)
+    assert rel_err(zo.double().cpu().numpy(), z_ref) <= (1e-12 if dtype == "f64" else 2e-6)
+    assert rel_err(f.double().cpu().numpy(), O.framelet_synthesis(O.soft(z_ref, 0.03), levels)) <= (
+        1e-11 if dtype == "f64" else 1e-5)
+    ctx.close()
