@@ -31,6 +31,11 @@
 
 namespace mlba {
 
+// complex sums in FP32: one paired instruction each (a - b as the exact
+// a + (-1) b)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
 // ---------------------------------------------------------------------------
 // small DFTs (forward: exp(-2 pi i jk/R); INV: conjugate)
 template <typename T2, bool INV>
