@@ -244,7 +244,10 @@ int mlba_op_blur_adjoint(mlba_ctx* ctx, const void* t, void* out, int on_device)
  * Uses the context's C (DFT or DCT) through the batched transform kernels. */
 int mlba_op_precond(mlba_ctx* ctx, const void* r, void* out, double alpha, int which, int on_device);
 /* One fused framelet pass: z_out = z_in + W u, f = W^T S_mu(z_out)
- * (Eq. MLBA2 second half; Section 6.1).  z_*: z_store type; u, f: N_f x N_f. */
+ * (Eq. MLBA2 second half; Section 6.1).  z_*: z_store type; u, f: N_f x N_f.
+ * The first call allocates two z-sized scratch buffers (MLBA_E_NOMEM if it
+ * cannot), which the context keeps until it is destroyed; make it before any
+ * stream capture. */
 int mlba_op_frame(mlba_ctx* ctx, const void* z_in, const void* u, void* z_out,
                   void* f, double mu, int on_device);
 /* alpha solving alpha ||(CC^T + alpha I)^{-1} r|| = qn ||r|| (Eq. Alg4_rev_7);
@@ -318,7 +321,9 @@ void mlba_batch_destroy(mlba_batch* b);
  * prefetch distance in rows, how it was chosen (0 built-in default, 1
  * measured at create, 2 read from the tuning cache, 3 forced by
  * opts.frame_shape) and the measured microseconds per launch (1, 2).  Shapes
- * apply to levels <= 2; with more levels tile_x = tile_y = prefetch = 0.
+ * apply to levels <= 2; with more levels tile_x = tile_y = prefetch = 0.  The
+ * built-in default's tile has fewer rows in batches that would leave the chip
+ * idle.
  * Any output pointer may be NULL.  No counterpart in the paper. */
 int mlba_batch_tiles(mlba_batch* b, int* frame_shape, int* tile_x, int* tile_y, int* prefetch,
                      int* how, float* us);
