@@ -719,8 +719,9 @@ __device__ __forceinline__ const T* frame_u(const Prob& pd, int u_slot) {
 // odd positions land in the output sub-lattices a and a + d (two contiguous runs
 // of writes).  A thread walks down the chunk's rows with the horizontally
 // filtered rows y - d, y, y + d in registers: 3 (RB + 2) / RB loads per output
-// instead of 9.  The kernel is bound by those loads (4126^2: 55 us a launch with
-// one row per CTA, 0.136 GB); small images keep one row per CTA (lowpass_rows).
+// instead of 9.  The kernel is bound by those loads (4126^2, 0.136 GB: 55 us a
+// launch with one row per CTA, 40 with 8); small images keep one row per CTA
+// (lowpass_rows).
 template <typename T, int RB>
 __global__ void __launch_bounds__(LP_THREADS)
 k_lowpass(const Prob* __restrict__ probs, const State* __restrict__ states,
@@ -1045,7 +1046,7 @@ void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch) {
 // planes are consecutive along the warp, its group is one or more 16-byte
 // words (a whole sector or more for 4- and 8-byte elements wherever the
 // polyphase order puts it); then the low-pass plane.  HBM-bound: 751^2, L = 2,
-// FP32: 13 us a direction (2 x 38 MB); element by element it took 42.
+// FP32 (2 x 38 MB): 15 us in, 12 us out; element by element it took 42 each.
 template <typename E, bool TO_INTERNAL>
 __global__ void __launch_bounds__(256)
 k_zlayout(E* __restrict__ dst, const E* __restrict__ src, int levels, int nf) {

@@ -672,7 +672,7 @@ int stencil_rows(const mlba_batch* B) {
 // full CTAs the transforms spread over more of them instead.  Both sides of the line
 // (one CTA holding up to TR_CAP values against 2 per SM; a pass measured alone):
 // 256^2 DCT rows 10.5 -> 6.7 us, forward columns with the candidate sums 29.5
-// -> 18 us; 256^2 FP64 columns 111 -> 36 us; 1000^2 DFT, all three passes
+// -> 18 us; 256^2 FP64 columns 111 -> 36 us (20 in radix 4); 1000^2 DFT, all three passes
 // 48 -> 40 us.  The 64-problem batch has 2400 full CTAs and keeps them (the
 // split measured no gain there).
 constexpr int TR_FILL_CTAS = 304;
@@ -1049,8 +1049,8 @@ int time_frame_shape(mlba_batch* B, int shape, float* us) {
 // 3 at 8, 4 at 4).  Halve while the doubled number of warps is resident at
 // once: about 20 FP32 warps per SM; in FP64 one warp per scheduler, because the
 // FP64 pipe is already full with one.  Measured per launch, 32 rows against
-// the choice: 256^2 FP32 32 -> 10 us (4 rows), 72^2 FP64 L = 1 150 -> 27 us (4);
-// 1044^2 BF16 z 45 -> 39 us (16; 8: 44, 4: 54); the 64-problem batch stays at
+// the choice: 256^2 FP32 32 -> 10 us (4 rows), 72^2 FP64 L = 1 150 -> 21 us (4);
+// 1044^2 BF16 z 45 -> 39 us (16; 8: 44, 4: 54; 31 with the row routine); the 64-problem batch stays at
 // 32 (16: +0.5 %, 8: +10 %).  L >= 3 starts at 16 in FP32 (a step at 4096^2:
 // as 32; at 2048^2: 470 us, 32: 486, 8: 527; at 1024^2: 194, 32: 218, 8: 209;
 // at 512^2 the choice is 4: 119, 32: 169).
