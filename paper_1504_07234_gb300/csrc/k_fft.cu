@@ -60,11 +60,13 @@ __device__ __forceinline__ void dft3(T2* v) {
   T2 a = v[0], b = v[1], c = v[2];
   T2 t1 = cadd(b, c), t2 = csub(b, c);
   T2 m; m.x = a.x - T(0.5) * t1.x; m.y = a.y - T(0.5) * t1.y;
-  // forward: X1 = m - i h t2, X2 = m + i h t2
-  T2 ih; ih.x = -h * t2.y; ih.y = h * t2.x;   // i h t2
+  // forward: X1 = m - i h t2, X2 = m + i h t2 (one rounding each)
+  T2 p, q;                                    // m + i h t2, m - i h t2
+  p.x = fma(-h, t2.y, m.x); p.y = fma(h, t2.x, m.y);
+  q.x = fma(h, t2.y, m.x); q.y = fma(-h, t2.x, m.y);
   v[0] = cadd(a, t1);
-  if (INV) { v[1] = cadd(m, ih); v[2] = csub(m, ih); }
-  else { v[1] = csub(m, ih); v[2] = cadd(m, ih); }
+  v[1] = INV ? p : q;
+  v[2] = INV ? q : p;
 }
 template <typename T2, bool INV>
 __device__ __forceinline__ void dft5(T2* v) {
@@ -1528,25 +1530,8 @@ k_rows_inv_dot(const Prob* __restrict__ probs, State* states, const int2* __rest
   if (!rows_inv_body<T>(item, probs, states, SL_PZ, FIRST ? 0 : 1, dot)) return;
   double vals[1], tot[1];
   vals[0] = block_sum<NT>(dot.acc, red);
-  if (last_block_reduce<NT, 1>(pd, st, item.y, pd.nblk_rows, vals, tot, red) && threadIdx.x == 0) {
-    const double rho = tot[0];
-    if (FIRST) {
-      st.prho = rho;
-      st.prho0 = rho;
-      st.psteps = 0;
-      st.pdone = (rho <= 0.0) ? 1 : 0;
-    } else {
-      st.psteps += 1;
-      // relative residual of the symmetric system (psys): sqrt(r_k^T M r_k / r_0^T M r_0)
-      const double rel = sqrt(fmax(rho, 0.0) / st.prho0);
-      if (rel <= pd.pcg_tol || st.psteps >= pd.pcg_max) {
-        st.pdone = 1;
-      } else {
-        st.pbeta = rho / st.prho;
-        st.prho = rho;
-      }
-    }
-  }
+  if (last_block_reduce<NT, 1>(pd, st, item.y, pd.nblk_rows, vals, tot, red) && threadIdx.x == 0)
+    pcg_scalars(pd, st, tot[0], FIRST);
 }
 
 

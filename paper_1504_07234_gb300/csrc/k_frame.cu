@@ -231,15 +231,19 @@ __device__ __forceinline__ double f3_flip(double v, int m) {
 //   z0 += s / 4 + h_b / 2,  z1 += (sqrt 2 / 4) d,  z2 += h_b / 2 - s / 4,
 // and the transpose the same way: 14 operations per horizontal mask instead
 // of 19 (FP32: an issue-bound sweep; FP64: the pipe is full).
-template <bool LOW, typename T, typename TZ>
+// BF16 z: the masks tap by tap, in one fixed order (the rounding of z to 8 bits
+// makes the last bit of these sums matter, see the host's stencil_variant).
+// PARTS: a row's three shares are summed by themselves and then added to its
+// rows (k_frame_lev); else every tap is added to them directly (k_frame3).
+template <bool LOW, bool PARTS, typename T, typename TZ>
 __device__ __forceinline__ void f3_row(const T (&ha)[3], const T (&hb)[3], const T (&hc)[3],
                                        const ZGroup<TZ>& zi, TZ zl, int mrow, int mcol, T mu,
                                        ZGroup<TZ>& zo, TZ& zlo, T (&pa)[3], T (&pb)[3], T (&pc)[3]) {
   const T s2q = T(0.35355339059327376220);               // sqrt(2) / 4
   const int m11 = mrow ^ mcol;
+  constexpr bool TAPS = sizeof(TZ) == 2;
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    const T s = ha[j] + hc[j], d = ha[j] - hc[j];
     auto in = [&](int i) {                               // z of band (i, j), mirrored sign applied
       T v = T(ld_z(&zi.e[3 * i + j - 1]));
       if (i == 1 && j == 1) v = f3_flip(v, m11);
@@ -247,6 +251,29 @@ __device__ __forceinline__ void f3_row(const T (&ha)[3], const T (&hb)[3], const
       else if (j == 1) v = f3_flip(v, mcol);
       return v;
     };
+    if constexpr (TAPS) {
+      // (a quarter of a sum is exactly the sum of the quarters)
+      const T q = T(0.25) * (ha[j] + hc[j]);
+      T a0 = PARTS ? T(0) : pa[j], a1 = PARTS ? T(0) : pb[j], a2 = T(0);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        if (i == 0 && j == 0 && !LOW) continue;
+        const T b0 = i == 0 ? T(0.25) : i == 1 ? s2q : T(-0.25), b2 = i == 1 ? -s2q : b0;
+        const T a = i == 1 ? b0 * ha[j] + b2 * hc[j] : fma(T(0.5), hb[j], i == 0 ? q : -q);
+        const T zn = (i == 0 && j == 0 ? T(ld_z(&zl)) : in(i)) + a;
+        if (i == 0 && j == 0) zlo = to_z(zn, (TZ*)nullptr);
+        else zo.e[3 * i + j - 1] = to_z(zn, (TZ*)nullptr);
+        const T x = f3_soft(zn, mu);
+        a0 += b0 * x;
+        if (i != 1) a1 += T(0.5) * x;
+        a2 += b2 * x;
+      }
+      pa[j] = PARTS ? pa[j] + a0 : a0;
+      pb[j] = PARTS ? pb[j] + a1 : a1;
+      pc[j] = a2;
+      continue;
+    }
+    const T s = ha[j] + hc[j], d = ha[j] - hc[j];
     T x0 = T(0);
     if (j > 0 || LOW) {
       const T v = j == 0 ? T(ld_z(&zl)) : in(0);
@@ -276,8 +303,16 @@ __device__ __forceinline__ void f3_hrow(T cm, T c0, T cp, T (&h)[3]) {
   h[2] = fma(T(0.5), c0, -t);
 }
 // horizontal synthesis parts of a completed row: A(x + D) + B(x) + C(x - D)
-template <typename T>
+// (TZ: BF16 z term by term, as f3_row)
+template <typename TZ, typename T>
 __device__ __forceinline__ void f3_abc(const T (&P)[3], T& A, T& B, T& C) {
+  if (sizeof(TZ) == 2) {
+    const T s2q = T(0.35355339059327376220);
+    A = T(0.25) * P[0] + s2q * P[1] - T(0.25) * P[2];
+    B = T(0.5) * (P[0] + P[2]);
+    C = T(0.25) * P[0] - s2q * P[1] - T(0.25) * P[2];
+    return;
+  }
   const T e = T(0.25) * (P[0] - P[2]), s2q = T(0.35355339059327376220);
   A = fma(s2q, P[1], e);
   B = T(0.5) * (P[0] + P[2]);
@@ -482,7 +517,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     const int zwo = zqo[kq];
     ZGroup<TZ> zo;
     TZ zlo = TZ(0.0f);
-    f3_row<TOP, T, TZ>(hr[ia], hr[ib], hr[ic], zq[RING > 0 ? 0 : kq], zl[kq], zqm[kq], mcol, mu, zo, zlo,
+    f3_row<TOP, false, T, TZ>(hr[ia], hr[ib], hr[ic], zq[RING > 0 ? 0 : kq], zl[kq], zqm[kq], mcol, mu, zo, zlo,
                        pr[ia], pr[ib], pr[ic]);
     if (own) {
       uint4* dstz = reinterpret_cast<uint4*>(zout + (gbase + 8 * zwo));
@@ -507,7 +542,7 @@ __device__ __forceinline__ void f3_level(const Prob& pd, const T* __restrict__ c
     const int r = y - D;
     if (r >= yo0) {
       T A, B, C;
-      f3_abc(pr[ia], A, B, C);
+      f3_abc<TZ>(pr[ia], A, B, C);
       const T out = B + __shfl_down_sync(FULL, A, D) + __shfl_up_sync(FULL, C, D);
       if (LEV == 2 && L == 2) {
         // s_1 row r (lanes 2..29) -> (b0 x b0)^T s_1 row r - 1 (lanes 3..28)
@@ -932,7 +967,7 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
     const int zwo = zqo[kq];
     ZGroup<TZ> zo;
     TZ zlo = TZ(0.0f);
-    f3_row<TOP, T, TZ>(hr[ia], hr[ib], hr[ic], zq[kq], zl[kq], zqm[kq], mcol, mu, zo, zlo, pr[ia],
+    f3_row<TOP, true, T, TZ>(hr[ia], hr[ib], hr[ic], zq[kq], zl[kq], zqm[kq], mcol, mu, zo, zlo, pr[ia],
                        pr[ib], pr[ic]);
     if (own) {
       uint4* dz = reinterpret_cast<uint4*>(zout + (gbase + 8 * zwo));
@@ -960,7 +995,7 @@ k_frame_lev(const Prob* __restrict__ probs, State* __restrict__ states,
     // row y - 1 is complete
     const int r = y - 1;
     T A, B, C;
-    f3_abc(pr[ia], A, B, C);
+    f3_abc<TZ>(pr[ia], A, B, C);
     T out = B + __shfl_down_sync(FULL, A, 1) + __shfl_up_sync(FULL, C, 1);
     if (r >= seg_lo && own_c) {
       // (b0 x b0)^T s_l at (r, mx): rows r - 1, r, r + 1 = y

@@ -109,20 +109,25 @@ k_persist(const Prob* __restrict__ probs, State* __restrict__ states, int nprob,
             if (i >= cnt) continue;
             unsigned char* sm = smraw + (size_t)sub2 * stencil_slot;
             const BlkSub<STENCIL_THREADS> b{1 + sub2};
-            // (the rows per thread of the graph schedule: the norm's partial
-            // sums then add up in the same order)
+            // (the variant of the graph schedule: every sum then adds up in the
+            // same order; with BF16 z that is always the row-first one)
             auto tile = [&](auto rc) {
               constexpr int R = decltype(rc)::value;
+              constexpr bool RF = sizeof(TZ) == 2;
               if (sg.kind == PS_RESID)
-                stencil_body<T, ST_FWD_RESID, R>(it[i], probs, states, SL_F, SL_R, SL_G, 0, sm, red[sub2], &flag[sub2], b);
+                stencil_body<T, ST_FWD_RESID, R, RF>(it[i], probs, states, SL_F, SL_R, SL_G, 0, sm, red[sub2], &flag[sub2], b);
               else if (sg.kind == PS_CORR)
-                stencil_body<T, ST_CORR, R>(it[i], probs, states, -1, SL_V, SL_V, 0, sm, red[sub2], &flag[sub2], b);
+                stencil_body<T, ST_CORR, R, RF>(it[i], probs, states, -1, SL_V, SL_V, 0, sm, red[sub2], &flag[sub2], b);
               else
-                stencil_body<T, ST_REBLUR, R>(it[i], probs, states, -1, -1, SL_U, 0, sm, red[sub2], &flag[sub2], b);
+                stencil_body<T, ST_REBLUR, R, RF>(it[i], probs, states, -1, -1, SL_U, 0, sm, red[sub2], &flag[sub2], b);
             };
-            if (sg.rows == 2) tile(std::integral_constant<int, 2>{});
-            else if (sg.rows == 4) tile(std::integral_constant<int, 4>{});
-            else tile(std::integral_constant<int, 8>{});
+            if constexpr (sizeof(TZ) == 2) {
+              tile(std::integral_constant<int, 8>{});
+            } else {
+              if (sg.variant == 2) tile(std::integral_constant<int, 2>{});
+              else if (sg.variant == 4) tile(std::integral_constant<int, 4>{});
+              else tile(std::integral_constant<int, 8>{});
+            }
             b.sync();   // the next item's tile loads overwrite this one's shared memory
           }
           break;

@@ -174,21 +174,31 @@ __host__ __device__ constexpr int st_pitch(int RX, int elem) {
 // rank-one PSF: pitch in pairs of the column-pass result (row pairs x columns),
 // odd so that the lanes of the row pass (one row pair each) hit different banks
 __host__ __device__ constexpr int st_tpitch(int RX, int elem) { return (st_pitch(RX, elem) + 2) | 1; }
+// rank-one PSF, row pass first: pitch of its result, and whether that needs a
+// tile of its own (else the rows fit the threads' registers and overwrite the input)
+constexpr int ST_RP = ST_TX + 2;
+__host__ __device__ constexpr bool st_rows_tile(int RY) { return 4 * RY > 2 * STENCIL_THREADS; }
 // shared memory of a tile: weights, runs (general PSF), the source rows
 // and columns of the tile, input tile (which the
 // column-pass result and the output tile of a rank-one PSF overwrite)
-__host__ __device__ constexpr size_t st_smem(int R, int p, int sep, int nrw, int nruns, int elem) {
-  const int RY = 4 * R + p - 1, RX = ST_TX + p - 1;
+__host__ __device__ constexpr size_t st_smem(int variant, int p, int sep, int nrw, int nruns, int elem) {
+  const int R = st_rows_of(variant), RY = 4 * R + p - 1, RX = ST_TX + p - 1;
   const int nw = sep ? 2 * p : nrw, we = elem == 4 ? 2 : 1;
-  const size_t in = (size_t)RY * st_pitch(RX, elem), tmp = sep ? (size_t)4 * R * st_tpitch(RX, elem) : 0;
-  return (((size_t)nw * we + 3) / 4 * 4 + (in > tmp ? in : tmp)) * elem + (sep ? 0 : (size_t)nruns * 16) +
+  size_t in = (size_t)RY * st_pitch(RX, elem);
+  const size_t tmp = sep ? (size_t)4 * R * st_tpitch(RX, elem) : 0;
+  if (sep && (variant & ST_ROW_FIRST)) in += st_rows_tile(RY) ? (size_t)RY * ST_RP : 0;
+  else if (tmp > in) in = tmp;
+  return (((size_t)nw * we + 3) / 4 * 4 + in) * elem + (sep ? 0 : (size_t)nruns * 16) +
          (size_t)((2 * (RY + RX) + 3) / 4 * 4) * 4;
 }
 
 #ifndef MLBA_BODIES_ONLY
-int stencil_tiles(int outN, int R) { return ((outN + ST_TX - 1) / ST_TX) * ((outN + 4 * R - 1) / (4 * R)); }
-size_t stencil_smem(int R, int p, int sep, int nrw, int nruns, int elem) {
-  return st_smem(R, p, sep, nrw, nruns, elem);
+int stencil_tiles(int outN, int variant) {
+  const int ty = 4 * st_rows_of(variant);
+  return ((outN + ST_TX - 1) / ST_TX) * ((outN + ty - 1) / ty);
+}
+size_t stencil_smem(int variant, int p, int sep, int nrw, int nruns, int elem) {
+  return st_smem(variant, p, sep, nrw, nruns, elem);
 }
 #endif
 
@@ -203,15 +213,16 @@ size_t stencil_smem(int R, int p, int sep, int nrw, int nruns, int elem) {
 //    windows, over the tile's 64 + p - 1 columns), kept in registers and written
 //    over the input tile as pairs of rows, then the row pass on the row pairs
 //    (R-column windows): both passes are paired FMAs on conflict-free loads.
-//    The row-first order did 32 + p - 1 rows for 32 with scalar FMAs from
-//    four-way conflicting loads.
+//    Row pass first (ROWF; 32 + p - 1 rows for 32, four-way conflicting loads:
+//    4096^2, p = 31, FP32 z: residual 166 us against 126): problems whose z is
+//    BF16, see st_variant.
 // Forward (A f)(y, x) = sum_{a,b} H[a][b] f_ext(y + c - a, x + c - b); the
 // correlation (ne x ne) is sum_{a,b} H[a][b] t(y - 2c + a, x - 2c + b).
 // (FP32: 8 CTAs per SM, 64 registers; the tile of the largest PSF of a batch
 // decides how many fit in shared memory)
 // One stencil item (tile) on the thread group `blk` of STENCIL_THREADS threads,
 // with its shared memory at smraw, 32 doubles of reduction space and one int.
-template <typename T, int MODE, int R, typename BLK>
+template <typename T, int MODE, int R, bool ROWF, typename BLK>
 __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __restrict__ probs,
                                              State* __restrict__ states, int src_slot, int dst_slot,
                                              int aux_slot, int pcg, unsigned char* smraw,
@@ -238,8 +249,8 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   const int RP = st_pitch(RX, (int)sizeof(T));
   const bool sep = pd.sep != 0;
 
-  // shared memory: weights, column runs (general PSF), input tile, row-pass
-  // tile (rank-one PSF)
+  // shared memory: weights, column runs (general PSF), tables of source rows
+  // and columns, input tile (and a row-pass tile: ROWF, tall tiles)
   const int nw = sep ? 2 * p : pd.nrw;
   TW* s_w = reinterpret_cast<TW*>(smraw);
   constexpr int WE = (int)(sizeof(TW) / sizeof(T));
@@ -386,7 +397,48 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   T2 acc[R];
 #pragma unroll
   for (int j = 0; j < R; ++j) { acc[j].x = T(0); acc[j].y = T(0); }
-  if (sep) {
+  if (ROWF && sep) {
+    // row pass: h(y, x) = sum_t wx[t] in(y, x + t), an item being 8 columns of a
+    // row pair; written over the input tile (row y at the start of its row) once
+    // every thread holds its items, or into a tile of its own
+    static_assert(!ROWF || R == 8, "row pass first: 8 rows per thread");
+    constexpr int RND = 2;
+    auto rows = [&](int it, T2 (&h)[8]) {
+      const T* base = s_in + 2 * (it >> 3) * RP + xs + (it & 7) * 8;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { h[j].x = T(0); h[j].y = T(0); }
+      window_run<T, 8>(h, s_w, p, [&](int q) { T2 v; v.x = base[q]; v.y = base[RP + q]; return v; });
+    };
+    auto put = [&](int it, const T2 (&h)[8], T* to, int pitch) {
+      T* d = to + 2 * (it >> 3) * pitch + (it & 7) * 8;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { d[j] = h[j].x; d[pitch + j] = h[j].y; }
+    };
+    T* hb = s_in;
+    int hp = RP;
+    if (!st_rows_tile(RY)) {
+      T2 h[RND][8];
+#pragma unroll
+      for (int i = 0; i < RND; ++i)
+        if (tid + i * NT < 4 * RY) rows(tid + i * NT, h[i]);
+      blk.sync();
+#pragma unroll
+      for (int i = 0; i < RND; ++i)
+        if (tid + i * NT < 4 * RY) put(tid + i * NT, h[i], hb, hp);
+    } else {
+      hb = s_in + RY * RP;
+      hp = ST_RP;
+      for (int it = tid; it < 4 * RY; it += NT) {
+        T2 h[8];
+        rows(it, h);
+        put(it, h, hb, hp);
+      }
+    }
+    blk.sync();
+    // column pass: out(y, x) = sum_t wy[t] h(y + t, x)
+    hb += y8 * hp + x2;
+    window_run<T, R>(acc, s_w + p, p, [&](int q) { return *reinterpret_cast<const T2*>(hb + q * hp); });
+  } else if (sep) {
     // column pass: tmp(y, c) = sum_t wy[t] in(y + t, c) for the tile's columns
     // in pairs, an item being R rows of a pair.  Pairs are aligned in shared
     // memory where the tile's shifted columns fit 64 pairs (else they start at
@@ -528,15 +580,15 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   }
 }
 
-template <typename T, int MODE, int R>
+template <typename T, int MODE, int R, bool ROWF = false>
 __global__ void __launch_bounds__(STENCIL_THREADS, sizeof(T) == 4 ? 8 : 4)
 k_stencil(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __restrict__ items,
           int src_slot, int dst_slot, int aux_slot, int pcg) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double red[32];
   __shared__ int flag;
-  stencil_body<T, MODE, R>(items[blockIdx.x], probs, states, src_slot, dst_slot, aux_slot, pcg, smraw,
-                        red, &flag, BlkFull{});
+  stencil_body<T, MODE, R, ROWF>(items[blockIdx.x], probs, states, src_slot, dst_slot, aux_slot, pcg, smraw,
+                                 red, &flag, BlkFull{});
 }
 
 template <typename T, int MODE>
@@ -547,8 +599,9 @@ k_vec(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __
   const Prob& pd = probs[item.x];
   State& st = states[item.x];
   if (st.stopped) return;
-  // FINISH always copies the solution out
-  if (pcg && st.pdone && MODE != VEC_PCG_FINISH) return;
+  // RHO0 starts a solve; FINISH always copies the solution out
+  constexpr bool DOT = MODE == VEC_PCG_RHO0 || MODE == VEC_PCG_RHO;
+  if (pcg && st.pdone && MODE != VEC_PCG_RHO0 && MODE != VEC_PCG_FINISH) return;
   const int n = pd.n;
   const size_t nn = (size_t)n * n;
   const size_t chunk = (size_t)VEC_THREADS * VEC_PER_THREAD;
@@ -561,6 +614,8 @@ k_vec(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __
   const T* __restrict__ V = static_cast<const T*>(pd.buf[SL_V]);
   const T* __restrict__ PX = static_cast<const T*>(pd.buf[SL_PX]);
   const T* __restrict__ PZ = static_cast<const T*>(pd.buf[SL_PZ]);
+  const T* __restrict__ RES = static_cast<const T*>(pd.buf[MODE == VEC_PCG_RHO0 ? SL_R : SL_PRES]);
+  T dot = T(0);
   const T beta = MODE == VEC_PCG_PUPD ? T(st.pbeta) : T(0);
   const bool any = MODE == VEC_PCG_FINISH && st.psteps > 0;
 #pragma unroll
@@ -572,9 +627,20 @@ k_vec(const Prob* __restrict__ probs, State* __restrict__ states, const int2* __
       U[i] = fold_fetch<T>(pd, V, a, b);
     } else if (MODE == VEC_PCG_PUPD) {
       PP[i] = PZ[i] + beta * PP[i];
+    } else if (DOT) {
+      const T z = PZ[i];
+      dot += RES[i] * z;
+      if (MODE == VEC_PCG_RHO0) PP[i] = z;
     } else if (MODE == VEC_PCG_FINISH) {
       TT[i] = any ? PX[i] : T(0);
     }
+  }
+  if (DOT) {
+    __shared__ double red[32];
+    double tot[1];
+    const double vals[1] = {block_sum<VEC_THREADS>((double)dot, red)};
+    if (last_block_reduce<VEC_THREADS, 1>(pd, st, item.y, pd.nblk_vec, vals, tot, red) && threadIdx.x == 0)
+      pcg_scalars(pd, st, tot[0], MODE == VEC_PCG_RHO0);
   }
   if (MODE == VEC_PCG_FINISH && item.y == 0 && threadIdx.x == 0) {
     const int it = st.iter - 1;
@@ -749,33 +815,36 @@ void launch_fc_out(const Prob* probs, State* states, const int2* items, int nite
 }
 
 // ---------------------------------------------------------------------------
-// the stencil kernel of a mode and of the rows per thread
-template <typename T, int R>
+// the stencil kernel of a mode and a variant (st_variant)
+template <typename T, int R, bool ROWF = false>
 auto stencil_kernel_r(int mode) {
   switch (mode) {
-    case ST_FWD_RESID: return k_stencil<T, ST_FWD_RESID, R>;
-    case ST_FWD_STORE: return k_stencil<T, ST_FWD_STORE, R>;
-    case ST_FWD_PCGQ: return k_stencil<T, ST_FWD_PCGQ, R>;
-    case ST_REBLUR: return k_stencil<T, ST_REBLUR, R>;
-    default: return k_stencil<T, ST_CORR, R>;
+    case ST_FWD_RESID: return k_stencil<T, ST_FWD_RESID, R, ROWF>;
+    case ST_FWD_STORE: return k_stencil<T, ST_FWD_STORE, R, ROWF>;
+    case ST_FWD_PCGQ: return k_stencil<T, ST_FWD_PCGQ, R, ROWF>;
+    case ST_REBLUR: return k_stencil<T, ST_REBLUR, R, ROWF>;
+    default: return k_stencil<T, ST_CORR, R, ROWF>;
   }
 }
 template <typename T>
-auto stencil_kernel(int mode, int R) {
+auto stencil_kernel(int mode, int variant) {
+  if constexpr (sizeof(T) == 4)
+    if (variant & ST_ROW_FIRST) return stencil_kernel_r<T, 8, true>(mode);
+  const int R = st_rows_of(variant);
   return R == 2 ? stencil_kernel_r<T, 2>(mode) : R == 4 ? stencil_kernel_r<T, 4>(mode) : stencil_kernel_r<T, 8>(mode);
 }
 
 template <typename T>
 void launch_stencil(int mode, const Prob* probs, State* states, const int2* items, int nitems,
-                    int src, int dst, int aux, int pcg, int rows, size_t smem, cudaStream_t s) {
+                    int src, int dst, int aux, int pcg, int variant, size_t smem, cudaStream_t s) {
   if (nitems <= 0) return;
-  stencil_kernel<T>(mode, rows)<<<nitems, STENCIL_THREADS, smem, s>>>(probs, states, items, src, dst, aux, pcg);
+  stencil_kernel<T>(mode, variant)<<<nitems, STENCIL_THREADS, smem, s>>>(probs, states, items, src, dst, aux, pcg);
 }
 
 template <typename T>
-cudaError_t stencil_set_smem(int rows) {
+cudaError_t stencil_set_smem(int variant) {
   for (int mode : {(int)ST_FWD_RESID, (int)ST_FWD_STORE, (int)ST_FWD_PCGQ, (int)ST_REBLUR, (int)ST_CORR}) {
-    const cudaError_t e = cudaFuncSetAttribute((const void*)stencil_kernel<T>(mode, rows),
+    const cudaError_t e = cudaFuncSetAttribute((const void*)stencil_kernel<T>(mode, variant),
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_LIMIT);
     if (e != cudaSuccess) return e;
   }
@@ -789,6 +858,8 @@ void launch_vec(int mode, const Prob* probs, State* states, const int2* items, i
   dim3 g(nitems), b(VEC_THREADS);
   switch (mode) {
     case VEC_FOLD: k_vec<T, VEC_FOLD><<<g, b, 0, s>>>(probs, states, items, pcg); break;
+    case VEC_PCG_RHO0: k_vec<T, VEC_PCG_RHO0><<<g, b, 0, s>>>(probs, states, items, pcg); break;
+    case VEC_PCG_RHO: k_vec<T, VEC_PCG_RHO><<<g, b, 0, s>>>(probs, states, items, pcg); break;
     case VEC_PCG_PUPD: k_vec<T, VEC_PCG_PUPD><<<g, b, 0, s>>>(probs, states, items, pcg); break;
     default: k_vec<T, VEC_PCG_FINISH><<<g, b, 0, s>>>(probs, states, items, pcg); break;
   }

@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <new>
 #include <string>
+#include <type_traits>
 
 #include "../../include/mlba.h"
 #include "mlba_internal.cuh"
@@ -117,7 +118,7 @@ struct mlba_batch {
   std::vector<int2*> allocs;
   void* op_z[2] = {nullptr, nullptr};   // mlba_op_frame: z in the internal order (first call)
   size_t smem_stencil = 0, smem_fft = 0;
-  int st_rows = 8;              // stencils: rows per thread (stencil_rows)
+  int st_variant = 8;           // stencils: rows per thread and pass order (stencil_variant)
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool has_data = false;
@@ -180,13 +181,14 @@ int vec_blocks(size_t elems) {
 // of loads and sums) while the launch has at most one CTA per SM then.  A step
 // with 32 / 8: 256^2 FP32 83 / 81 us, 300^2 FP64 166 / 112; the 64-problem batch
 // 1.020 / 1.024 ms, 4096^2 1.09 / 1.16.
-void spec_geometry(std::vector<HostProb>& v) {
+// (bf16: always 32, see stencil_variant)
+void spec_geometry(std::vector<HostProb>& v, bool bf16) {
   size_t ns = 0;
   for (const HostProb& h : v) if (h.pd.ns) ns += spec_elems(h.pd);
   for (HostProb& h : v) {
     Prob& pd = h.pd;
     const size_t tot = pd.ns ? ns : spec_elems(pd);       // (not 4-NS: the operator entry point)
-    pd.spec_pt = tot <= (size_t)152 * SPEC_THREADS * SPEC_PER_THREAD_MIN ? SPEC_PER_THREAD_MIN : SPEC_PER_THREAD;
+    pd.spec_pt = !bf16 && tot <= (size_t)152 * SPEC_THREADS * SPEC_PER_THREAD_MIN ? SPEC_PER_THREAD_MIN : SPEC_PER_THREAD;
     pd.nblk_spec = (int)((spec_elems(pd) + SPEC_THREADS * pd.spec_pt - 1) / (SPEC_THREADS * pd.spec_pt));
   }
 }
@@ -330,7 +332,7 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
   State* S = B->d_states;
   if (part & PART_A) {
     // a2: r = g - A f with ||r||^2 and the stop rule
-    launch_stencil<T>(ST_FWD_RESID, P, S, L.blur.dev, L.blur.count, SL_F, SL_R, SL_G, 0, B->st_rows, B->smem_stencil, s);
+    launch_stencil<T>(ST_FWD_RESID, P, S, L.blur.dev, L.blur.count, SL_F, SL_R, SL_G, 0, B->st_variant, B->smem_stencil, s);
     // (FFT blur path: f extended by the BCs, A f by convolution with the PSF)
     if (L.fc_out_r.count) {
       launch_fc_pad<T>(P, S, L.fc_pad_f.dev, L.fc_pad_f.count, 0, -1, s);
@@ -395,14 +397,24 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
       // (the first M r ignores pdone of the previous solve and sets it)
       launch_rows_fwd<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_R, 0, B->smem_fft, s);
       launch_cols<T>(P, S, L.cols_kry.dev, L.cols_kry.count, COL_FUSED, 0, 0.0, 0, B->smem_fft, s);
-      launch_rows_inv_dot<T>(P, S, L.rows_kry.dev, L.rows_kry.count, 1, B->smem_fft, s);
+      // z = M r into PZ and <r, z>
+      const bool vec_dot = std::is_same<TZ, __nv_bfloat16>::value;     // (stencil_variant)
+      auto inv_dot = [&](int first) {
+        if (vec_dot) {
+          launch_rows_inv<T>(P, S, L.rows_kry.dev, L.rows_kry.count, SL_PZ, !first, B->smem_fft, s);
+          launch_vec<T>(first ? VEC_PCG_RHO0 : VEC_PCG_RHO, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
+        } else {
+          launch_rows_inv_dot<T>(P, S, L.rows_kry.dev, L.rows_kry.count, first, B->smem_fft, s);
+        }
+      };
+      inv_dot(1);
       for (int k = 0; k < maxs; ++k) {
-        launch_stencil<T>(ST_CORR, P, S, L.corr_kry.dev, L.corr_kry.count, SL_PP, SL_V, SL_V, 1, B->st_rows, B->smem_stencil, s);
+        launch_stencil<T>(ST_CORR, P, S, L.corr_kry.dev, L.corr_kry.count, SL_PP, SL_V, SL_V, 1, B->st_variant, B->smem_stencil, s);
         launch_vec<T>(VEC_FOLD, P, S, L.vec_kry_bc.dev, L.vec_kry_bc.count, 1, s);
-        launch_stencil<T>(ST_FWD_PCGQ, P, S, L.blur_kry.dev, L.blur_kry.count, -1, SL_PQ, SL_PP, 1, B->st_rows, B->smem_stencil, s);
+        launch_stencil<T>(ST_FWD_PCGQ, P, S, L.blur_kry.dev, L.blur_kry.count, -1, SL_PQ, SL_PP, 1, B->st_variant, B->smem_stencil, s);
         launch_rows_fwd_step<T>(P, S, L.rows_kry.dev, L.rows_kry.count, k == 0, B->smem_fft, s);
         launch_cols<T>(P, S, L.cols_kry.dev, L.cols_kry.count, COL_FUSED, 1, 0.0, 0, B->smem_fft, s);
-        launch_rows_inv_dot<T>(P, S, L.rows_kry.dev, L.rows_kry.count, 0, B->smem_fft, s);
+        inv_dot(0);
         if (k + 1 < maxs) launch_vec<T>(VEC_PCG_PUPD, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
       }
       launch_vec<T>(VEC_PCG_FINISH, P, S, L.vec_kry.dev, L.vec_kry.count, 1, s);
@@ -411,8 +423,8 @@ void enqueue_step(mlba_batch* B, const StepLists& L, int part, cudaStream_t s) {
   if (part & PART_B) {
     // a6: full correlation of t (A^T up to the BC fold); antireflective BCs:
     // the reblurring A' t into U
-    launch_stencil<T>(ST_CORR, P, S, L.corr.dev, L.corr.count, -1, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, s);
-    launch_stencil<T>(ST_REBLUR, P, S, L.reblur.dev, L.reblur.count, -1, -1, SL_U, 0, B->st_rows, B->smem_stencil, s);
+    launch_stencil<T>(ST_CORR, P, S, L.corr.dev, L.corr.count, -1, SL_V, SL_V, 0, B->st_variant, B->smem_stencil, s);
+    launch_stencil<T>(ST_REBLUR, P, S, L.reblur.dev, L.reblur.count, -1, -1, SL_U, 0, B->st_variant, B->smem_stencil, s);
     // (FFT blur path: t placed at (c, c), or extended antireflectively, and
     // correlated with the PSF)
     if (L.fc_pad_a.count) {
@@ -604,11 +616,11 @@ int build_split(mlba_batch* B) {
 
 int set_smem_attrs(mlba_batch* B) {
   if (B->dtype == MLBA_F64) {
-    CK(stencil_set_smem<double>(B->st_rows));
+    CK(stencil_set_smem<double>(B->st_variant));
     CK(fft_set_smem<double>());
     CK((frame_set_smem<double, double>()));
   } else {
-    CK(stencil_set_smem<float>(B->st_rows));
+    CK(stencil_set_smem<float>(B->st_variant));
     CK(fft_set_smem<float>());
     if (B->z_store == MLBA_BF16) CK((frame_set_smem<float, __nv_bfloat16>()));
     else CK((frame_set_smem<float, float>()));
@@ -656,7 +668,20 @@ void destroy_batch(mlba_batch* B) {
 // rows.  A step, 8 / 4 / 2 rows: 64^2 FP64 114 / 96 / 88 us; 256^2 FP64 L = 4
 // 387 / 308 / 284; 256^2 FP32 83 / 81 / 82; 226^2 FP32 100 / 96 / 95; 512^2 FP32
 // 68 / 68 / 69; 1024^2 FP32 (Algorithm 2) 576 / 593 / 670; 4096^2 1190 / 1258 / 1470.
-int stencil_rows(const mlba_batch* B) {
+//
+// BF16 z rounds every coefficient to 8 bits, so the last bit of any sum before
+// it decides a rounding now and then, and one rounding of a low-pass coefficient
+// moves a pixel by up to 2e-3 of the maximum (L = 1).  A batch with BF16 z
+// therefore keeps one order of its sums whatever its size: 8 rows per thread
+// (the residual norm's partial sums), the row pass of a rank-one PSF first, the
+// masks tap by tap (k_frame.cu), whole transform CTAs and 32 values per thread in
+// the alpha_n sums, and the inner products of Algorithm 2 over vectors.
+// A pass in that order, against the shape-dependent one: 1024^2 Algorithm 1
+// (2 iterations) 249 / 247 us, 256^2 4-NS rank one (8) 854 / 661, 1024^2
+// Algorithm 2 (3) 1604 / 1550, 4096^2 4-NS rank one L = 2 (4) 5113 / 4229, L = 4
+// 6798 / 5898, the 64-problem batch (8) 8064 / 7740.
+int stencil_variant(const mlba_batch* B) {
+  if (B->z_store == MLBA_BF16) return 8 | ST_ROW_FIRST;
   const double resident = B->dtype == MLBA_F64 ? 152.0 : 304.0;
   for (int rows = 8;; rows /= 2) {
     double tiles = 0.0;      // at half the rows
@@ -688,7 +713,11 @@ int transform_fill(const std::vector<HostProb>& v, int launches) {
 // fill: complex values a CTA should hold (at least one transform, at most
 // TR_CAP).
 constexpr int TR_THIN = 1024;   // values per CTA up to which the plan is thin (fft_plan)
-void transform_geometry(Prob& pd, int fill, bool f64) {
+// bf16: BF16 z (stencil_variant): a 4-NS problem's alpha_n sums run over the
+// columns of a CTA, so its CTAs are full ones whatever the batch's size.
+void transform_geometry(Prob& pd, int fill, bool f64, bool bf16) {
+  const bool whole = bf16 && pd.ns;
+  if (whole) fill = TR_CAP;
   const int n = pd.n;
   const int cap = std::max(1, std::min(fill, TR_CAP) / std::max(pd.nfft, n));      // transforms per CTA
   const int pairs = (n + 1) / 2;
@@ -706,7 +735,7 @@ void transform_geometry(Prob& pd, int fill, bool f64) {
     pd.col_g = std::max(1, (units + nb - 1) / nb);
     // DFT: an even number of complex columns where two fit a CTA, so that the
     // passes move them in pairs (16-byte words)
-    if (!dct && (pd.col_g & 1) && std::min(TR_CAP, 2 * fill) / std::max(pd.nfft, n) >= 2)
+    if (!whole && !dct && (pd.col_g & 1) && std::min(TR_CAP, 2 * fill) / std::max(pd.nfft, n) >= 2)
       pd.col_g += pd.col_g == 1 || (pd.col_g + 1) * std::max(pd.nfft, n) <= TR_CAP ? 1 : -1;
     pd.cb = dct ? 2 * pd.col_g : pd.col_g;
     pd.nblk_cols = ((dct ? n : pd.half) + pd.cb - 1) / pd.cb;
@@ -1127,7 +1156,7 @@ int time_blur_paths(mlba_batch* B, int i, float* t_dir, float* t_fft) {
   State* S = B->d_opstates;
   cudaStream_t s = B->stream;
   auto direct = [&] {
-    launch_stencil<T>(ST_FWD_STORE, P, S, L[0].dev, L[0].count, SL_F, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, s);
+    launch_stencil<T>(ST_FWD_STORE, P, S, L[0].dev, L[0].count, SL_F, SL_AUX1, SL_AUX1, 0, B->st_variant, B->smem_stencil, s);
   };
   auto fft = [&] {
     launch_fc_pad<T>(P, S, L[1].dev, L[1].count, 0, SL_F, s);
@@ -1182,7 +1211,7 @@ int build_persist(mlba_batch* B) {
   std::vector<std::vector<PersistStage>> groups;
   auto st = [B](int kind, const ItemList& l) {
     PersistStage p;
-    p.kind = kind; p.count = l.count; p.items = l.dev; p.sync = 0; p.rows = B->st_rows;
+    p.kind = kind; p.count = l.count; p.items = l.dev; p.sync = 0; p.variant = B->st_variant;
     return p;
   };
   groups.push_back({st(PS_RESID, L.blur)});
@@ -1287,18 +1316,19 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
       h.pd.fc = (o.blur_path == 1) ? 1 : 0;       // 2: measured below
     }
   }
-  B->st_rows = stencil_rows(B);
+  B->st_variant = stencil_variant(B);
   for (HostProb& h : B->hp) {
-    h.pd.nblk_blur = stencil_tiles(h.pd.n, B->st_rows);
-    h.pd.nblk_corr = stencil_tiles(h.pd.ne, B->st_rows);
+    h.pd.nblk_blur = stencil_tiles(h.pd.n, B->st_variant);
+    h.pd.nblk_corr = stencil_tiles(h.pd.ne, B->st_variant);
   }
   // transforms per CTA: as many as fit, or fewer so that the batch's row and
   // column passes have about two CTAs per SM
   {
     const int fill = transform_fill(B->hp, 1), ffill = transform_fill(B->fc, 2);   // (forward, adjoint entries)
-    for (HostProb& h : B->hp) transform_geometry(h.pd, fill, o.dtype == MLBA_F64);
-    spec_geometry(B->hp);
-    for (HostProb& h : B->fc) transform_geometry(h.pd, ffill, o.dtype == MLBA_F64);
+    const bool f64 = o.dtype == MLBA_F64, bf16 = B->z_store == MLBA_BF16;
+    for (HostProb& h : B->hp) transform_geometry(h.pd, fill, f64, bf16);
+    spec_geometry(B->hp, bf16);
+    for (HostProb& h : B->fc) transform_geometry(h.pd, ffill, f64, bf16);
   }
   if (o.stream) { B->stream = (cudaStream_t)o.stream; }
   else {
@@ -1489,7 +1519,7 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
     size_t smem_st = 0, smem_fft = 0;
     for (int i = 0; i < count; ++i) {
       const Prob& pd = B->hp[i].pd;
-      const size_t st_b = stencil_smem(B->st_rows, pd.p, pd.sep, pd.nrw, pd.nruns, (int)ts);
+      const size_t st_b = stencil_smem(B->st_variant, pd.p, pd.sep, pd.nrw, pd.nruns, (int)ts);
       smem_st = std::max(smem_st, st_b);
       if (pd.transform != TR_NONE) {
         // (antireflective columns also keep two weighted end values per transform)
@@ -1839,7 +1869,7 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
     if (stage == 0) {
       CK(cudaGraphLaunch(B->exec, s));
     } else if (B->dtype == MLBA_F64) {
-      if (stage == 1) launch_stencil<double>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->st_rows, B->smem_stencil, s);
+      if (stage == 1) launch_stencil<double>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->st_variant, B->smem_stencil, s);
       if (stage == 2) {
         launch_rows_fwd<double>(P, S, B->rows_spec.dev, B->rows_spec.count, SL_R, 0, B->smem_fft, s);
         launch_cols<double>(P, S, B->cols_stat.dev, B->cols_stat.count, COL_FUSED, 0, 0.0, 0, B->smem_fft, s);
@@ -1851,12 +1881,12 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
         launch_ar_rows<double>(P, S, B->ar_rows.dev, B->ar_rows.count, SL_T, 1, 0, B->smem_fft, s);
       }
       if (stage == 3) {
-        launch_stencil<double>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, s);
-        launch_stencil<double>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->st_rows, B->smem_stencil, s);
+        launch_stencil<double>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->st_variant, B->smem_stencil, s);
+        launch_stencil<double>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->st_variant, B->smem_stencil, s);
       }
       if (stage == 4) launch_frame<double, double>(P, S, B->frame.dev, B->frame.count, B->frame.sec, -1, SL_F, nullptr, nullptr, 0.0, B->levels, B->frame_shape, B->frame_seg, s);
     } else {
-      if (stage == 1) launch_stencil<float>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->st_rows, B->smem_stencil, s);
+      if (stage == 1) launch_stencil<float>(ST_FWD_RESID, P, S, B->blur.dev, B->blur.count, SL_F, SL_R, SL_G, 0, B->st_variant, B->smem_stencil, s);
       if (stage == 2) {
         launch_rows_fwd<float>(P, S, B->rows_spec.dev, B->rows_spec.count, SL_R, 0, B->smem_fft, s);
         launch_cols<float>(P, S, B->cols_stat.dev, B->cols_stat.count, COL_FUSED, 0, 0.0, 0, B->smem_fft, s);
@@ -1868,8 +1898,8 @@ int mlba_batch_profile(mlba_batch* B, int stage, int reps, float* ms) {
         launch_ar_rows<float>(P, S, B->ar_rows.dev, B->ar_rows.count, SL_T, 1, 0, B->smem_fft, s);
       }
       if (stage == 3) {
-        launch_stencil<float>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, s);
-        launch_stencil<float>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->st_rows, B->smem_stencil, s);
+        launch_stencil<float>(ST_CORR, P, S, B->corr.dev, B->corr.count, -1, SL_V, SL_V, 0, B->st_variant, B->smem_stencil, s);
+        launch_stencil<float>(ST_REBLUR, P, S, B->reblur.dev, B->reblur.count, -1, -1, SL_U, 0, B->st_variant, B->smem_stencil, s);
       }
       if (stage == 4) {
         if (B->z_store == MLBA_BF16)
@@ -2216,10 +2246,10 @@ int mlba_op_blur(mlba_ctx* c, const void* f, void* out, int on_device) {
   }
   if (B->dtype == MLBA_F64)
     launch_stencil<double>(ST_FWD_STORE, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                           SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
+                           SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_variant, B->smem_stencil, B->stream);
   else
     launch_stencil<float>(ST_FWD_STORE, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                          SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
+                          SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_variant, B->smem_stencil, B->stream);
   CK(cudaGetLastError());
   return copy_out(B, out, pd.buf[SL_AUX1], (size_t)pd.n * pd.n * ts, on_device);
 }
@@ -2248,20 +2278,20 @@ int mlba_op_blur_adjoint(mlba_ctx* c, const void* t, void* out, int on_device) {
     // the reblurring matrix A' (Section 2.2), n x n
     if (B->dtype == MLBA_F64)
       launch_stencil<double>(ST_REBLUR, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                             SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
+                             SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_variant, B->smem_stencil, B->stream);
     else
       launch_stencil<float>(ST_REBLUR, B->d_probs, B->d_opstates, B->blur.dev, B->blur.count,
-                            SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_rows, B->smem_stencil, B->stream);
+                            SL_AUX0, SL_AUX1, SL_AUX1, 0, B->st_variant, B->smem_stencil, B->stream);
     CK(cudaGetLastError());
     return copy_out(B, out, pd.buf[SL_AUX1], (size_t)pd.n * pd.n * ts, on_device);
   }
   if (B->dtype == MLBA_F64) {
     launch_stencil<double>(ST_CORR, B->d_probs, B->d_opstates, B->corr_all.dev, B->corr_all.count,
-                           SL_AUX0, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, B->stream);
+                           SL_AUX0, SL_V, SL_V, 0, B->st_variant, B->smem_stencil, B->stream);
     if (pd.bc != BC_RECT) launch_vec<double>(VEC_FOLD, B->d_probs, B->d_opstates, B->vec_all.dev, B->vec_all.count, 0, B->stream);
   } else {
     launch_stencil<float>(ST_CORR, B->d_probs, B->d_opstates, B->corr_all.dev, B->corr_all.count,
-                          SL_AUX0, SL_V, SL_V, 0, B->st_rows, B->smem_stencil, B->stream);
+                          SL_AUX0, SL_V, SL_V, 0, B->st_variant, B->smem_stencil, B->stream);
     if (pd.bc != BC_RECT) launch_vec<float>(VEC_FOLD, B->d_probs, B->d_opstates, B->vec_all.dev, B->vec_all.count, 0, B->stream);
   }
   CK(cudaGetLastError());

@@ -344,6 +344,27 @@ __device__ bool last_block_reduce(const Prob& pd, State& st, int blk, int nblk,
   return last_block_reduce_b<NT, K>(pd, st, blk, nblk, vals, tot, sh, &is_last, BlkFull{});
 }
 
+// Algorithm 2: the scalars after the inner product rho = <res, M res> (one thread
+// of the problem); first: rho_0, the start of a solve
+__device__ __forceinline__ void pcg_scalars(const Prob& pd, State& st, double rho, bool first) {
+  if (first) {
+    st.prho = rho;
+    st.prho0 = rho;
+    st.psteps = 0;
+    st.pdone = (rho <= 0.0) ? 1 : 0;
+    return;
+  }
+  st.psteps += 1;
+  // relative residual of the symmetric system (psys): sqrt(r_k^T M r_k / r_0^T M r_0)
+  const double rel = sqrt(fmax(rho, 0.0) / st.prho0);
+  if (rel <= pd.pcg_tol || st.psteps >= pd.pcg_max) {
+    st.pdone = 1;
+  } else {
+    st.pbeta = rho / st.prho;
+    st.prho = rho;
+  }
+}
+
 // BC fold of the extended correlation: u(a,b) = sum over the padded positions
 // that copy (a,b) (transpose of the Table 1 padding).
 template <typename T>

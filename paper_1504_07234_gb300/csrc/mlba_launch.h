@@ -31,7 +31,11 @@ void launch_balance(const Prob* probs, State* states, const int2* items, int nit
 enum {
   VEC_FOLD = 0,       // U = BC fold of V
   VEC_PCG_PUPD = 1,   // PP = PZ + beta PP
-  VEC_PCG_FINISH = 2  // T = PX (0 when no step was taken), beta_n recorded
+  VEC_PCG_FINISH = 2, // T = PX (0 when no step was taken), beta_n recorded
+  // BF16 z (else inside the inverse row pass): <res, M res>, each thread's 8
+  // strided terms in T, and the PCG scalars; RHO0: res = r, PP = PZ
+  VEC_PCG_RHO0 = 3,
+  VEC_PCG_RHO = 4
 };
 // column-pass modes (k_fft.cu)
 enum {
@@ -48,6 +52,10 @@ enum { W_INV = 0, W_TIKH = 1 };
 // with larger ones valid (227 KB per CTA less the kernels' static arrays).
 constexpr int SMEM_LIMIT = 220 * 1024;
 constexpr int STENCIL_THREADS = 128;
+// Stencil variant: rows per thread (2, 4, 8), plus ST_ROW_FIRST (8 rows, FP32)
+// where a rank-one PSF's row pass goes first.
+constexpr int ST_ROW_FIRST = 16;
+constexpr int st_rows_of(int variant) { return variant & (ST_ROW_FIRST - 1); }
 constexpr int VEC_THREADS = 256;
 constexpr int VEC_PER_THREAD = 8;
 constexpr int TR_CAP = 4096;          // complex values held by one transform CTA
@@ -60,7 +68,7 @@ constexpr int SPEC_SUMS = 17;        // block sums of the bracketing pass (2 x 8
 
 template <typename T>
 void launch_stencil(int mode, const Prob* probs, State* states, const int2* items, int nitems,
-                    int src, int dst, int aux, int pcg, int rows, size_t smem, cudaStream_t s);
+                    int src, int dst, int aux, int pcg, int variant, size_t smem, cudaStream_t s);
 template <typename T>
 void launch_vec(int mode, const Prob* probs, State* states, const int2* items, int nitems,
                 int pcg, cudaStream_t s);
@@ -112,8 +120,8 @@ int lowpass_rows(int nf);                         // rows per CTA of a low-pass 
 int lowpass_blocks(int nf, int levels);           // CTAs of one low-pass launch
 void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch);
 bool is_frame_kernel(const void* func);  // func is one of the framelet-update kernels
-int stencil_tiles(int outN, int R);      // CTAs of the stencil (R rows per thread) for an outN x outN output
-size_t stencil_smem(int R, int p, int sep, int nrw, int nruns, int elem);   // its shared memory
+int stencil_tiles(int outN, int variant);  // CTAs of the stencil for an outN x outN output
+size_t stencil_smem(int variant, int p, int sep, int nrw, int nruns, int elem);   // its shared memory
 // z layout: the 8 high-pass bands of a level contiguous per position, in
 // the polyphase order of the level's dilation for L >= 3 (z_index);
 // conversion to / from band-major planes
@@ -129,7 +137,7 @@ struct PersistStage {
   int kind, count;
   const int2* items;
   int sync;            // 1: a grid barrier follows (the next stage reads what this one wrote)
-  int rows;            // stencil stages: rows per thread
+  int variant;         // stencil stages
 };
 size_t persist_smem(int dtype_bytes, int zs_bytes, int levels, size_t smem_stencil, size_t smem_fft,
                     int* stencil_slot, int* frame_slot);
@@ -145,7 +153,7 @@ cudaError_t persist_graph_set_k(cudaGraphExec_t x, cudaGraphNode_t knode, int zs
 size_t persist_ctl_bytes();
 int persist_threads();
 template <typename T>
-cudaError_t stencil_set_smem(int rows);
+cudaError_t stencil_set_smem(int variant);
 template <typename T>
 cudaError_t fft_set_smem();
 
