@@ -1363,7 +1363,9 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
         (size_t)pd.nbands * nf2 * zs,          // z1
         nspec * ts * (pd.transform == TR_DCT || pd.transform == TR_AR ? 1 : 2),   // lam
         nspec * ts,                            // |lambda|^2 in T precision
-        (pd.ns ? nspec : 1) * ts,              // 4-NS weighted power
+        // 4-NS weighted power; a context's operator mlba_op_ns_alpha writes it
+        // whatever the algorithm
+        (pd.ns || (count == 1 && pd.transform != TR_AR) ? nspec : 1) * ts,
         (pd.levels >= 3 ? (size_t)(pd.levels - 1) * nf2 : 1) * ts,   // low-pass chain (L >= 3)
         (pd.levels >= 3 ? (size_t)(pd.levels - 1) * nf2 : 1) * ts,   // synthesis partials
         spec ? (size_t)pd.nfft * 2 * ts : ts,  // tw

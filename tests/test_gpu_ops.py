@@ -148,6 +148,38 @@ def test_ns_alpha(M, dtype, transform, psf, n):
     ctx.close()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("precond,transform,psf,n", [("bccb", "dft", "motion7", 100), ("tikh", "dct", "gauss9", 64),
+                                                     ("krylov", "dft", "gauss9", 61), ("sym", "dct", "disk2", 256)])
+def test_ns_alpha_of_any_spectral_context(M, dtype, precond, transform, psf, n):
+    """The operator does not need a 4-NS context: its weighted powers have room
+    in every context with a DFT or DCT spectrum.  It leaves the context as it
+    was: the operators and the iterates after it are those of a fresh one, bit
+    for bit (the powers must not reach the buffers beside them)."""
+    h = PSFS[psf]
+    bc = "reflective" if transform == "dct" else "periodic"
+    r = np.random.default_rng(3).standard_normal((n, n))
+    g = np.random.default_rng(4).uniform(0.0, 1.0, (n, n))
+    out = []
+    for first in (True, False):
+        ctx = M.Context(h, n, bc, precond, dtype=dtype, transform=transform, levels=3, max_iter=4, stop=False)
+        if first:
+            hs = O.symmetrize(h) if precond == "sym" else h
+            pre = O.SpectralPrecond(hs, n, transform)
+            for qn in (0.5, 0.9):
+                ref = O.ns_alpha(np.abs(pre.forward(r)) ** 2, pre.sigma, qn)
+                got = ctx.ns_alpha(r, qn)
+                assert abs(got - ref) <= (1e-10 if dtype == "f64" else 1e-5) * ref, (qn, got, ref)
+        res = [ctx.precond(r, 0.05, "tikh"), ctx.blur(g), ctx.blur_adjoint(r)]
+        ctx.set_data(g, 0.1)
+        ctx.iterate(3)
+        res += [ctx.result(), ctx.history()[0]]
+        out.append([np.asarray(x) for x in res])
+        ctx.close()
+    for k, (x, y) in enumerate(zip(*out)):
+        assert np.array_equal(x, y), k
+
+
 @pytest.mark.parametrize("transform,psf", [("dft", "motion7"), ("dct", "gauss9")])
 def test_precond_largest_prime_length(M, transform, psf):
     """n = 4093, the largest prime below the 4096 limit: one direct-sum pass
