@@ -112,13 +112,15 @@ typedef struct mlba_opts {
                          update overlaps the other's residual and preconditioner; 0 advances
                          the whole batch launch by launch.  The iterates are the same. */
   int autotune;       /* tile shape of the framelet kernel (FP32, levels <= 2): 0 (default) the
-                         built-in shape; 1 measure every candidate shape at create on the
-                         batch's own buffers and keep the fastest, reusing an earlier
-                         measurement from the on-disk cache (MLBA_TUNE_CACHE, else
+                         built-in shape (its row segments follow from the batch's size); 1
+                         measure it and every other candidate at create on the batch's own
+                         buffers and keep the fastest, reusing an earlier measurement from the
+                         on-disk cache (MLBA_TUNE_CACHE, else
                          $XDG_CACHE_HOME/mlba_tune.txt, else $HOME/.cache/mlba_tune.txt; an
                          unwritable cache is skipped); 2 measure, ignoring the cache.  Every
                          shape computes the same values; only the time differs. */
-  int frame_shape;    /* -1 (default): as autotune says; 0 .. MLBA_FRAME_SHAPES - 1: force it */
+  int frame_shape;    /* -1 (default): as autotune says; 0 .. MLBA_FRAME_SHAPES - 1: force it, with
+                         its full 32-row segments (FP32, levels <= 2) */
   int blur_path;      /* how A and A^T (A' for antireflective BCs) are applied (Sections 2.1,
                          2.2): 0 (default) direct stencils with the BCs in the index math;
                          1 FFT convolution on a 2^a 3^b 5^c size M >= n + p - 1 (the input

@@ -1021,30 +1021,30 @@ void tune_store(const std::string& key, int shape, float us) {
   std::fclose(f);
 }
 
-void launch_frame_any(mlba_batch* B, const int2* items, int count, int shape, cudaStream_t s) {
+void launch_frame_any(mlba_batch* B, const int2* items, int count, int shape, int seg, cudaStream_t s) {
   if (B->dtype == MLBA_F64)
     launch_frame<double, double>(B->d_probs, B->d_states, items, count, nullptr, -1, SL_F, nullptr,
-                                 nullptr, 0.0, B->levels, shape, 32, s);
+                                 nullptr, 0.0, B->levels, shape, seg, s);
   else if (B->z_store == MLBA_BF16)
     launch_frame<float, __nv_bfloat16>(B->d_probs, B->d_states, items, count, nullptr, -1, SL_F,
-                                       nullptr, nullptr, 0.0, B->levels, shape, 32, s);
+                                       nullptr, nullptr, 0.0, B->levels, shape, seg, s);
   else
     launch_frame<float, float>(B->d_probs, B->d_states, items, count, nullptr, -1, SL_F, nullptr,
-                               nullptr, 0.0, B->levels, shape, 32, s);
+                               nullptr, 0.0, B->levels, shape, seg, s);
 }
 
-std::vector<int2> frame_items(const mlba_batch* B, int shape) {
+std::vector<int2> frame_items(const mlba_batch* B, int shape, int seg) {
   std::vector<int2> v;
   for (size_t i = 0; i < B->hp.size(); ++i) {
-    const int nb = frame_tiles(B->hp[i].pd.nf, B->levels, shape, 32);
+    const int nb = frame_tiles(B->hp[i].pd.nf, B->levels, shape, seg);
     for (int k = 0; k < nb; ++k) v.push_back(make_int2((int)i, k));
   }
   return v;
 }
 
 // mean microseconds of one framelet launch of `shape` over the whole batch
-int time_frame_shape(mlba_batch* B, int shape, float* us) {
-  const std::vector<int2> items = frame_items(B, shape);
+int time_frame_shape(mlba_batch* B, int shape, int seg, float* us) {
+  const std::vector<int2> items = frame_items(B, shape, seg);
   int2* dev = nullptr;
   CK(cudaMalloc(&dev, items.size() * sizeof(int2)));
   if (cudaMemcpy(dev, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -1055,9 +1055,9 @@ int time_frame_shape(mlba_batch* B, int shape, float* us) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   const int warm = 2, reps = 6;
-  for (int r = 0; r < warm; ++r) launch_frame_any(B, dev, (int)items.size(), shape, B->stream);
+  for (int r = 0; r < warm; ++r) launch_frame_any(B, dev, (int)items.size(), shape, seg, B->stream);
   cudaEventRecord(e0, B->stream);
-  for (int r = 0; r < reps; ++r) launch_frame_any(B, dev, (int)items.size(), shape, B->stream);
+  for (int r = 0; r < reps; ++r) launch_frame_any(B, dev, (int)items.size(), shape, seg, B->stream);
   cudaEventRecord(e1, B->stream);
   const cudaError_t err = cudaEventSynchronize(e1);
   float ms = 0.f;
@@ -1096,12 +1096,15 @@ int frame_segment(const mlba_batch* B) {
 int choose_frame_shape(mlba_batch* B, const mlba_opts& o) {
   B->frame_shape = 0;
   B->frame_tuned = 0;
-  // (a forced or measured shape, and the persistent schedule, keep 32 rows)
-  B->frame_seg = 32;
-  if (B->levels > 2 || (o.frame_shape < 0 && !o.autotune && !o.persistent)) B->frame_seg = frame_segment(B);
+  // Shape 0 has the segments of frame_segment, measured or not; the other
+  // shapes, and a forced one (the persistent schedule forces 0), 32 rows.
+  B->frame_seg = frame_segment(B);
+  const int seg0 = B->frame_seg;
+  auto seg_of = [&](int shape) { return shape == 0 ? seg0 : 32; };
   const bool shaped = B->levels <= 2 && B->dtype != MLBA_F64;   // FP64: one shape
   if (!shaped) return MLBA_OK;
   if (o.frame_shape >= 0) {
+    B->frame_seg = 32;
     B->frame_shape = o.frame_shape;
     B->frame_tuned = 3;
     return MLBA_OK;
@@ -1111,7 +1114,7 @@ int choose_frame_shape(mlba_batch* B, const mlba_opts& o) {
   int sh = 0;
   float us = 0.f;
   if (o.autotune == 1 && tune_lookup(key, &sh, &us)) {
-    B->frame_shape = sh; B->frame_tuned = 2; B->frame_us = us;
+    B->frame_shape = sh; B->frame_seg = seg_of(sh); B->frame_tuned = 2; B->frame_us = us;
     return MLBA_OK;
   }
   // (the timed launches, at iteration 0, read z[1] and write z[0])
@@ -1122,11 +1125,11 @@ int choose_frame_shape(mlba_batch* B, const mlba_opts& o) {
   float tbest = 0.f;
   for (int k = 0; k < FRAME_SHAPES; ++k) {
     float t = 0.f;
-    const int rc = time_frame_shape(B, k, &t);
+    const int rc = time_frame_shape(B, k, seg_of(k), &t);
     if (rc != MLBA_OK) return rc;
     if (k == 0 || t < tbest) { best = k; tbest = t; }
   }
-  B->frame_shape = best; B->frame_tuned = 1; B->frame_us = tbest;
+  B->frame_shape = best; B->frame_seg = seg_of(best); B->frame_tuned = 1; B->frame_us = tbest;
   tune_store(key, best, tbest);
   return MLBA_OK;
 }

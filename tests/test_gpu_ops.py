@@ -268,6 +268,28 @@ def test_transform_ctas_full_and_split(M, n, transform, psf):
     assert rel_err(out[1], out[0]) <= 1e-5
 
 
+@pytest.mark.parametrize("dtype,n,levels", [("f32", 256, 2), ("f32", 128, 1), ("f64", 100, 2), ("f64", 64, 1)])
+def test_autotune_knows_the_short_segments(M, tmp_path, monkeypatch, dtype, n, levels):
+    """A tuned batch of one small image keeps the built-in tile (short row
+    segments, about a third of the time of any 32-row shape), measured or read
+    from the cache; FP64 has one shape, which the option leaves alone."""
+    monkeypatch.setenv("MLBA_TUNE_CACHE", str(tmp_path / "tune.txt"))
+    desc = dict(psf=PSFS["disk2"], g=I.true_image(n, n), delta=0.1, bc="reflective", precond="tikh")
+    tiles, out = [], []
+    for tune in (0, 2, 1):
+        b = M.Batch([desc], dtype=dtype, levels=levels, stop=False, max_iter=3, autotune=tune)
+        tiles.append(b.tiles())
+        b.iterate(2)
+        out.append(b.result(0))
+        b.close()
+    assert tiles[0]["tile_y"] < 64, tiles[0]
+    for t, f in zip(tiles[1:], out[1:]):
+        assert (t["frame_shape"], t["tile_y"], t["prefetch"]) == (0, tiles[0]["tile_y"], tiles[0]["prefetch"]), t
+        assert np.array_equal(f, out[0])
+    if dtype == "f32":
+        assert [t["how"] for t in tiles] == ["default", "measured", "cache"]
+
+
 @pytest.mark.parametrize("dtype,zs", [("f32", "f32"), ("f32", "bf16"), ("f64", "f64")])
 @pytest.mark.parametrize("levels", [1, 2])
 def test_frame_segments_give_the_same_iterates(M, dtype, zs, levels):
