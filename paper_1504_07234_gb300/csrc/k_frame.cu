@@ -1076,6 +1076,15 @@ void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch) {
   *prefetch = F3_SHAPES[shape].ring > 0 ? F3_SHAPES[shape].ring : F3_SHAPES[shape].pf;
 }
 
+// raise when the sweep changes so that shapes may rank differently
+constexpr unsigned F3_SWEEP_VERSION = 2;
+unsigned frame_shapes_id() {
+  unsigned h = 2166136261u ^ F3_SWEEP_VERSION;
+  for (const F3Shape& s : F3_SHAPES)
+    for (int v : {s.nwr, s.pf, s.ring}) h = (h ^ (unsigned)v) * 16777619u;
+  return h;
+}
+
 // Planar (band-major) <-> internal z layout (z_index), elements E of 2, 4 or 8
 // bytes.  A thread moves one pixel's 8 bands of a level: its accesses to the
 // planes are consecutive along the warp, its group is one or more 16-byte

@@ -964,6 +964,8 @@ uint64_t fnv1a(uint64_t h, const void* p, size_t n) {
   return h;
 }
 
+int frame_segment(const mlba_batch* B);
+
 std::string tune_key(const mlba_batch* B) {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -976,10 +978,12 @@ std::string tune_key(const mlba_batch* B) {
     const int v[5] = {hp.pd.n, hp.pd.nf, hp.pd.bc, hp.pd.use_adj, hp.pd.c};
     h = fnv1a(h, v, sizeof(v));
   }
+  // (an entry is about the kernels that were measured: the shape table, the
+  // version of the sweep and the segments of shape 0)
   char buf[320];
-  std::snprintf(buf, sizeof(buf), "frame3 %s sm%d%d dt%d zs%d L%d count%zu h%016llx",
-                name.empty() ? "gpu" : name.c_str(), prop.major, prop.minor, B->dtype, B->z_store,
-                B->levels, B->hp.size(), (unsigned long long)h);
+  std::snprintf(buf, sizeof(buf), "frame3 k%08x.%d %s sm%d%d dt%d zs%d L%d count%zu h%016llx",
+                frame_shapes_id(), frame_segment(B), name.empty() ? "gpu" : name.c_str(), prop.major,
+                prop.minor, B->dtype, B->z_store, B->levels, B->hp.size(), (unsigned long long)h);
   return std::string(buf);
 }
 

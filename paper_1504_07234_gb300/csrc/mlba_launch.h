@@ -119,6 +119,7 @@ int lev_tiles(int nf, int lev, int seg);                   // CTAs of one level 
 int lowpass_rows(int nf);                         // rows per CTA of a low-pass launch (L >= 3)
 int lowpass_blocks(int nf, int levels);           // CTAs of one low-pass launch
 void frame_shape(int shape, int seg, int* tile_x, int* tile_y, int* prefetch);
+unsigned frame_shapes_id();              // of the shape table and the sweep's version
 bool is_frame_kernel(const void* func);  // func is one of the framelet-update kernels
 int stencil_tiles(int outN, int variant);  // CTAs of the stencil for an outN x outN output
 size_t stencil_smem(int variant, int p, int sep, int nrw, int nruns, int elem);   // its shared memory

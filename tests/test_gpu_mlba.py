@@ -633,3 +633,27 @@ def test_tile_shapes_give_identical_iterates(M, zs, tmp_path, monkeypatch):
             assert np.array_equal(f0[i], fk[i]), i
             assert s0[i] == sk[i], i
     assert (tmp_path / "tune.txt").read_text().startswith("frame3 ")
+
+
+def test_tuning_cache_entries_belong_to_the_kernels_measured(M, tmp_path, monkeypatch):
+    """An entry whose key names other kernels (another shape table or version
+    of the sweep, or none) is not taken: the batch measures and adds its own."""
+    path = tmp_path / "tune.txt"
+    monkeypatch.setenv("MLBA_TUNE_CACHE", str(path))
+    p = small("reflective", "tikh", n=60, iters=2)
+    desc = dict(psf=p.psf, g=p.g, delta=p.delta, bc=p.bc, precond=p.precond)
+
+    def how():
+        b = M.Batch([desc], dtype="f32", levels=2, stop=False, max_iter=2, autotune=1)
+        t = b.tiles()
+        b.close()
+        return t["how"]
+
+    assert (how(), how()) == ("measured", "cache")
+    key = path.read_text().split("\t")[0].split(" ")
+    others = [[w for w in key if not w.startswith("k")]]            # the form before kernels were named
+    others.append(["frame3", "k00000000" + key[1][9:]] + key[2:])   # another table
+    for other in others:
+        path.write_text(" ".join(other) + "\t7 1.000\n")
+        assert how() == "measured", other
+        assert how() == "cache"
