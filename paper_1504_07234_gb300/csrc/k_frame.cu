@@ -229,8 +229,10 @@ __device__ __forceinline__ double f3_flip(double v, int m) {
 // the antisymmetric bands.  The masks are applied through their sums and
 // differences: with s = h_a + h_c, d = h_a - h_c,
 //   z0 += s / 4 + h_b / 2,  z1 += (sqrt 2 / 4) d,  z2 += h_b / 2 - s / 4,
-// and the transpose the same way: 14 operations per horizontal mask instead
-// of 19 (FP32: an issue-bound sweep; FP64: the pipe is full).
+// and the transpose the same way: 15 operations per horizontal mask instead
+// of 19 (FP32: an issue-bound sweep; FP64: the pipe is full).  A correction is
+// complete before z is added, so z is rounded once per update at its own
+// magnitude.
 // BF16 z: the masks tap by tap, in one fixed order (the rounding of z to 8 bits
 // makes the last bit of these sums matter, see the host's stencil_variant).
 // PARTS: a row's three shares are summed by themselves and then added to its
@@ -273,17 +275,17 @@ __device__ __forceinline__ void f3_row(const T (&ha)[3], const T (&hb)[3], const
       pc[j] = a2;
       continue;
     }
-    const T s = ha[j] + hc[j], d = ha[j] - hc[j];
+    const T q = T(0.25) * (ha[j] + hc[j]), d = ha[j] - hc[j];
     T x0 = T(0);
     if (j > 0 || LOW) {
       const T v = j == 0 ? T(ld_z(&zl)) : in(0);
-      const T zn = fma(T(0.5), hb[j], fma(T(0.25), s, v));
+      const T zn = v + fma(T(0.5), hb[j], q);
       if (j == 0) zlo = to_z(zn, (TZ*)nullptr);
       else zo.e[j - 1] = to_z(zn, (TZ*)nullptr);
       x0 = f3_soft(zn, mu);
     }
     const T z1 = fma(s2q, d, in(1));
-    const T z2 = fma(T(0.5), hb[j], fma(T(-0.25), s, in(2)));
+    const T z2 = in(2) + fma(T(0.5), hb[j], -q);
     zo.e[3 + j - 1] = to_z(z1, (TZ*)nullptr);
     zo.e[6 + j - 1] = to_z(z2, (TZ*)nullptr);
     const T x1 = f3_soft(z1, mu), x2 = f3_soft(z2, mu);

@@ -268,6 +268,26 @@ def test_transform_ctas_full_and_split(M, n, transform, psf):
     assert rel_err(out[1], out[0]) <= 1e-5
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("levels", [1, 2, 3])
+def test_frame_rounds_z_once(M, dtype, levels):
+    """z + W u has one rounding at the magnitude of z: where z is far larger
+    than u the result is within half a unit in the last place of the exact sum,
+    plus the correction's own rounding (at most 10 additions and products of
+    values up to 2 max |u| per level: 64 eps max |u| for three levels)."""
+    n = 61
+    ft = np.float32 if dtype == "f32" else np.float64
+    rng = np.random.default_rng(17)
+    zi = (rng.choice([-1.0, 1.0], (8 * levels + 1, n, n)) * rng.uniform(1000.0, 2000.0, (8 * levels + 1, n, n))).astype(ft)
+    u = rng.uniform(-1.0, 1.0, (n, n)).astype(ft)
+    ctx = M.Context(PSFS["gauss9"], n, "reflective", "none", dtype=dtype, levels=levels)
+    zo = ctx.frame(zi, u, 0.1)[0].cpu().numpy()
+    ctx.close()
+    ref = zi.astype(np.longdouble) + O.framelet_analysis(u.astype(np.float64), levels).astype(np.longdouble)
+    ulp = np.spacing(np.maximum(np.abs(zo), np.abs(ref.astype(ft))))
+    assert (np.abs(zo - ref) <= 0.5 * ulp + 64 * np.finfo(ft).eps * np.abs(u).max()).all()
+
+
 @pytest.mark.parametrize("dtype,n,levels", [("f32", 256, 2), ("f32", 128, 1), ("f64", 100, 2), ("f64", 64, 1)])
 def test_autotune_knows_the_short_segments(M, tmp_path, monkeypatch, dtype, n, levels):
     """A tuned batch of one small image keeps the built-in tile (short row
