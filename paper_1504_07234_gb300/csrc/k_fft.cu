@@ -1460,28 +1460,32 @@ k_rows_inv(const Prob* __restrict__ probs, State* __restrict__ states, const int
 // First: the first step, whose vectors are x = 0, res = r (not stored).
 //
 // Forward rows: x += a p, res -= a q on this CTA's rows, then the transform of
-// res.  The CTA's own writes are ordered for its loads by the barrier.
+// res.  The CTA's own writes are ordered for its loads by the barrier.  (The
+// update is a function of its own: its pointers are restrict, and the transform
+// reads res through another one.)
+template <typename T, bool FIRST>
+__device__ __forceinline__ void pcg_update(T* __restrict__ px, T* __restrict__ res, const T* __restrict__ r,
+                                           const T* __restrict__ pp, const T* __restrict__ pq, T a, size_t beg,
+                                           size_t end) {
+  constexpr int NT = tr_nt(sizeof(T));
+#pragma unroll 4
+  for (size_t i = beg + threadIdx.x; i < end; i += NT) {
+    px[i] = FIRST ? a * pp[i] : px[i] + a * pp[i];
+    res[i] = (FIRST ? r[i] : res[i]) - a * pq[i];
+  }
+}
 template <typename T, bool FIRST>
 __global__ void __launch_bounds__(tr_nt(sizeof(T)), tr_minb(sizeof(T)))
 k_rows_fwd_step(const Prob* __restrict__ probs, State* states, const int2* __restrict__ items) {
-  constexpr int NT = tr_nt(sizeof(T));
   const int2 item = items[blockIdx.x];
   const Prob& pd = probs[item.x];
   const State& st = states[item.x];
   if (tr_skip(st, 1)) return;
   const int N = pd.n, row0 = 2 * item.y * pd.row_g;
   const size_t beg = (size_t)row0 * N, end = (size_t)min(N, row0 + 2 * pd.row_g) * N;
-  T* __restrict__ px = static_cast<T*>(pd.buf[SL_PX]);
-  T* __restrict__ res = static_cast<T*>(pd.buf[SL_PRES]);
-  const T* __restrict__ r = static_cast<const T*>(pd.buf[SL_R]);
-  const T* __restrict__ pp = static_cast<const T*>(pd.buf[SL_PP]);
-  const T* __restrict__ pq = static_cast<const T*>(pd.buf[SL_PQ]);
-  const T a = T(st.pa);
-#pragma unroll 4
-  for (size_t i = beg + threadIdx.x; i < end; i += NT) {
-    px[i] = FIRST ? a * pp[i] : px[i] + a * pp[i];
-    res[i] = (FIRST ? r[i] : res[i]) - a * pq[i];
-  }
+  pcg_update<T, FIRST>(static_cast<T*>(pd.buf[SL_PX]), static_cast<T*>(pd.buf[SL_PRES]),
+                       static_cast<const T*>(pd.buf[SL_R]), static_cast<const T*>(pd.buf[SL_PP]),
+                       static_cast<const T*>(pd.buf[SL_PQ]), T(st.pa), beg, end);
   __syncthreads();
   rows_fwd_body<T>(item, probs, states, SL_PRES, 1);
 }
