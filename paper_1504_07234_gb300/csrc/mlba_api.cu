@@ -1380,7 +1380,9 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
         spec ? (size_t)pd.n * 2 * ts : ts,     // dtw
         (size_t)pd.nruns * 16, 2 * (size_t)pd.nrw * ts,   // tap runs and weights (both orders)
         (size_t)pd.p * ts, (size_t)pd.p * ts,  // hy, hx
-        std::max({3 * (size_t)pd.nblk_blur, 3 * (size_t)pd.nblk_vec, (size_t)SPEC_SUMS * std::max(pd.nblk_spec, pd.nblk_cols), (size_t)1}) * 8,  // partial
+        // partial sums: stencils, vectors, the alpha_n passes, the row passes of Algorithm 2
+        std::max({3 * (size_t)pd.nblk_blur, 3 * (size_t)pd.nblk_vec,
+                  (size_t)SPEC_SUMS * std::max(pd.nblk_spec, pd.nblk_cols), (size_t)pd.nblk_rows, (size_t)1}) * 8,
         (size_t)(pd.max_iter + 2) * 8, (size_t)(pd.max_iter + 2) * 8, (size_t)(pd.max_iter + 2) * 4};
     szs[i] = sz;
   }
