@@ -362,6 +362,10 @@ class Context(_Base):
                                       ctypes.c_void_p(uu.data_ptr()), ctypes.c_void_p(zo.data_ptr()),
                                       ctypes.c_void_p(f.data_ptr()), float(mu), 1), "mlba_op_frame")
         self._leave()
+        # (the call does not wait: inputs allocated on another stream than the
+        # current one must outlive the work enqueued here)
+        zi.record_stream(self.stream)
+        uu.record_stream(self.stream)
         return zo, f
 
     def ns_alpha(self, r, qn):

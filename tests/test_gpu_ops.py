@@ -288,6 +288,38 @@ def test_frame_rounds_z_once(M, dtype, levels):
     assert (np.abs(zo - ref) <= 0.5 * ulp + 64 * np.finfo(ft).eps * np.abs(u).max()).all()
 
 
+def test_frame_inputs_of_another_stream(M):
+    """The operator reads its inputs after the call has returned.  Inputs that
+    were allocated on a side stream and are dropped right after the call are
+    not handed out again by the allocator while the context's stream is busy."""
+    import torch
+    n, levels = 90, 2
+    ctx = M.Context(PSFS["gauss9"], n, "reflective", "none", dtype="f32", levels=levels)
+    rng = np.random.default_rng(6)
+    zh = rng.standard_normal((8 * levels + 1, n, n)).astype(np.float32)
+    uh = rng.standard_normal((n, n)).astype(np.float32)
+    want = [t.cpu() for t in ctx.frame(zh, uh, 0.3)]
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        z, u = torch.from_numpy(zh).cuda(), torch.from_numpy(uh).cuda()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(ctx.stream):
+        torch.cuda._sleep(50_000_000)                # some 25 ms before the operator starts
+    got = ctx.frame(z, u, 0.3)
+    old = (z.data_ptr(), u.data_ptr())
+    shapes = (z.shape, u.shape)
+    del z, u
+    with torch.cuda.stream(side):
+        new = [torch.empty(s, device="cuda") for s in shapes]       # (no launch before both are there)
+        for t in new:
+            t.fill_(7.0)
+    assert not set(old) & {t.data_ptr() for t in new}
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a.cpu(), b)
+    ctx.close()
+
+
 @pytest.mark.parametrize("dtype,n,levels", [("f32", 256, 2), ("f32", 128, 1), ("f64", 100, 2), ("f64", 64, 1)])
 def test_autotune_knows_the_short_segments(M, tmp_path, monkeypatch, dtype, n, levels):
     """A tuned batch of one small image keeps the built-in tile (short row
