@@ -589,3 +589,63 @@ def test_lowpass_chunks(M, dtype, levels, n):
     assert rel_err(f.double().cpu().numpy(), O.framelet_synthesis(O.soft(z_ref, 0.03), levels)) <= (
         1e-11 if dtype == "f64" else 1e-5)
     ctx.close()
+
+
+def fp64_plan(n, count):
+    """The launch rules of a batch of `count` FP64 4-NS problems of size n (DCT):
+    (radix-16 plan, spectral values per thread of an alpha_n pass)."""
+    pairs = (n + 1) // 2
+    cap = max(1, min(4096, int(count * pairs * n / 304)) // n)
+    g = -(-pairs // -(-pairs // cap))                        # transforms per CTA
+    padded = -(-n // (2 * g)) * 2 * g                        # columns, whole blocks
+    return g * n > 1024, 8 if count * n * padded <= 152 * 256 * 8 else 32
+
+
+@pytest.mark.parametrize("n,count,plan", [(64, 1, (False, 8)), (256, 4, (False, 8)), (256, 6, (False, 32)),
+                                          (250, 5, (False, 32)), (256, 50, (True, 32)), (300, 40, (True, 32)),
+                                          (96, 400, (True, 32))])
+def test_fp64_plans_of_every_batch_size(M, n, count, plan):
+    """FP64 4-NS batches on both sides of the two lines: radix-4 or radix-16 plans
+    (more than 1024 values per CTA), 8 or 32 spectral values per thread (more than
+    one CTA per SM at 8).  The first and last images against the oracle."""
+    assert fp64_plan(n, count) == plan
+    h = I.psf_disk(2)
+    f = I.true_image(n + h.shape[0] - 1, n)
+    g, delta = I.observe(f, h, 0.02, n)
+    desc = dict(psf=h, g=g, delta=delta, bc="reflective", precond="tikh_ns", transform="dct")
+    b = M.Batch([desc] * count, dtype="f64", levels=1, stop=False, max_iter=4)
+    b.iterate(2)
+    ref = O.mlba(g, h, delta, "reflective", "tikh_ns", 10 / 255, 0.05, 1, 2, stop=False, transform="dct")
+    for i in (0, count - 1):
+        assert rel_err(b.result(i), ref["f"]) <= 1e-9
+    b.close()
+
+
+@pytest.mark.parametrize("dtype,zs", [("f32", "f32"), ("f32", "bf16"), ("f64", "f64")])
+@pytest.mark.parametrize("levels", [3, 4])
+@pytest.mark.parametrize("two_group", [True, False])
+def test_lowpass_rows_of_a_mixed_batch(M, dtype, zs, levels, two_group):
+    """One batch with images on both sides of the width (1216) from which the
+    low-pass chain takes eight rows per CTA: both sections of the frame list are
+    launched, in both groups.  Every image ends with the bits it has alone (the
+    algorithms here have no sum that depends on the launch geometry); in FP64,
+    where the radix plan depends on the batch, within 1e-12."""
+    descs = []
+    for k, (n, bc, precond) in enumerate([(1216, "reflective", "tikh"), (90, "rect", "bccb"),
+                                          (1217, "periodic", "bccb"), (1220, "reflective", "tikh"),
+                                          (57, "reflective", "tikh")]):
+        descs.append(dict(psf=PSFS["disk2" if k % 2 else "gauss9"], g=I.true_image(n, n), delta=0.1, bc=bc,
+                          precond=precond, alpha=0.3))
+    kw = dict(dtype=dtype, z_store=zs, levels=levels, stop=False, max_iter=3, two_group=two_group)
+    b = M.Batch(descs, **kw)
+    b.iterate(2)
+    got = [b.result(i) for i in range(len(descs))]
+    b.close()
+    for i, d in enumerate(descs):
+        one = M.Batch([d], **kw)
+        one.iterate(2)
+        if dtype == "f64":
+            assert rel_err(got[i], one.result(0)) <= 1e-12, i
+        else:
+            assert np.array_equal(one.result(0), got[i]), i
+        one.close()
