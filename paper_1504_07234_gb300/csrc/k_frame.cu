@@ -820,10 +820,6 @@ struct LV {
   static constexpr int TY = SEG;
   static constexpr int CW = 34, CH = TY + 4;      // c tile: positions tx0 - 2.., ty0 - 2..
 };
-template <typename T, int SEG>
-__host__ __device__ constexpr size_t lev_smem_bytes() {
-  return (size_t)LV<SEG>::CW * LV<SEG>::CH * sizeof(T);
-}
 // tiles of one sub-lattice pair and of the whole level
 __host__ __device__ inline void lev_tile_grid(int nf, int dp, int seg, int* tx, int* ty) {
   const int m = Poly(nf, dp).count_max();

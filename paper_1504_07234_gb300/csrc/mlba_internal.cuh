@@ -123,7 +123,6 @@ template <typename T2> __device__ __forceinline__ T2 csub(T2 a, T2 b) { a.x -= b
 template <typename T2> __device__ __forceinline__ T2 cmul(T2 a, T2 b) {
   T2 r; r.x = a.x * b.x - a.y * b.y; r.y = a.x * b.y + a.y * b.x; return r;
 }
-template <typename T2> __device__ __forceinline__ T2 cconj(T2 a) { a.y = -a.y; return a; }
 
 // storage conversions for z
 __device__ __forceinline__ float ld_z(const float* p) { return *p; }
@@ -156,15 +155,6 @@ __device__ __forceinline__ int refl_half(int e, int n, int* odd) {
 // bring the 128-byte line of p into L2 (no registers, no wait)
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-// L2 prefetch of every 128-byte line of [p, p + bytes) by the threads
-// tid = 0 .. nt - 1 of a group
-__device__ __forceinline__ void prefetch_range(const void* p, size_t bytes, int tid, int nt) {
-  const size_t a0 = reinterpret_cast<size_t>(p) & ~size_t(127);
-  const size_t a1 = reinterpret_cast<size_t>(p) + bytes;
-  for (size_t a = a0 + (size_t)tid * 128; a < a1; a += (size_t)nt * 128)
-    prefetch_l2(reinterpret_cast<const void*>(a));
 }
 
 // n / d by a multiply-high: m = floor((2^32 - 1) / d) + 1 gives the exact
@@ -205,21 +195,6 @@ struct Poly {
     if (p < big) { a = p / (Q + 1); m = p - a * (Q + 1); }
     else { const int r = p - big; a = R + r / Q; m = r - (a - R) * Q; }
     return a + (m << sh);
-  }
-};
-
-// Poly::inv with the two quotients by multiply-high (device code)
-struct PolyInv {
-  Poly P;
-  FastDiv q1, q0;
-  int big;
-  __device__ __forceinline__ PolyInv(int nf, int d)
-      : P(nf, d), q1(P.Q + 1), q0(P.Q > 0 ? P.Q : 1), big(P.R * (P.Q + 1)) {}
-  __device__ __forceinline__ int inv(int p) const {
-    int a, m;
-    if (p < big) { a = q1.div(p); m = p - a * (P.Q + 1); }
-    else { const int r = p - big; const int k = q0.div(r); a = P.R + k; m = r - k * P.Q; }
-    return a + (m << P.sh);
   }
 };
 
@@ -275,32 +250,6 @@ __device__ __forceinline__ double block_sum_b(double v, double* sh, BLK b) {
 template <int NT>
 __device__ __forceinline__ double block_sum(double v, double* sh) {
   return block_sum_b<NT>(v, sh, BlkFull{});
-}
-
-// block-wide sums of K doubles with one barrier: warp shuffles, then one
-// thread per value sums the warp partials in warp order (results in thread 0's
-// out[] after the call; every thread must call)
-template <int NT, int K>
-__device__ __forceinline__ void block_sum_k(double (&v)[K], double (&out)[K], double* sh) {
-  constexpr int NW = NT / 32;
-#pragma unroll
-  for (int k = 0; k < K; ++k)
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) sh[k * NW + w] = v[k];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double s = 0.0;
-      for (int i = 0; i < NW; ++i) s += sh[k * NW + i];
-      out[k] = s;
-    }
-  }
 }
 
 // Last-block reduction: every block of problem `pi` calls this with its K
