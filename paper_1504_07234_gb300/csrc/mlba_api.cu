@@ -694,17 +694,25 @@ int stencil_variant(const mlba_batch* B) {
 // `launches` launches each.
 // A CTA is a chain of barrier-separated phases, so a launch with fewer CTAs
 // than the chip has SMs takes as long as its fullest CTA: below TR_FILL_CTAS
-// full CTAs the transforms spread over more of them instead.  Both sides of the line
+// full CTAs the transforms spread over more of them instead (about two per SM of a
+// batch of one; the launches of a batch of several hold one group's or one kind's
+// share of them).  Both sides of the line
 // (one CTA holding up to TR_CAP values against 2 per SM; a pass measured alone):
 // 256^2 DCT rows 10.5 -> 6.7 us, forward columns with the candidate sums 29.5
 // -> 18 us; 256^2 FP64 columns 111 -> 36 us (20 in radix 4); 1000^2 DFT, all three passes
 // 48 -> 40 us.  The 64-problem batch has 2400 full CTAs and keeps them (the
 // split measured no gain there).
-constexpr int TR_FILL_CTAS = 304;
-int transform_fill(const std::vector<HostProb>& v, int launches) {
+// FP64: one CTA of 512 threads is resident per SM, so more CTAs than SMs are more
+// waves: full ones stay where they already fill two thirds of the chip
+// (TR_FULL64).  The preconditioner's passes, full / split: 900^2 DFT 226 / 208 us,
+// 4-NS DCT 276 / 257; 960^2 213 / 258, 267 / 325; 1024^2 206 / 272, 260 / 336;
+// 1280^2 418 / 443, 520 / 543.
+constexpr int TR_FILL_CTAS = 304, TR_FULL64 = 104;
+int transform_fill(const std::vector<HostProb>& v, int launches, bool f64) {
   double elems = 0.0;
   for (const HostProb& h : v)
     if (h.pd.transform != TR_NONE) elems += (double)((h.pd.n + 1) / 2) * h.pd.nfft;
+  if (f64 && elems / launches > (double)TR_FULL64 * TR_CAP) return TR_CAP;
   return (int)std::min<double>(TR_CAP, elems / launches / TR_FILL_CTAS);
 }
 
@@ -733,9 +741,10 @@ void transform_geometry(Prob& pd, int fill, bool f64, bool bf16) {
     const int units = dct ? pairs : pd.half;           // complex columns to transform
     const int nb = (units + cap - 1) / cap;
     pd.col_g = std::max(1, (units + nb - 1) / nb);
-    // DFT: an even number of complex columns where two fit a CTA, so that the
-    // passes move them in pairs (16-byte words)
-    if (!whole && !dct && (pd.col_g & 1) && std::min(TR_CAP, 2 * fill) / std::max(pd.nfft, n) >= 2)
+    // FP32 DFT: an even number of complex columns where two fit a CTA, so that the
+    // passes move them in pairs (16-byte words; an FP64 value is one, and one
+    // column per CTA keeps the thin plan: 768^2, three passes 158 us, 210 in pairs)
+    if (!whole && !dct && !f64 && (pd.col_g & 1) && std::min(TR_CAP, 2 * fill) / std::max(pd.nfft, n) >= 2)
       pd.col_g += pd.col_g == 1 || (pd.col_g + 1) * std::max(pd.nfft, n) <= TR_CAP ? 1 : -1;
     pd.cb = dct ? 2 * pd.col_g : pd.col_g;
     pd.nblk_cols = ((dct ? n : pd.half) + pd.cb - 1) / pd.cb;
@@ -1331,8 +1340,8 @@ int create_batch(const mlba_problem* probs, int count, const mlba_opts* opts_in,
   // transforms per CTA: as many as fit, or fewer so that the batch's row and
   // column passes have about two CTAs per SM
   {
-    const int fill = transform_fill(B->hp, 1), ffill = transform_fill(B->fc, 2);   // (forward, adjoint entries)
     const bool f64 = o.dtype == MLBA_F64, bf16 = B->z_store == MLBA_BF16;
+    const int fill = transform_fill(B->hp, 1, f64), ffill = transform_fill(B->fc, 2, f64);   // (forward, adjoint entries)
     for (HostProb& h : B->hp) transform_geometry(h.pd, fill, f64, bf16);
     spec_geometry(B->hp, bf16);
     for (HostProb& h : B->fc) transform_geometry(h.pd, ffill, f64, bf16);
