@@ -674,7 +674,7 @@ void destroy_batch(mlba_batch* B) {
 // moves a pixel by up to 2e-3 of the maximum (L = 1).  A batch with BF16 z
 // therefore keeps one order of its sums whatever its size: 8 rows per thread
 // (the residual norm's partial sums), the row pass of a rank-one PSF first, the
-// masks tap by tap (k_frame.cu), whole transform CTAs and 32 values per thread in
+// masks tap by tap (k_frame.cu), full column CTAs and 32 values per thread in
 // the alpha_n sums, and the inner products of Algorithm 2 over vectors.
 // A pass in that order, against the shape-dependent one: 1024^2 Algorithm 1
 // (2 iterations) 249 / 247 us, 256^2 4-NS rank one (8) 854 / 661, 1024^2
@@ -722,12 +722,12 @@ int transform_fill(const std::vector<HostProb>& v, int launches, bool f64) {
 // TR_CAP).
 constexpr int TR_THIN = 1024;   // values per CTA up to which the plan is thin (fft_plan)
 // bf16: BF16 z (stencil_variant): a 4-NS problem's alpha_n sums run over the
-// columns of a CTA, so its CTAs are full ones whatever the batch's size.
+// columns of a CTA, so its column CTAs are full ones whatever the batch's size.
 void transform_geometry(Prob& pd, int fill, bool f64, bool bf16) {
   const bool whole = bf16 && pd.ns;
-  if (whole) fill = TR_CAP;
   const int n = pd.n;
   const int cap = std::max(1, std::min(fill, TR_CAP) / std::max(pd.nfft, n));      // transforms per CTA
+  const int ccap = whole ? TR_CAP / std::max(pd.nfft, n) : cap;                    // column pass
   const int pairs = (n + 1) / 2;
   {
     const int nb = (pairs + cap - 1) / cap;            // row CTAs, then pairs spread evenly
@@ -739,7 +739,7 @@ void transform_geometry(Prob& pd, int fill, bool f64, bool bf16) {
     // (real spectra, DCT and antireflective, move real columns in pairs)
     const bool dct = pd.transform == TR_DCT || pd.transform == TR_AR;
     const int units = dct ? pairs : pd.half;           // complex columns to transform
-    const int nb = (units + cap - 1) / cap;
+    const int nb = (units + ccap - 1) / ccap;
     pd.col_g = std::max(1, (units + nb - 1) / nb);
     // FP32 DFT: an even number of complex columns where two fit a CTA, so that the
     // passes move them in pairs (16-byte words; an FP64 value is one, and one
