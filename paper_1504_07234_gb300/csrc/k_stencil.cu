@@ -109,62 +109,71 @@ template <> struct Pair<double> {
   }
 };
 
+// single values with the same weights (the row pass of the row-first order)
+template <typename T> struct One {
+  using type = T;
+  using weight = typename Pair<T>::weight;
+  static __device__ __forceinline__ float fma(float a, float2 w, float acc) { return fmaf(a, w.x, acc); }
+  static __device__ __forceinline__ double fma(double a, double w, double acc) { return ::fma(a, w, acc); }
+};
+
 // B taps t .. t + B - 1 of a run for R outputs: acc[j] += w[t + u] v[t + u + j].
 // The window is a ring: slot (ROT + j) % R holds v[t + j] on entry, slot
 // (ROT + B + j) % R holds v[t + B + j] on exit, so every register index is static
 // and no value moves (copying the window cost 400 of 2700 instructions per warp
 // at 31 taps).  The value past the last tap's reach is not loaded.
-template <typename T, int R, int B, int ROT, typename LD>
-__device__ __forceinline__ void window_taps(typename Pair<T>::type (&acc)[R], typename Pair<T>::type (&win)[R],
-                                            const typename Pair<T>::weight* __restrict__ w, int t, int len,
+template <typename P, int R, int B, int ROT, typename LD>
+__device__ __forceinline__ void window_taps(typename P::type (&acc)[R], typename P::type (&win)[R],
+                                            const typename P::weight* __restrict__ w, int t, int len,
                                             LD ld) {
 #pragma unroll
   for (int u = 0; u < B; ++u) {
-    const typename Pair<T>::weight wt = w[t + u];
+    const typename P::weight wt = w[t + u];
 #pragma unroll
-    for (int j = 0; j < R; ++j) acc[j] = Pair<T>::fma(win[(ROT + u + j) % R], wt, acc[j]);
+    for (int j = 0; j < R; ++j) acc[j] = P::fma(win[(ROT + u + j) % R], wt, acc[j]);
     if (u + 1 < B || t + B < len) win[(ROT + u) % R] = ld(t + u + R);
   }
 }
-template <typename T, int R, int ROT, typename LD>
-__device__ __forceinline__ void window_tail3(typename Pair<T>::type (&acc)[R], typename Pair<T>::type (&win)[R],
-                                             const typename Pair<T>::weight* __restrict__ w, int t, int len,
+template <typename P, int R, int ROT, typename LD>
+__device__ __forceinline__ void window_tail3(typename P::type (&acc)[R], typename P::type (&win)[R],
+                                             const typename P::weight* __restrict__ w, int t, int len,
                                              LD ld) {
   if (t + 2 <= len) {
-    window_taps<T, R, 2, ROT>(acc, win, w, t, len, ld);
-    if (t + 2 < len) window_taps<T, R, 1, ROT + 2>(acc, win, w, t + 2, len, ld);
+    window_taps<P, R, 2, ROT>(acc, win, w, t, len, ld);
+    if (t + 2 < len) window_taps<P, R, 1, ROT + 2>(acc, win, w, t + 2, len, ld);
   } else if (t < len) {
-    window_taps<T, R, 1, ROT>(acc, win, w, t, len, ld);
+    window_taps<P, R, 1, ROT>(acc, win, w, t, len, ld);
   }
 }
 
 // acc[j] += sum_t w[t] v[t + j], j < R, over a run of len taps, v[i] = ld(i)
-// pairs of values: blocks of 8 (R = 8) or 4 taps, then the rest by halves.
-template <typename T, int R, typename LD>
-__device__ __forceinline__ void window_run(typename Pair<T>::type (&acc)[R],
-                                           const typename Pair<T>::weight* __restrict__ w, int len, LD ld) {
+// (P: pairs of values, or single ones): blocks of 8 (R = 8) or 4 taps, then the
+// rest by halves.
+template <typename P, int R, typename LD>
+__device__ __forceinline__ void window_run(typename P::type (&acc)[R],
+                                           const typename P::weight* __restrict__ w, int len, LD ld) {
   constexpr int B0 = R >= 8 ? 8 : 4;       // a multiple of R: the ring is aligned after a block
-  typename Pair<T>::type win[R];
+  typename P::type win[R];
 #pragma unroll
   for (int j = 0; j < R; ++j) win[j] = ld(j);
   int t = 0;
 #pragma unroll 1
-  for (; t + B0 <= len; t += B0) window_taps<T, R, B0, 0>(acc, win, w, t, len, ld);
+  for (; t + B0 <= len; t += B0) window_taps<P, R, B0, 0>(acc, win, w, t, len, ld);
   if constexpr (B0 == 8) {
     if (t + 4 <= len) {
-      window_taps<T, R, 4, 0>(acc, win, w, t, len, ld);
-      window_tail3<T, R, 4>(acc, win, w, t + 4, len, ld);
+      window_taps<P, R, 4, 0>(acc, win, w, t, len, ld);
+      window_tail3<P, R, 4>(acc, win, w, t + 4, len, ld);
       return;
     }
   }
-  window_tail3<T, R, 0>(acc, win, w, t, len, ld);
+  window_tail3<P, R, 0>(acc, win, w, t, len, ld);
 }
 
 // Stencil tile geometry: 64 x 4 R outputs per CTA of 128 threads; a thread
 // owns two neighbouring columns over R rows.  The input tile (4 R + p - 1) x
 // (64 + p - 1) lives in shared memory with an even row pitch (pairs of columns
 // are one 8-byte word when the column is even).  R = 8 reuses each loaded value
-// most; small images take fewer rows per thread (the host's stencil_rows).
+// most; small images take fewer rows per thread (the host's stencil_variant).
 constexpr int ST_TX = 64;
 // row pitch of the input tile: a multiple of 16 bytes with room for the
 // shift (< 16 bytes) that aligns a row's source to 16 bytes
@@ -177,7 +186,7 @@ __host__ __device__ constexpr int st_tpitch(int RX, int elem) { return (st_pitch
 // rank-one PSF, row pass first: pitch of its result, and whether that needs a
 // tile of its own (else the rows fit the threads' registers and overwrite the input)
 constexpr int ST_RP = ST_TX + 2;
-__host__ __device__ constexpr bool st_rows_tile(int RY) { return 4 * RY > 2 * STENCIL_THREADS; }
+__host__ __device__ constexpr bool st_rows_tile(int RY) { return 8 * RY > 4 * STENCIL_THREADS; }
 // shared memory of a tile: weights, runs (general PSF), the source rows
 // and columns of the tile, input tile (which the
 // column-pass result and the output tile of a rank-one PSF overwrite)
@@ -213,9 +222,9 @@ size_t stencil_smem(int variant, int p, int sep, int nrw, int nruns, int elem) {
 //    windows, over the tile's 64 + p - 1 columns), kept in registers and written
 //    over the input tile as pairs of rows, then the row pass on the row pairs
 //    (R-column windows): both passes are paired FMAs on conflict-free loads.
-//    Row pass first (ROWF; 32 + p - 1 rows for 32, four-way conflicting loads:
-//    4096^2, p = 31, FP32 z: residual 166 us against 126): problems whose z is
-//    BF16, see st_variant.
+//    Row pass first (ROWF; 32 + p - 1 rows for 32, single values, four-way
+//    conflicting loads: 4096^2, p = 33, residual and correlation 147 + 131 us): z in
+//    BF16 (the host's stencil_variant).
 // Forward (A f)(y, x) = sum_{a,b} H[a][b] f_ext(y + c - a, x + c - b); the
 // correlation (ne x ne) is sum_{a,b} H[a][b] t(y - 2c + a, x - 2c + b).
 // (FP32: 8 CTAs per SM, 64 registers; the tile of the largest PSF of a batch
@@ -399,45 +408,46 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
   for (int j = 0; j < R; ++j) { acc[j].x = T(0); acc[j].y = T(0); }
   if (ROWF && sep) {
     // row pass: h(y, x) = sum_t wx[t] in(y, x + t), an item being 8 columns of a
-    // row pair; written over the input tile (row y at the start of its row) once
-    // every thread holds its items, or into a tile of its own
+    // row; written over the input tile (row y at the start of its row) once every
+    // thread holds its items, or into a tile of its own.  (Two rows at a time as
+    // pairs: 4096^2, p = 33, 226 + 215 us for the residual and the correlation.)
     static_assert(!ROWF || R == 8, "row pass first: 8 rows per thread");
-    constexpr int RND = 2;
-    auto rows = [&](int it, T2 (&h)[8]) {
-      const T* base = s_in + 2 * (it >> 3) * RP + xs + (it & 7) * 8;
+    constexpr int RND = 4;
+    auto row = [&](int it, T (&h)[8]) {
+      const T* base = s_in + (it >> 3) * RP + xs + (it & 7) * 8;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { h[j].x = T(0); h[j].y = T(0); }
-      window_run<T, 8>(h, s_w, p, [&](int q) { T2 v; v.x = base[q]; v.y = base[RP + q]; return v; });
+      for (int j = 0; j < 8; ++j) h[j] = T(0);
+      window_run<One<T>, 8>(h, s_w, p, [&](int q) { return base[q]; });
     };
-    auto put = [&](int it, const T2 (&h)[8], T* to, int pitch) {
-      T* d = to + 2 * (it >> 3) * pitch + (it & 7) * 8;
+    auto put = [&](int it, const T (&h)[8], T* to, int pitch) {
+      T* d = to + (it >> 3) * pitch + (it & 7) * 8;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { d[j] = h[j].x; d[pitch + j] = h[j].y; }
+      for (int j = 0; j < 8; ++j) d[j] = h[j];
     };
     T* hb = s_in;
     int hp = RP;
     if (!st_rows_tile(RY)) {
-      T2 h[RND][8];
+      T h[RND][8];
 #pragma unroll
       for (int i = 0; i < RND; ++i)
-        if (tid + i * NT < 4 * RY) rows(tid + i * NT, h[i]);
+        if (tid + i * NT < 8 * RY) row(tid + i * NT, h[i]);
       blk.sync();
 #pragma unroll
       for (int i = 0; i < RND; ++i)
-        if (tid + i * NT < 4 * RY) put(tid + i * NT, h[i], hb, hp);
+        if (tid + i * NT < 8 * RY) put(tid + i * NT, h[i], hb, hp);
     } else {
       hb = s_in + RY * RP;
       hp = ST_RP;
-      for (int it = tid; it < 4 * RY; it += NT) {
-        T2 h[8];
-        rows(it, h);
+      for (int it = tid; it < 8 * RY; it += NT) {
+        T h[8];
+        row(it, h);
         put(it, h, hb, hp);
       }
     }
     blk.sync();
     // column pass: out(y, x) = sum_t wy[t] h(y + t, x)
     hb += y8 * hp + x2;
-    window_run<T, R>(acc, s_w + p, p, [&](int q) { return *reinterpret_cast<const T2*>(hb + q * hp); });
+    window_run<Pair<T>, R>(acc, s_w + p, p, [&](int q) { return *reinterpret_cast<const T2*>(hb + q * hp); });
   } else if (sep) {
     // column pass: tmp(y, c) = sum_t wy[t] in(y + t, c) for the tile's columns
     // in pairs, an item being R rows of a pair.  Pairs are aligned in shared
@@ -458,9 +468,9 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
         const int gr = fnp.div(it), cp = it - gr * np;
         const T* base = s_in + (gr * R) * RP + c0 + 2 * cp;
         if (al)
-          window_run<T, R>(tv[i], s_w + p, p, [&](int q) { return *reinterpret_cast<const T2*>(base + q * RP); });
+          window_run<Pair<T>, R>(tv[i], s_w + p, p, [&](int q) { return *reinterpret_cast<const T2*>(base + q * RP); });
         else
-          window_run<T, R>(tv[i], s_w + p, p, [&](int q) { T2 v; v.x = base[q * RP]; v.y = base[q * RP + 1]; return v; });
+          window_run<Pair<T>, R>(tv[i], s_w + p, p, [&](int q) { T2 v; v.x = base[q * RP]; v.y = base[q * RP + 1]; return v; });
       }
     }
     blk.sync();
@@ -488,7 +498,7 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
     constexpr int NRP = ST_TY / 2;               // row pairs of the tile; 64 / R column groups
     const int rp = tid % NRP, xg = (tid / NRP) * R;
     const T2* hb = tmp + rp * TP + (xs - c0) + xg;
-    window_run<T, R>(acc, s_w, p, [&](int q) { return hb[q]; });
+    window_run<Pair<T>, R>(acc, s_w, p, [&](int q) { return hb[q]; });
     blk.sync();
     // to the epilogue's layout (two columns x R rows) through shared memory
     constexpr int OP = ST_TX + 2;
@@ -511,7 +521,7 @@ __device__ __forceinline__ void stencil_body(const int2 item, const Prob* __rest
       const int r0 = CORR ? y8 + rn.y : y8 + 2 * c - rn.z;
       const T* base = s_in + r0 * RP + xs + col;
       const bool aligned = ((xs + col) & 1) == 0;
-      window_run<T, R>(acc, s_w + rn.w, len, [&](int q) -> T2 {
+      window_run<Pair<T>, R>(acc, s_w + rn.w, len, [&](int q) -> T2 {
         const T* v = base + q * RP;
         if (aligned) return *reinterpret_cast<const T2*>(v);
         T2 o; o.x = v[0]; o.y = v[1]; return o;

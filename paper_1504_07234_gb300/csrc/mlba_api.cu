@@ -665,9 +665,11 @@ void destroy_batch(mlba_batch* B) {
 // chip; with fewer than about two tiles per SM a launch lasts as long as one
 // tile, and in FP64, whose pipe one warp per scheduler fills, as long as the
 // fullest scheduler: then the smallest height whose tiles still fit, down to 2
-// rows.  A step, 8 / 4 / 2 rows: 64^2 FP64 114 / 96 / 88 us; 256^2 FP64 L = 4
-// 387 / 308 / 284; 256^2 FP32 83 / 81 / 82; 226^2 FP32 100 / 96 / 95; 512^2 FP32
-// 68 / 68 / 69; 1024^2 FP32 (Algorithm 2) 576 / 593 / 670; 4096^2 1190 / 1258 / 1470.
+// rows.  (The tiles are counted over the whole batch; batches of two or more run
+// as two groups with about half of them each.)  A step, 8 / 4 / 2 rows: 64^2 FP64
+// 114 / 96 / 88 us; 256^2 FP64 L = 4 387 / 308 / 284; 256^2 FP32 83 / 81 / 82;
+// 226^2 FP32 100 / 96 / 95; 512^2 FP32 68 / 68 / 69; 1024^2 FP32 (Algorithm 2)
+// 576 / 593 / 670; 4096^2 1190 / 1258 / 1470.
 //
 // BF16 z rounds every coefficient to 8 bits, so the last bit of any sum before
 // it decides a rounding now and then, and one rounding of a low-pass coefficient
@@ -676,10 +678,10 @@ void destroy_batch(mlba_batch* B) {
 // (the residual norm's partial sums), the row pass of a rank-one PSF first, the
 // masks tap by tap (k_frame.cu), full column CTAs and 32 values per thread in
 // the alpha_n sums, and the inner products of Algorithm 2 over vectors.
-// A pass in that order, against the shape-dependent one: 1024^2 Algorithm 1
-// (2 iterations) 249 / 247 us, 256^2 4-NS rank one (8) 854 / 661, 1024^2
-// Algorithm 2 (3) 1604 / 1550, 4096^2 4-NS rank one L = 2 (4) 5113 / 4229, L = 4
-// 6798 / 5898, the 64-problem batch (8) 8064 / 7740.
+// A pass in that order / in the shape-dependent one: 1024^2 Algorithm 1 (2
+// iterations) 252 / 245 us, 256^2 4-NS rank one (8) 810 / 661, 1024^2 Algorithm 2
+// (3) 1577 / 1548, 4096^2 4-NS rank one L = 2 (4) 4506 / 4223, L = 4 6194 / 5891,
+// the 64-problem batch (8) 7959 / 7726.
 int stencil_variant(const mlba_batch* B) {
   if (B->z_store == MLBA_BF16) return 8 | ST_ROW_FIRST;
   const double resident = B->dtype == MLBA_F64 ? 152.0 : 304.0;
@@ -1090,7 +1092,8 @@ int time_frame_shape(mlba_batch* B, int shape, int seg, float* us) {
 // recomputed halo rows (L = 2: 2.25 swept rows per owned row at 32, 2.5 at 16,
 // 3 at 8, 4 at 4).  Halve while the doubled number of warps is resident at
 // once: about 20 FP32 warps per SM; in FP64 one warp per scheduler, because the
-// FP64 pipe is already full with one.  Measured per launch, 32 rows against
+// FP64 pipe is already full with one.  (Counted over the whole batch, whose two
+// groups launch about half each.)  Measured per launch, 32 rows against
 // the choice: 256^2 FP32 32 -> 10 us (4 rows), 72^2 FP64 L = 1 150 -> 21 us (4);
 // 1044^2 BF16 z 45 -> 39 us (16; 8: 44, 4: 54; 31 with the row routine); the 64-problem batch stays at
 // 32 (16: +0.5 %, 8: +10 %).  L >= 3 starts at 16 in FP32 (a step at 4096^2:
