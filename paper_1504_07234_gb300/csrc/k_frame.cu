@@ -147,7 +147,7 @@ constexpr int F3_SEG_NWR = 2;   // warps per CTA of the sweeps with shorter segm
 // the same order (a warp's sweep does not depend on its CTA), so the choice
 // changes the time only.  Shape 0 is the default; FP64 always uses it.  Its
 // queue of one row (the L2 prefetch hides the rest) lets the sweep keep its
-// rings in place (f3_level): a launch of 4096^2, L = 2 went from 419 to 406 us
+// rings in place (f3_level): a launch of 4096^2, L = 2 went from 419 to 411 us
 // together with the sum / difference form of the masks (f3_row).
 // Shapes with ring > 0 stream each warp's z rows through a ring of `ring`
 // row slots in shared memory, filled by bulk asynchronous copies (one 1 KB
@@ -232,7 +232,8 @@ __device__ __forceinline__ double f3_flip(double v, int m) {
 // and the transpose the same way: 15 operations per horizontal mask instead
 // of 19 (FP32: an issue-bound sweep; FP64: the pipe is full).  A correction is
 // complete before z is added, so z is rounded once per update at its own
-// magnitude.
+// magnitude (z inside the chain of multiply-adds: 14 operations, 406 us for a
+// launch of 4096^2, L = 2 instead of 411, two roundings).
 // BF16 z: the masks tap by tap, in one fixed order (the rounding of z to 8 bits
 // makes the last bit of these sums matter, see the host's stencil_variant).
 // PARTS: a row's three shares are summed by themselves and then added to its
